@@ -198,19 +198,28 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   const int n_small = std::min(nM, nN), n_big = std::max(nM, nN);
   // Long-K tall-skinny steps expand the small operand into scratch A (after
   // the small operand itself when that one is permuted into scratch A)
-  const size_t tr_used = (nM <= nN && perm_a) ? ((8 * (size_t(1) << a_req.size()) + 4095) & ~size_t(4095)) : 0;
+  const size_t tr_used = perm_a ? ((8 * (size_t(1) << a_req.size()) + 4095) & ~size_t(4095)) : 0;
   char* tr_scratch = scratch_a + tr_used;
   const size_t tr_avail = scratch_a_bytes > tr_used ? scratch_a_bytes - tr_used : 0;
   const bool tc_rows_ok = choice != 0 && choice != 1 && ctx->precision != TNQ_PREC_FP32 && n_small <= 7 &&
                           !use_dot(nM, nN, nK) &&
                           tc_rows_supported(1 << n_small, 1 << n_big, 1 << nK, 1 << nH, n_big + nH, ctx->precision) &&
                           tc_rows_scratch_bytes(1 << n_small, 1 << nK, 1 << nH, ctx->precision) <= tr_avail;
-  if (tc_rows_ok || (!use_tc && (rows_capable(nM, nN) || use_dot(nM, nN, nK)) && part)) {
-    // bandwidth-bound skinny step: complex64 operands in [h][m|n][k] order
-    // The large operand of a short-K rows step is read in place (fused gather)
-    // instead of being permuted first.
-    const bool small_is_a = nM <= nN;
-    const bool gather = tc_rows_ok || (!use_dot(nM, nN, nK) && nK <= 5 && (small_is_a ? perm_b : perm_a));
+  // A batch whose expanded small operands do not fit one CTA leaves the tensor
+  // cores unless a row's arithmetic would bound the CUDA cores: each batch
+  // entry would fill its own S' and few tiles.  The plain TF32 mode keeps its
+  // operand rounding.
+  const bool batched = tc_rows_ok && choice == -1 && gather_bound(nM, nN, nK) &&
+                       !tc_rows_shared_ok(1 << n_small, 1 << nK, 1 << nH, ctx->precision);
+  const bool tc_rows = tc_rows_ok && !batched;
+  const bool round_tf32 = batched && ctx->precision == TNQ_PREC_TF32;
+  // The A side is never the larger one (both hold the H and K labels), so M is
+  // the small side of a skinny step.
+  const bool gather = tc_rows || batched || (!use_tc && !use_dot(nM, nN, nK) && gather_bound(nM, nN, nK));
+  if (gather || (!use_tc && (rows_capable(nM, nN) || use_dot(nM, nN, nK)) && part)) {
+    // bandwidth-bound skinny step: complex64 operands in [h][m|n][k] order; the
+    // large operand of a short-K step is read in its stored layout (fused
+    // gather) instead of being permuted first.
     // Dot steps read an operand in place when its stored layout starts with at
     // least 2^5 K values in the required K order (one contiguous run) and keeps
     // every K bit above the run in K order too (the kernel steps its K offset
@@ -244,48 +253,43 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
     DotOp dot_a, dot_b;
     const bool inpl_a = perm_a && inplace_dot(a_src, a_labels, a_req, &dot_a);
     const bool inpl_b = perm_b && inplace_dot(b_src, b_labels, b_req, &dot_b);
-    if (perm_a && !inpl_a && !(gather && !small_is_a)) {
+    if (perm_a && !inpl_a) {
       build_perm_desc(a_labels.data(), (int)a_labels.size(), a_req.data(), (int)a_req.size(), slice_labels.data(),
                       ns, PM_C64, nK, &d);
       TNQ_CUDA(perm(ctx, d, a_src, scratch_a, nullptr, slice_id, 16.0 * std::ldexp(1.0, (int)a_req.size())));
     }
-    if (perm_b && !inpl_b && !(gather && small_is_a)) {
+    if (perm_b && !inpl_b && !gather) {
       build_perm_desc(b_labels.data(), (int)b_labels.size(), b_req.data(), (int)b_req.size(), slice_labels.data(),
                       ns, PM_C64, nK, &d);
       TNQ_CUDA(perm(ctx, d, b_src, scratch_b, nullptr, slice_id, 16.0 * std::ldexp(1.0, (int)b_req.size())));
     }
     if (gather) {
       // large operand: required order [K][rows][H]; find each bit in its stored labels
-      const std::vector<int>& src_l = small_is_a ? b_labels : a_labels;
-      const std::vector<int>& req = small_is_a ? b_req : a_req;
-      auto spos = [&](int l) { return int(std::find(src_l.begin(), src_l.end(), l) - src_l.begin()); };
+      auto spos = [&](int l) { return int(std::find(b_labels.begin(), b_labels.end(), l) - b_labels.begin()); };
       GatherDesc gd;
       gd.nk = nK;
-      for (int j = 0; j < nK; ++j) gd.kpos[j] = spos(req[j]);
-      gd.nrow = (int)req.size() - nK;
-      for (int j = 0; j < gd.nrow; ++j) gd.rowpos[j] = spos(req[nK + j]);
+      for (int j = 0; j < nK; ++j) gd.kpos[j] = spos(b_req[j]);
+      gd.nrow = (int)b_req.size() - nK;
+      for (int j = 0; j < gd.nrow; ++j) gd.rowpos[j] = spos(b_req[nK + j]);
       gd.n_slice = ns;
       for (int j = 0; j < 32; ++j) gd.slice_src[j] = j < ns ? spos(slice_labels[j]) : -1;
       for (int j = 0; j < ns; ++j)
-        if (gd.slice_src[j] >= (int)src_l.size()) gd.slice_src[j] = -1;
+        if (gd.slice_src[j] >= (int)b_labels.size()) gd.slice_src[j] = -1;
       const int M = 1 << nM, N = 1 << nN, K = 1 << nK, H = 1 << nH;
-      const void* Ssm = small_is_a ? (perm_a ? (const void*)scratch_a : a_src) : (perm_b ? (const void*)scratch_b : b_src);
-      const void* Gs = small_is_a ? b_src : a_src;
+      const void* Ssm = perm_a ? (const void*)scratch_a : a_src;
       KernelRecord r{4, ctx->cur_step, nH, nM, nN, nK, 8.0 * work,
                      8.0 * (std::ldexp(1.0, nH + nM + nK) + std::ldexp(1.0, nH + nN + nK) +
                             (acc ? 2.0 : 1.0) * std::ldexp(1.0, nH + nM + nN)),
                      0.f};
-      if (tc_rows_ok) r.kind = 5;
+      if (tc_rows) r.kind = 5;
       int slot = timing_begin(ctx);
       cudaError_t e;
-      if (tc_rows_ok)
-        e = small_is_a ? launch_cgemm_tc_rows(Ssm, Gs, gd, C, acc, M, N, K, H, N, 1, slice_id, ctx->precision, err,
-                                              ctx->sm_count, ctx->stream, tr_scratch, tr_avail)
-                       : launch_cgemm_tc_rows(Ssm, Gs, gd, C, acc, N, M, K, H, 1, N, slice_id, ctx->precision, err,
-                                              ctx->sm_count, ctx->stream, tr_scratch, tr_avail);
+      if (tc_rows)
+        e = launch_cgemm_tc_rows(Ssm, b_src, gd, C, acc, M, N, K, H, slice_id, ctx->precision, err, ctx->sm_count,
+                                 ctx->stream, tr_scratch, tr_avail);
       else
-        e = small_is_a ? launch_cgemm_rows_gather(Ssm, Gs, gd, C, acc, M, N, K, H, N, 1, slice_id, ctx->stream)
-                       : launch_cgemm_rows_gather(Ssm, Gs, gd, C, acc, N, M, K, H, 1, N, slice_id, ctx->stream);
+        e = launch_cgemm_rows_gather(Ssm, b_src, gd, C, acc, M, N, K, H, slice_id, round_tf32, ctx->sm_count,
+                                     ctx->stream);
       timing_end(ctx, slot, r);
       TNQ_CUDA(e);
       ctx->launches++;
@@ -309,10 +313,7 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
       if (e == cudaSuccess) e = launch_reduce_splits(part, splits, out_elems, C, acc, ctx->sm_count, ctx->stream);
     } else {
       splits = rows_splits(nH, nM, nN, nK);
-      if (nM <= nN)
-        e = launch_cgemm_rows(A, B, C, acc, part, splits, M, N, K, H, N, 1, ctx->stream);
-      else
-        e = launch_cgemm_rows(B, A, C, acc, part, splits, N, M, K, H, 1, N, ctx->stream);
+      e = launch_cgemm_rows(A, B, C, acc, part, splits, M, N, K, H, ctx->stream);
       if (e == cudaSuccess && splits > 1)
         e = launch_reduce_splits(part, splits, out_elems, C, acc, ctx->sm_count, ctx->stream);
     }

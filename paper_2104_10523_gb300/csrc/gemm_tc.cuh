@@ -34,8 +34,7 @@ cudaError_t launch_cgemm_tc(const TcGemmArgs& g, int sm_count, cudaStream_t st);
 
 struct GatherDesc;
 
-// Tall-skinny tensor-core GEMM (gemm_tc_rows.cu): out[h][s][g] (strides
-// s_stride_out, g_stride_out; batch stride ns * ng) = sum_k S[h][s][k] G[h][g][k]
+// Tall-skinny tensor-core GEMM (gemm_tc_rows.cu): out[h][s][g] = sum_k S[h][s][k] G[h][g][k]
 // for a small operand S ([batch][ns][K] complex64, ns <= 128, K <= 256) and a
 // large one G read in
 // its stored bit order through gd, split into BF16 or TF32 hi/lo parts in
@@ -47,8 +46,10 @@ bool tc_rows_supported(int ns, int ng, int K, int batch, int nrow, int precision
 size_t tc_rows_scratch_bytes(int ns, int K, int batch, int precision);
 cudaError_t tc_rows_prepare();
 cudaError_t launch_cgemm_tc_rows(const void* Ssmall, const void* Gsrc, const GatherDesc& gd, void* C, void* acc, int ns,
-                                 int ng, int K, int batch, long long s_stride_out, long long g_stride_out, int slice_id,
-                                 int precision, int* err, int sm_count, cudaStream_t st, void* scratch = nullptr,
-                                 size_t scratch_bytes = 0);
+                                 int ng, int K, int batch, int slice_id, int precision, int* err, int sm_count,
+                                 cudaStream_t st, void* scratch = nullptr, size_t scratch_bytes = 0);
+// Whether one CTA holds the expanded small operands of every batch entry (else
+// each CTA serves one entry).
+bool tc_rows_shared_ok(int ns, int K, int batch, int precision);
 
 }  // namespace tnq

@@ -24,7 +24,8 @@
 // for Npad = 256), ceil(2K / k_step) in plain TF32; four TMEM accumulator
 // buffers for Npad <= 64, two above, at most all 512 columns.  When the
 // expanded small operand of every batch entry does not fit in shared memory,
-// each batch entry gets its own launch.
+// a CTA serves one batch entry (its own S'), all entries in one launch: a
+// launch per entry cost 8 us each (TF32, 2^11 entries of 32 x 128 x 8: 20 ms).
 //
 // A tile's K range may be cut into one-atom K-parts: a shared-memory stage
 // then holds one part of a tile (the MMAs of a tile accumulate over its
@@ -91,6 +92,7 @@ constexpr int TR_BPRIME_BUDGET = 128 * 1024;
 constexpr int TR_SMEM_LIMIT = 225 * 1024;      // dynamic shared memory of one CTA
 constexpr int TR_SMEM_HALF = 110 * 1024;       // the same, two CTAs per SM
 constexpr int TR_KMAX = 256;                  // longest K (in resident mode: 64)
+constexpr int TR_ENTRY_Y_LOG2 = 15;           // per-entry grids: batch bits on the grid's y (the rest on z)
 constexpr int TR_ROWTAB_DIGITS = 7;           // 4-bit digits of a tile index (nrow <= 35)
 
 struct TrParams {
@@ -118,8 +120,9 @@ struct TrParams {
   int split;              // 1: three products (hi/lo); 0: one TF32 product
   int pairs;              // the lowest stored bit of G is K bit 0: 16-byte loads
   int row_tab;            // 1: every stored position of the row bits above 7 is below 32 (digit table)
-  long long s_stride, g_stride;
   int tiles_per_h;        // ng / 128
+  int hbits;              // per-entry grids: batch bits taken from the grid's y and z (batch and gd.nrow exclude them)
+  int hpos[24];           // their stored positions in G
   long long total_tiles;
   int slice_id;
   uint32_t idesc;         // MMA of N = npad
@@ -205,7 +208,7 @@ __device__ __forceinline__ void store_chunk(uint8_t* hi, uint8_t* lo, int r, con
 
 // Expanded small operand S' for every batch entry: rows n < npad of the reals
 // the MMAs read, hi and lo, built by the converter threads at kernel start.
-__device__ void build_bprime(const TrParams& P, uint8_t* bp, int tid, int nthreads) {
+__device__ void build_bprime(const TrParams& P, const float2* S, uint8_t* bp, int tid, int nthreads) {
   const int es = P.kind_bf16 ? 2 : 4;
   const int reals = P.nks * (32 / es);
   const int per_h = P.npad * reals;
@@ -217,7 +220,7 @@ __device__ void build_bprime(const TrParams& P, uint8_t* bp, int tid, int nthrea
     const int s = n >> 1, k = q >> 1;
     float x = 0.f;
     if (s < P.ns && k < P.K) {
-      const float2 a = P.S[(size_t(h) * P.ns + s) * P.K + k];
+      const float2 a = S[(size_t(h) * P.ns + s) * P.K + k];
       // row (s, re): [sr, -si] per k; row (s, im): [si, sr]
       x = (n & 1) ? ((q & 1) ? a.x : a.y) : ((q & 1) ? -a.y : a.x);
     }
@@ -239,7 +242,7 @@ __device__ void build_bprime(const TrParams& P, uint8_t* bp, int tid, int nthrea
 // S' of every batch entry expanded into global memory (streamed mode), in the
 // layout build_bprime gives it in shared memory.
 __global__ void build_bprime_kernel(const __grid_constant__ TrParams P, uint8_t* dst) {
-  build_bprime(P, dst, int(blockIdx.x * blockDim.x + threadIdx.x), int(gridDim.x * blockDim.x));
+  build_bprime(P, P.S, dst, int(blockIdx.x * blockDim.x + threadIdx.x), int(gridDim.x * blockDim.x));
 }
 
 // Tile t = h * tph + gt (batch entry h, tile gt within it), stepped by the
@@ -301,6 +304,9 @@ __device__ __forceinline__ void load_chunk(const TrParams& P, const uint32_t* ko
 template <int CH, int DEPTH, int MODE, int MINB>
 __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const __grid_constant__ TrParams P) {
   extern __shared__ uint8_t smem_raw[];
+  // batch entry of a per-entry grid (0 otherwise), read where it is needed: the
+  // two-per-SM kernels have no register to keep it in
+  auto entry = [] { return blockIdx.y + (blockIdx.z << TR_ENTRY_Y_LOG2); };
   constexpr int kBF16 = MODE == 2 ? 1 : 0, kSplit = MODE != 0 ? 1 : 0;
   __shared__ __align__(8) uint64_t full_bar[TR_MAX_STAGES];
   __shared__ __align__(8) uint64_t empty_bar[TR_MAX_STAGES];
@@ -352,7 +358,7 @@ __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const _
         if ((v >> b) & 1) o |= 1u << P.gd.rowpos[7 + 4 * n + b];
       rowtab[n][v] = o;
     }
-  if (warp < TR_CONV_WARPS && !P.stream_bp) build_bprime(P, bprime, threadIdx.x, 32 * TR_CONV_WARPS);
+  if (warp < TR_CONV_WARPS && !P.stream_bp) build_bprime(P, P.S + size_t(entry()) * P.ns * P.K, bprime, threadIdx.x, 32 * TR_CONV_WARPS);
   if (warp == TR_MMA_WARP) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                  "r"(tmem_cols)
@@ -381,7 +387,7 @@ __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const _
     size_t soff = 0;
     for (int j = 0; j < P.gd.n_slice; ++j)
       if (P.gd.slice_src[j] >= 0 && ((P.slice_id >> j) & 1)) soff |= size_t(1) << P.gd.slice_src[j];
-    const size_t lo = soff | deposit(r, P.gd.rowpos, 7);
+    const size_t lo = soff | deposit(entry(), P.hpos, P.hbits) | deposit(r, P.gd.rowpos, 7);
     // row r of tile t is row 128 t + r of the (batch-major) row index, whose
     // bits above the lowest 7 are t itself
     auto row_base = [&](uint32_t t) {
@@ -550,7 +556,7 @@ __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const _
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t h = hg.h;
       const uint32_t g = hg.gt * 128u + uint32_t(row);
-      const size_t obase = size_t(h) * P.ns * P.ng + size_t(g) * P.g_stride;
+      const size_t obase = (size_t(entry()) + h) * P.ns * P.ng + g;
       const uint32_t base = tmem + lane_addr + uint32_t(b * P.acc_cols);
       // 32 columns (16 outputs) at a time
       // EC columns (EC / 2 outputs) at a time; the TMEM loads of the next EC
@@ -593,7 +599,7 @@ __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const _
           const int s = c0 / 2 + j;
           if (s < P.ns) {
             const float re = o[2 * j], im = o[2 * j + 1];
-            const size_t o_at = obase + size_t(s) * P.s_stride;
+            const size_t o_at = obase + size_t(s) * P.ng;
             if (P.acc) {
               double2 a = P.acc[o_at];
               a.x += double(re);
@@ -729,10 +735,12 @@ bool tc_rows_supported(int ns, int ng, int K, int batch, int nrow, int precision
 
 namespace {
 
+// entry_bits > 0: a per-entry grid over 2^entry_bits batch entries, whose
+// stored positions in G are entry_pos; batch and gd.nrow then exclude them.
 cudaError_t launch_tc_rows_one(const void* Ssmall, const void* Gsrc, const GatherDesc& gd, void* C, void* acc, int ns,
-                               int ng, int K, int batch, long long s_stride_out, long long g_stride_out, int slice_id,
-                               int precision, int* err, int sm_count, cudaStream_t st, void* scratch = nullptr,
-                               size_t scratch_bytes = 0) {
+                               int ng, int K, int batch, int slice_id, int precision, int* err, int sm_count,
+                               cudaStream_t st, void* scratch = nullptr, size_t scratch_bytes = 0, int entry_bits = 0,
+                               const int* entry_pos = nullptr) {
   TrParams P;
   P.S = reinterpret_cast<const float2*>(Ssmall);
   P.G = reinterpret_cast<const float2*>(Gsrc);
@@ -793,8 +801,6 @@ cudaError_t launch_tc_rows_one(const void* Ssmall, const void* Gsrc, const Gathe
   P.row_tab = gd.nrow - 7 <= 4 * TR_ROWTAB_DIGITS ? 1 : 0;
   for (int j = 7; j < gd.nrow; ++j)
     if (gd.rowpos[j] >= 32) P.row_tab = 0;
-  P.s_stride = s_stride_out;
-  P.g_stride = g_stride_out;
   P.tiles_per_h = ng / 128;
   P.total_tiles = (long long)P.tiles_per_h * batch;
   // 32-bit tile counters: cursors run up to 2 items (4 grid strides) past the end
@@ -807,7 +813,13 @@ cudaError_t launch_tc_rows_one(const void* Ssmall, const void* Gsrc, const Gathe
   P.C = reinterpret_cast<float2*>(C);
   P.acc = reinterpret_cast<double2*>(acc);
   P.err = err;
-  const long long grid = std::min<long long>(P.total_tiles, (two ? 2 : 1) * std::max(1, sm_count));
+  const long long slots = (two ? 2 : 1) * std::max(1, sm_count);
+  P.hbits = entry_bits;
+  for (int j = 0; j < entry_bits; ++j) P.hpos[j] = entry_pos[j];
+  // a per-entry grid gives every entry its share of the resident CTAs (at least one)
+  const int ybits = std::min(entry_bits, TR_ENTRY_Y_LOG2);
+  const dim3 grid{unsigned(std::min<long long>(P.total_tiles, std::max<long long>(1, slots >> entry_bits))),
+                  1u << ybits, 1u << (entry_bits - ybits)};
   const size_t smem = size_t(P.stages) * (2 * P.patoms * TR_ATOM_BYTES + (P.stream_bp ? 2 * size_t(P.bp_part) : 0)) +
                       (P.stream_bp ? 0 : bp_all) + 1024;
   if (P.stream_bp) {
@@ -818,49 +830,39 @@ cudaError_t launch_tc_rows_one(const void* Ssmall, const void* Gsrc, const Gathe
   }
   const int mode = P.kind_bf16 ? 2 : (P.split ? 1 : 0);
   const TrKernel k = two ? kTrKernels2[mode] : kTrKernels[ch == 16 ? 1 : 0][mode];
-  k<<<unsigned(grid), TR_THREADS, smem, st>>>(P);
+  k<<<grid, TR_THREADS, smem, st>>>(P);
   return cudaGetLastError();
 }
 
 }  // namespace
 
+bool tc_rows_shared_ok(int ns, int K, int batch, int precision) {
+  if (K > TR_RESIDENT_KMAX) return true;
+  const bool bf16 = precision == TNQ_PREC_BF16X3;
+  const size_t bp_all = tr_bprime_bytes(ns, K, batch, bf16);
+  return bp_all <= size_t(TR_BPRIME_BUDGET) && tr_stages(tr_atoms(K, bf16), bp_all).stages >= 2;
+}
+
 cudaError_t launch_cgemm_tc_rows(const void* Ssmall, const void* Gsrc, const GatherDesc& gd, void* C, void* acc, int ns,
-                                 int ng, int K, int batch, long long s_stride_out, long long g_stride_out, int slice_id,
-                                 int precision, int* err, int sm_count, cudaStream_t st, void* scratch,
-                                 size_t scratch_bytes) {
+                                 int ng, int K, int batch, int slice_id, int precision, int* err, int sm_count,
+                                 cudaStream_t st, void* scratch, size_t scratch_bytes) {
   if (!tc_rows_supported(ns, ng, K, batch, gd.nrow, precision) || !err) return cudaErrorNotSupported;
   if (gd.nk > 8 || gd.nrow > 32 || (1 << gd.nk) != K) return cudaErrorInvalidValue;
   cudaError_t pe = tc_rows_prepare();
   if (pe != cudaSuccess) return pe;
-  const bool bf16 = precision == TNQ_PREC_BF16X3;
-  if (K > TR_RESIDENT_KMAX)
-    return launch_tc_rows_one(Ssmall, Gsrc, gd, C, acc, ns, ng, K, batch, s_stride_out, g_stride_out, slice_id,
-                              precision, err, sm_count, st, scratch, scratch_bytes);
-  const size_t bp_all = tr_bprime_bytes(ns, K, batch, bf16);
-  if (bp_all <= size_t(TR_BPRIME_BUDGET) && tr_stages(tr_atoms(K, bf16), bp_all).stages >= 2)
-    return launch_tc_rows_one(Ssmall, Gsrc, gd, C, acc, ns, ng, K, batch, s_stride_out, g_stride_out, slice_id,
-                              precision, err, sm_count, st);
-  // S' of every batch entry does not fit: one launch per entry, whose batch
-  // bits (the row bits above the ng bits) become extra slice bits of G
+  if (tc_rows_shared_ok(ns, K, batch, precision))
+    return launch_tc_rows_one(Ssmall, Gsrc, gd, C, acc, ns, ng, K, batch, slice_id, precision, err, sm_count, st,
+                              scratch, scratch_bytes);
+  // S' of every batch entry does not fit one CTA: a per-entry grid, whose batch
+  // bits (the row bits above the ng bits) come from the CTA index
   int gbits = 0;
   while ((1 << gbits) < ng) ++gbits;
   const int hbits = gd.nrow - gbits;
-  if (hbits < 0 || (1 << hbits) != batch || gd.n_slice + hbits > 30) return cudaErrorNotSupported;
+  if (hbits < 0 || (1 << hbits) != batch || hbits > 24) return cudaErrorNotSupported;
   GatherDesc g1 = gd;
   g1.nrow = gbits;
-  for (int j = 0; j < hbits; ++j) g1.slice_src[gd.n_slice + j] = gd.rowpos[gbits + j];
-  g1.n_slice = gd.n_slice + hbits;
-  const float2* S = reinterpret_cast<const float2*>(Ssmall);
-  for (int h = 0; h < batch; ++h) {
-    const size_t ob = size_t(h) * ns * ng;
-    cudaError_t e = launch_tc_rows_one(S + size_t(h) * ns * K, Gsrc, g1,
-                                       C ? static_cast<void*>(reinterpret_cast<float2*>(C) + ob) : nullptr,
-                                       acc ? static_cast<void*>(reinterpret_cast<double2*>(acc) + ob) : nullptr, ns,
-                                       ng, K, 1, s_stride_out, g_stride_out, slice_id | (h << gd.n_slice), precision,
-                                       err, sm_count, st);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  return launch_tc_rows_one(Ssmall, Gsrc, g1, C, acc, ns, ng, K, 1, slice_id, precision, err, sm_count, st, nullptr, 0,
+                            hbits, gd.rowpos + gbits);
 }
 
 }  // namespace tnq

@@ -50,11 +50,10 @@ cudaError_t launch_reduce_splits(const void* part, int splits, size_t n, void* C
                                  cudaStream_t st);
 
 // Skinny steps (see skinny.cu).  rows: C = S x G^T for a small operand S of
-// ns <= 32 rows; output element (h, s, g) at h*ns*ng + s*s_stride + g*g_stride.
+// ns <= 32 rows and ng rows of the large operand; output [batch][ns][ng].
 // dot: M, N <= 8; always writes FP32 partials [splits][batch][M][N].
 cudaError_t launch_cgemm_rows(const void* Ssmall, const void* Gbig, void* C, void* acc, void* part, int splits,
-                              int ns, int ng, int K, int batch, long long s_stride_out, long long g_stride_out,
-                              cudaStream_t st);
+                              int ns, int ng, int K, int batch, cudaStream_t st);
 cudaError_t launch_cdot(const void* A, const void* B, void* part, int splits, int M, int N, int K, int batch,
                         cudaStream_t st);
 // Operand of the dot kernel addressed through bit deposits: element (row r of
@@ -82,10 +81,12 @@ struct GatherDesc {
   int n_slice;
   int slice_src[32];
 };
-// rows kernel with K <= 32 reading the large operand in place (fused permute).
+// rows kernel with K <= 32 and ns <= 128 reading the large operand in place
+// (fused permute); output [batch][ns][ng].  round_tf32: both operands are
+// rounded to TF32 first.
 cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const void* Gsrc, const GatherDesc& gd, void* C, void* acc,
-                                     int ns, int ng, int K, int batch, long long s_stride_out, long long g_stride_out,
-                                     int slice_id, cudaStream_t st);
+                                     int ns, int ng, int K, int batch, int slice_id, bool round_tf32, int sm_count,
+                                     cudaStream_t st);
 
 // Projection leaves j < n_proj at leaves_base + j * stride_bytes:
 // P_j[(b << 1) | x] = [bits[b * row_len + tab[j]] == x] for b < n_valid, else 0.

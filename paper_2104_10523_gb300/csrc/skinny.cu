@@ -8,10 +8,9 @@
 //   rows kernel:  C[h][s][g] = sum_k S[h][s][k] G[h][g][k] for a small side of
 //                 at most 32 rows: each thread owns one row g of the large
 //                 operand, the small operand and a K slice of G are staged in
-//                 shared memory by coalesced loads; output strides make the
-//                 same kernel serve both "small M" and "small N".
-//   rows kernel, short K (<= 32): each thread loads its row of the large operand
-//                 into registers with 16-byte loads (no staging);
+//                 shared memory by coalesced loads;
+//   gather kernel: short K (<= 32), each thread loads its rows of the large
+//                 operand, in their stored bit layout, into registers;
 //   dot kernel:   M, N <= 8 and long K: every thread walks its own part of K
 //                 with 16-byte loads and keeps the M x N sums in registers; the
 //                 CTA reduces them and writes one partial per CTA.
@@ -26,11 +25,11 @@ namespace {
 constexpr int RW_THREADS = 128;  // rows of the large operand per CTA
 constexpr int RW_KC = 32;        // K elements staged per iteration
 constexpr int RW_SMAX = 32;
+constexpr int GATHER_SMAX = 128;  // small-operand rows of the gather kernel
 
 __global__ void __launch_bounds__(RW_THREADS) cgemm_rows_kernel(
     const float2* __restrict__ S, const float2* __restrict__ G, float2* __restrict__ C, double2* __restrict__ acc,
-    float2* __restrict__ part, int ns, int ng, int K, int batch, long long s_stride_out, long long g_stride_out,
-    int kchunk, int tiles_g) {
+    float2* __restrict__ part, int ns, int ng, int K, int batch, int kchunk, int tiles_g) {
   __shared__ float2 Gs[RW_THREADS][RW_KC + 1];
   __shared__ float2 Ss[RW_SMAX][RW_KC + 1];
   const int t = threadIdx.x;
@@ -81,7 +80,7 @@ __global__ void __launch_bounds__(RW_THREADS) cgemm_rows_kernel(
 #pragma unroll
   for (int s = 0; s < RW_SMAX; ++s) {
     if (s < ns) {
-      const size_t o = hbase + size_t(s) * s_stride_out + size_t(g) * g_stride_out;
+      const size_t o = hbase + size_t(s) * ng + g;
       if (part) {
         part[size_t(split) * batch * ns * ng + o] = make_float2(ar[s], ai[s]);
       } else if (acc) {
@@ -217,179 +216,123 @@ __global__ void __launch_bounds__(DOT_THREADS, 2) cdot_blk_kernel(const __grid_c
   }
 }
 
-// Small operand of ns <= 32 rows and K <= 32: each thread owns one row of the
-// large operand and reads it with 16-byte loads straight into registers.
-template <int KMAX, int ROWS>
-__global__ void __launch_bounds__(256) cgemm_rows_regk_kernel(const float2* __restrict__ S, const float2* __restrict__ G,
-                                                              float2* __restrict__ C, double2* __restrict__ acc, int ns,
-                                                              int ng, int K, int batch, long long s_stride,
-                                                              long long g_stride, int tiles_g) {
-  // ROWS rows of the large operand per thread (256 * ROWS per CTA): each small-
-  // operand value read from shared memory serves ROWS multiply-adds
-  __shared__ float2 Ss[RW_SMAX][KMAX];
-  const int tile = int(blockIdx.x % tiles_g);
-  const int h = int(blockIdx.x / tiles_g);
-  const float2* Sh = S + size_t(h) * ns * K;
-  for (int i = threadIdx.x; i < RW_SMAX * KMAX; i += blockDim.x) {
-    const int r = i / KMAX, kk = i % KMAX;
-    Ss[r][kk] = (r < ns && kk < K) ? Sh[size_t(r) * K + kk] : make_float2(0.f, 0.f);
+// Nearest TF32 value, ties away from zero (finite inputs).
+__device__ __forceinline__ float2 tf32_rna2(float2 v) {
+  return make_float2(__uint_as_float((__float_as_uint(v.x) + 0x1000u) & 0xffffe000u),
+                     __uint_as_float((__float_as_uint(v.y) + 0x1000u) & 0xffffe000u));
+}
+
+// Short-K rows kernel reading the large operand in its stored bit layout (no
+// separate permute): row R of the (g bits, then batch bits) row index starts at
+// the source offset sum_j bit_j(R) << rowpos[j], and element k of a row is
+// dep(k, kpos) further on.  One thread owns ROWS rows, held in registers; a CTA
+// owns cta_rows consecutive rows of the batch-major row index, so with short
+// rows (ng < cta_rows) it serves several batch entries, whose S rows it stages
+// together (one 16-byte pad per entry spreads the entries over the banks);
+// with ROWS = 2 a CTA stays within one entry.
+// ROUND rounds both operands to TF32 first (the products are then exact in
+// FP32: the arithmetic of the plain TF32 mode on the CUDA cores).
+//
+// Bound: HBM while 4 FFMA per (s, k) of a row stay below the 8 (K + ns) bytes
+// it moves.  One launch for every batch entry: 4096 entries of 4 x 2^12 x 8
+// took 33.5 ms as one tensor-core launch each (8 us a launch).
+template <int K, int ROWS, bool ROUND>
+__global__ void __launch_bounds__(256) cgemm_rows_gather_kernel(const float2* __restrict__ S,
+                                                                const float2* __restrict__ G,
+                                                                const __grid_constant__ GatherDesc gd,
+                                                                float2* __restrict__ C, double2* __restrict__ acc,
+                                                                int ns, int log_per, int log_ng, int cta_rows,
+                                                                int entries, int slice_id) {
+  extern __shared__ __align__(16) float2 Ss[];  // [entries][ns * K + 2]
+  __shared__ unsigned long long blk_base;
+  const int t = threadIdx.x;
+  const long long R0 = (long long)blockIdx.x * cta_rows;
+  const int h0 = int(R0 >> log_ng);
+  const int per = ns * K, pitch = per + 2;
+  for (int i = t; i < entries * per; i += 256) {
+    const float2 v = S[size_t(h0) * per + i];
+    Ss[i + 2 * (i >> log_per)] = ROUND ? tf32_rna2(v) : v;
   }
+  if (t == 0) {
+    unsigned long long o = 0;
+    for (int j = 0; j < gd.n_slice; ++j)
+      if (gd.slice_src[j] >= 0 && ((slice_id >> j) & 1)) o |= 1ull << gd.slice_src[j];
+    for (int j = 0; j < gd.nrow; ++j)
+      if ((R0 >> j) & 1) o |= 1ull << gd.rowpos[j];
+    blk_base = o;
+  }
+  size_t lo = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (j < gd.nrow && ((t >> j) & 1)) lo |= size_t(1) << gd.rowpos[j];
   __syncthreads();
-  int g[ROWS];
+  const bool pairs = K > 1 && gd.kpos[0] == 0;
   bool live[ROWS];
-  float2 gv[ROWS][KMAX];
+  float2 gv[ROWS][K];
 #pragma unroll
   for (int r = 0; r < ROWS; ++r) {
-    g[r] = tile * 256 * ROWS + r * 256 + threadIdx.x;
-    live[r] = g[r] < ng;
-    const float2* row = G + size_t(h) * ng * K + size_t(live[r] ? g[r] : 0) * K;
-    if ((K & 1) == 0) {
+    live[r] = r * 256 + t < cta_rows;
+    size_t base = size_t(blk_base) | lo;
+    if (r) base |= size_t(1) << gd.rowpos[8];  // ROWS <= 2: the row bit above the thread bits
 #pragma unroll
-      for (int kk = 0; kk < KMAX; kk += 2)
-        if (kk < K) {
-          const float4 v = live[r] ? *reinterpret_cast<const float4*>(row + kk) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int kk = 0; kk < K; ++kk) gv[r][kk] = make_float2(0.f, 0.f);
+    if (live[r]) {
+      const float2* p = G + base;
+      if (pairs) {
+        // the lowest K bit is the stored layout's stride-1 bit: pairs (k, k+1) are
+        // adjacent and 16-byte aligned (every other offset bit is >= 1)
+#pragma unroll
+        for (int kk = 0; kk + 1 < K; kk += 2) {
+          uint32_t ko = 0;
+#pragma unroll
+          for (int j = 1; (1 << j) < K; ++j)
+            if ((kk >> j) & 1) ko |= 1u << gd.kpos[j];
+          const float4 v = __ldg(reinterpret_cast<const float4*>(p + ko));
           gv[r][kk] = make_float2(v.x, v.y);
           gv[r][kk + 1] = make_float2(v.z, v.w);
         }
-    } else {
+      } else {
 #pragma unroll
-      for (int kk = 0; kk < KMAX; ++kk)
-        if (kk < K) gv[r][kk] = live[r] ? row[kk] : make_float2(0.f, 0.f);
-    }
-  }
-  const size_t hbase = size_t(h) * ns * ng;
+        for (int kk = 0; kk < K; ++kk) {
+          uint32_t ko = 0;
 #pragma unroll
-  for (int s = 0; s < RW_SMAX; ++s) {
-    if (s >= ns) break;
-    float ar[ROWS], ai[ROWS];
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r) ar[r] = ai[r] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < KMAX; ++kk) {
-      if (kk < K) {
-        const float2 a = Ss[s][kk];
-#pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
-          const float2 bb = gv[r][kk];
-          ar[r] = fmaf(a.x, bb.x, ar[r]);
-          ar[r] = fmaf(-a.y, bb.y, ar[r]);
-          ai[r] = fmaf(a.x, bb.y, ai[r]);
-          ai[r] = fmaf(a.y, bb.x, ai[r]);
+          for (int j = 0; (1 << j) < K; ++j)
+            if ((kk >> j) & 1) ko |= 1u << gd.kpos[j];
+          gv[r][kk] = __ldg(p + ko);
         }
       }
     }
+    if (ROUND) {
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-      if (!live[r]) continue;
-      const size_t o = hbase + size_t(s) * s_stride + size_t(g[r]) * g_stride;
-      if (acc) {
-        double2 v = acc[o];
-        v.x += ar[r];
-        v.y += ai[r];
-        acc[o] = v;
-      } else {
-        C[o] = make_float2(ar[r], ai[r]);
-      }
+      for (int kk = 0; kk < K; ++kk) gv[r][kk] = tf32_rna2(gv[r][kk]);
     }
   }
-}
-
-// As cgemm_rows_regk_kernel, but the large operand is read in its stored bit
-// layout (no separate permute): row g (its N or M index, then batch bits) starts
-// at the source offset sum_j bit_j(g) << rowpos[j], and element k of a row is
-// koff[k] further on.  Leaves with sliced labels add the slice offset.  The row
-// offset is split into the thread's low 8 row bits (computed once) and the
-// CTA's row-block bits above them (one deposit per block, in shared memory);
-// EXACT instances have K == KMAX at compile time, and the small operand is read
-// in 16-byte pairs of k.
-template <int KMAX, int ROWS, bool EXACT>
-__global__ void __launch_bounds__(256) cgemm_rows_gather_kernel(const float2* __restrict__ S,
-                                                                const float2* __restrict__ G, const GatherDesc gd,
-                                                                float2* __restrict__ C, double2* __restrict__ acc,
-                                                                int ns, int ng, int K, int batch, long long s_stride,
-                                                                long long g_stride, int tiles_g, int slice_id) {
-  static_assert(KMAX % 2 == 0, "pairs of k");
-  __shared__ __align__(16) float2 Ss[RW_SMAX][KMAX];
-  __shared__ uint32_t koff[KMAX];
-  __shared__ unsigned long long hib[ROWS];
-  const int tile = int(blockIdx.x % tiles_g);
-  const int h = int(blockIdx.x / tiles_g);
-  const float2* Sh = S + size_t(h) * ns * K;
-  for (int i = threadIdx.x; i < RW_SMAX * KMAX; i += blockDim.x) {
-    const int r = i / KMAX, kk = i % KMAX;
-    Ss[r][kk] = (r < ns && kk < K) ? Sh[size_t(r) * K + kk] : make_float2(0.f, 0.f);
-  }
-  for (int kk = threadIdx.x; kk < KMAX; kk += blockDim.x) {
-    uint32_t o = 0;
-    for (int j = 0; j < gd.nk; ++j)
-      if ((kk >> j) & 1) o |= 1u << gd.kpos[j];
-    koff[kk] = o;
-  }
-  // rows of block r: (tile * ROWS + r) * 256 + threadIdx.x of batch entry h;
-  // with ng a multiple of 256 the global row index's low 8 bits are threadIdx.x
-  const bool split8 = gd.nrow >= 8 && (ng & 255) == 0;
-  if (split8 && threadIdx.x < ROWS) {
-    const long long hi = ((long long)h * ng + (long long)(tile * ROWS + int(threadIdx.x)) * 256) >> 8;
-    unsigned long long o = 0;
-    for (int j = 8; j < gd.nrow; ++j)
-      if ((hi >> (j - 8)) & 1) o |= 1ull << gd.rowpos[j];
-    hib[threadIdx.x] = o;
-  }
-  size_t soff = 0;
-  for (int j = 0; j < gd.n_slice; ++j)
-    if (gd.slice_src[j] >= 0 && ((slice_id >> j) & 1)) soff |= size_t(1) << gd.slice_src[j];
-  size_t lo8 = 0;
-  if (split8)
-    for (int j = 0; j < 8; ++j)
-      if ((threadIdx.x >> j) & 1) lo8 |= size_t(1) << gd.rowpos[j];
-  __syncthreads();
-  const bool pairs = gd.nk >= 1 && gd.kpos[0] == 0;
-  int g[ROWS];
-  bool live[ROWS];
-  float2 gv[ROWS][KMAX];
+  // output [h][s][g]: the row's batch entry and g
+  size_t obase[ROWS];
+  const float2* Sr = Ss;
 #pragma unroll
   for (int r = 0; r < ROWS; ++r) {
-    g[r] = tile * 256 * ROWS + r * 256 + threadIdx.x;
-    live[r] = g[r] < ng;
-    size_t base = soff;
-    if (split8) {
-      base |= lo8 | size_t(hib[r]);
-    } else {
-      // global row index over (g, h): g's bits first, then the batch bits
-      const long long grow = (long long)h * ng + (live[r] ? g[r] : 0);
-      for (int j = 0; j < gd.nrow; ++j)
-        if ((grow >> j) & 1) base |= size_t(1) << gd.rowpos[j];
-    }
-    if (pairs) {
-      // the lowest K bit is the stored layout's stride-1 bit: pairs (k, k+1) are
-      // adjacent and 16-byte aligned (every other offset bit is >= 1)
-#pragma unroll
-      for (int kk = 0; kk < KMAX; kk += 2) {
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if ((EXACT || kk < K) && live[r]) v = *reinterpret_cast<const float4*>(G + base + koff[kk]);
-        gv[r][kk] = make_float2(v.x, v.y);
-        gv[r][kk + 1] = make_float2(v.z, v.w);
-      }
-    } else {
-#pragma unroll
-      for (int kk = 0; kk < KMAX; ++kk)
-        gv[r][kk] = ((EXACT || kk < K) && live[r]) ? G[base + koff[kk]] : make_float2(0.f, 0.f);
-    }
+    const long long R = R0 + (live[r] ? r * 256 + t : 0);
+    const size_t h = size_t(R >> log_ng);
+    obase[r] = ((h * size_t(ns)) << log_ng) + size_t(R & ((1ll << log_ng) - 1));
+    if (ROWS == 1) Sr = Ss + (int(h) - h0) * pitch;
   }
-  size_t obase[ROWS];
-#pragma unroll
-  for (int r = 0; r < ROWS; ++r) obase[r] = size_t(h) * ns * ng + size_t(g[r]) * g_stride;
-#pragma unroll
-  for (int s = 0; s < RW_SMAX; ++s) {
-    if (s >= ns) break;
+#pragma unroll 4
+  for (int s = 0; s < ns; ++s) {
     float ar[ROWS], ai[ROWS];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) ar[r] = ai[r] = 0.f;
-    // values beyond K are zero on both sides, so whole pairs are summed
+    if constexpr (K == 1) {
 #pragma unroll
-    for (int kk = 0; kk < KMAX; kk += 2) {
-      if (EXACT || kk < K) {
-        const float4 a2 = *reinterpret_cast<const float4*>(&Ss[s][kk]);
+      for (int r = 0; r < ROWS; ++r) {
+        const float2 a = Sr[s], b = gv[r][0];
+        ar[r] = fmaf(-a.y, b.y, a.x * b.x);
+        ai[r] = fmaf(a.y, b.x, a.x * b.y);
+      }
+    } else {
+#pragma unroll
+      for (int kk = 0; kk < K; kk += 2) {
+        const float4 a2 = *reinterpret_cast<const float4*>(Sr + s * K + kk);
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
           const float2 b0 = gv[r][kk], b1 = gv[r][kk + 1];
@@ -407,7 +350,7 @@ __global__ void __launch_bounds__(256) cgemm_rows_gather_kernel(const float2* __
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
       if (!live[r]) continue;
-      const size_t o = obase[r] + size_t(s) * s_stride;
+      const size_t o = obase[r] + (size_t(s) << log_ng);
       if (acc) {
         double2 v = acc[o];
         v.x += ar[r];
@@ -423,57 +366,61 @@ __global__ void __launch_bounds__(256) cgemm_rows_gather_kernel(const float2* __
 }  // namespace
 
 cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const void* Gsrc, const GatherDesc& gd, void* C, void* acc,
-                                     int ns, int ng, int K, int batch, long long s_stride_out, long long g_stride_out,
-                                     int slice_id, cudaStream_t st) {
-  if (ns < 1 || ns > RW_SMAX || K > 32 || gd.nrow > 32 || gd.nk > 5) return cudaErrorInvalidConfiguration;
-  const int rows = K <= 8 ? 2 : 1;  // rows per thread (more would cut occupancy)
-  const long long tg = (ng + 256 * rows - 1) / (256 * rows);
-  if (tg * batch > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  const dim3 g2{unsigned(tg * batch), 1u, 1u};
+                                     int ns, int ng, int K, int batch, int slice_id, bool round_tf32, int sm_count,
+                                     cudaStream_t st) {
+  if (ns < 1 || ns > GATHER_SMAX || K < 1 || K > 32 || gd.nrow > 32 || gd.nk > 5 || (1 << gd.nk) != K || (ng & (ng - 1)))
+    return cudaErrorInvalidConfiguration;
+  if (ns & (ns - 1)) return cudaErrorInvalidConfiguration;
+  int log_ng = 0, log_per = 0;
+  while ((1 << log_per) < ns * K) ++log_per;
+  while ((1 << log_ng) < ng) ++log_ng;
+  const long long total = (long long)ng * batch;
+  if (total != 1ll << gd.nrow) return cudaErrorInvalidConfiguration;
+  // two rows a thread (each S value read serves both) while registers allow
+  // and the halved grid still covers the chip
+  const int rows = K <= 8 && ng >= 512 && total >= 512ll * 4 * std::max(1, sm_count) ? 2 : 1;
+  long long cta_rows = std::min<long long>(total, 256 * rows);
+  const long long entry_bytes = 8ll * (ns * K + 2);
+  // S rows of every entry of the CTA within 32 KB: fewer rows where many entries meet
+  while (cta_rows > ng && (cta_rows / ng) * entry_bytes > 32 * 1024) cta_rows /= 2;
+  const int entries = int(std::max<long long>(1, cta_rows / ng));
+  const size_t smem = size_t(entries) * size_t(entry_bytes);
+  if (smem > 48 * 1024 || total / cta_rows > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  const unsigned grid = unsigned(total / cta_rows);
   const float2* Sp = reinterpret_cast<const float2*>(Ssmall);
   const float2* Gp = reinterpret_cast<const float2*>(Gsrc);
   float2* Cp = reinterpret_cast<float2*>(C);
   double2* Ap = reinterpret_cast<double2*>(acc);
-#define TNQ_GATHER(KM, R, EX)                                                                               \
-  cgemm_rows_gather_kernel<KM, R, EX><<<g2, 256, 0, st>>>(Sp, Gp, gd, Cp, Ap, ns, ng, K, batch, s_stride_out,  \
-                                                          g_stride_out, int(tg), slice_id)
+#define TNQ_GATHER1(K_, R_, T_) \
+  cgemm_rows_gather_kernel<K_, R_, T_><<<grid, 256, smem, st>>>(Sp, Gp, gd, Cp, Ap, ns, log_per, log_ng, int(cta_rows), entries, \
+                                                      slice_id)
+#define TNQ_GATHER(K_, R_)                   \
+  do {                                       \
+    if (round_tf32) TNQ_GATHER1(K_, R_, true); \
+    else TNQ_GATHER1(K_, R_, false);         \
+  } while (0)
+#define TNQ_GATHER12(K_)           \
+  do {                             \
+    if (rows == 2) TNQ_GATHER(K_, 2); \
+    else TNQ_GATHER(K_, 1);        \
+  } while (0)
   switch (K) {
-    case 2: TNQ_GATHER(2, 2, true); break;
-    case 4: TNQ_GATHER(4, 2, true); break;
-    case 8: TNQ_GATHER(8, 2, true); break;
-    case 16: TNQ_GATHER(16, 1, true); break;
-    case 32: TNQ_GATHER(32, 1, true); break;
-    default:
-      if (K <= 8) TNQ_GATHER(8, 2, false);
-      else if (K <= 16) TNQ_GATHER(16, 1, false);
-      else TNQ_GATHER(32, 1, false);
+    case 1: TNQ_GATHER12(1); break;
+    case 2: TNQ_GATHER12(2); break;
+    case 4: TNQ_GATHER12(4); break;
+    case 8: TNQ_GATHER12(8); break;
+    case 16: TNQ_GATHER(16, 1); break;
+    default: TNQ_GATHER(32, 1);
   }
+#undef TNQ_GATHER12
 #undef TNQ_GATHER
+#undef TNQ_GATHER1
   return cudaGetLastError();
 }
 
 cudaError_t launch_cgemm_rows(const void* Ssmall, const void* Gbig, void* C, void* acc, void* part, int splits,
-                              int ns, int ng, int K, int batch, long long s_stride_out, long long g_stride_out,
-                              cudaStream_t st) {
+                              int ns, int ng, int K, int batch, cudaStream_t st) {
   if (ns < 1 || ns > RW_SMAX || splits < 1 || splits > 65535) return cudaErrorInvalidConfiguration;
-  if (K <= 32 && splits == 1) {
-    // short rows: register-resident rows of the large operand
-    const int rows = K <= 8 ? 2 : 1;
-    const long long tg = (ng + 256 * rows - 1) / (256 * rows);
-    if (tg * batch > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    const dim3 g2{unsigned(tg * batch), 1u, 1u};
-    const float2* Sp = reinterpret_cast<const float2*>(Ssmall);
-    const float2* Gp = reinterpret_cast<const float2*>(Gbig);
-    float2* Cp = reinterpret_cast<float2*>(C);
-    double2* Ap = reinterpret_cast<double2*>(acc);
-    if (K <= 8)
-      cgemm_rows_regk_kernel<8, 2><<<g2, 256, 0, st>>>(Sp, Gp, Cp, Ap, ns, ng, K, batch, s_stride_out, g_stride_out, int(tg));
-    else if (K <= 16)
-      cgemm_rows_regk_kernel<16, 1><<<g2, 256, 0, st>>>(Sp, Gp, Cp, Ap, ns, ng, K, batch, s_stride_out, g_stride_out, int(tg));
-    else
-      cgemm_rows_regk_kernel<32, 1><<<g2, 256, 0, st>>>(Sp, Gp, Cp, Ap, ns, ng, K, batch, s_stride_out, g_stride_out, int(tg));
-    return cudaGetLastError();
-  }
   const long long tiles_g = (ng + RW_THREADS - 1) / RW_THREADS;
   if (tiles_g * batch > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   int kchunk = ((K + splits - 1) / splits + RW_KC - 1) / RW_KC * RW_KC;
@@ -481,7 +428,7 @@ cudaError_t launch_cgemm_rows(const void* Ssmall, const void* Gbig, void* C, voi
   cgemm_rows_kernel<<<grid, RW_THREADS, 0, st>>>(
       reinterpret_cast<const float2*>(Ssmall), reinterpret_cast<const float2*>(Gbig), reinterpret_cast<float2*>(C),
       reinterpret_cast<double2*>(acc), splits > 1 ? reinterpret_cast<float2*>(part) : nullptr, ns, ng, K, batch,
-      s_stride_out, g_stride_out, kchunk, int(tiles_g));
+      kchunk, int(tiles_g));
   return cudaGetLastError();
 }
 

@@ -28,6 +28,18 @@ inline bool skinny(int nM, int nN, int nK) {
 // Whether the rows kernel can run the step (small side <= 32 rows).
 inline bool rows_capable(int nM, int nN) { return (nM < nN ? nM : nN) <= 5; }
 
+// Whether the short-K gather kernel runs the step near the memory bound: K of at
+// most 32 (a row sits in registers) and a small side of at most 128 rows whose
+// 8 M K flops per row of the large operand stay below about 10 flops per byte
+// moved, the FFMA rate over the memory rate (60 TF/s achieved, 6 TB/s).
+inline bool gather_bound(int nM, int nN, int nK) {
+  const int s = nM < nN ? nM : nN;
+  if (nK > 5 || s > 7) return false;
+  if (s <= 5) return true;  // register rows beat staged or tiled kernels even above that line
+  const double m = std::ldexp(1.0, s), k = std::ldexp(1.0, nK);
+  return m * k <= 10.0 * (m + k);
+}
+
 // Tiny outputs (M, N <= 8) with a long contracted dimension: the dot kernel.
 inline bool use_dot(int nM, int nN, int nK) { return nM <= 3 && nN <= 3 && nK >= 10; }
 
