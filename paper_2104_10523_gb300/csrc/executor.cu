@@ -196,9 +196,14 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   // split and multiplied on the tensor cores in one kernel (choice 2, and the
   // default where the shape qualifies).
   const int n_small = std::min(nM, nN), n_big = std::max(nM, nN);
+  // The gather and tall-skinny kernels read the small operand in its stored
+  // layout too, while it stays in L2 (32 MB): each value is read by few CTAs,
+  // and a permute of its own is a launch (6 to 13 us for the gate-sized ones).
+  const bool small_in_place = a_labels.size() <= 22;
   // Long-K tall-skinny steps expand the small operand into scratch A (after
   // the small operand itself when that one is permuted into scratch A)
-  const size_t tr_used = perm_a ? ((8 * (size_t(1) << a_req.size()) + 4095) & ~size_t(4095)) : 0;
+  const size_t tr_used =
+      perm_a && !small_in_place ? ((8 * (size_t(1) << a_req.size()) + 4095) & ~size_t(4095)) : 0;
   char* tr_scratch = scratch_a + tr_used;
   const size_t tr_avail = scratch_a_bytes > tr_used ? scratch_a_bytes - tr_used : 0;
   const bool tc_rows_ok = choice != 0 && choice != 1 && ctx->precision != TNQ_PREC_FP32 && n_small <= 7 &&
@@ -253,7 +258,8 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
     DotOp dot_a, dot_b;
     const bool inpl_a = perm_a && inplace_dot(a_src, a_labels, a_req, &dot_a);
     const bool inpl_b = perm_b && inplace_dot(b_src, b_labels, b_req, &dot_b);
-    if (perm_a && !inpl_a) {
+    const bool small_gather = gather && perm_a && small_in_place;
+    if (perm_a && !inpl_a && !small_gather) {
       build_perm_desc(a_labels.data(), (int)a_labels.size(), a_req.data(), (int)a_req.size(), slice_labels.data(),
                       ns, PM_C64, nK, &d);
       TNQ_CUDA(perm(ctx, d, a_src, scratch_a, nullptr, slice_id, 16.0 * std::ldexp(1.0, (int)a_req.size())));
@@ -277,6 +283,21 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
         if (gd.slice_src[j] >= (int)b_labels.size()) gd.slice_src[j] = -1;
       const int M = 1 << nM, N = 1 << nN, K = 1 << nK, H = 1 << nH;
       const void* Ssm = perm_a ? (const void*)scratch_a : a_src;
+      SmallDesc sd;
+      sd.n = (int)a_req.size();
+      for (int j = 0; j < sd.n; ++j) sd.pos[j] = (signed char)j;
+      if (small_gather) {
+        auto apos = [&](int l) { return int(std::find(a_labels.begin(), a_labels.end(), l) - a_labels.begin()); };
+        size_t soff = 0;
+        for (int j = 0; j < ns; ++j) {
+          const int q = apos(slice_labels[j]);
+          // a sliced label the step keeps is an index, not fixed
+          const bool kept = std::find(a_req.begin(), a_req.end(), slice_labels[j]) != a_req.end();
+          if (!kept && q < (int)a_labels.size() && ((slice_id >> j) & 1)) soff |= size_t(1) << q;
+        }
+        for (int j = 0; j < sd.n; ++j) sd.pos[j] = (signed char)apos(a_req[j]);
+        Ssm = reinterpret_cast<const float2*>(a_src) + soff;
+      }
       KernelRecord r{4, ctx->cur_step, nH, nM, nN, nK, 8.0 * work,
                      8.0 * (std::ldexp(1.0, nH + nM + nK) + std::ldexp(1.0, nH + nN + nK) +
                             (acc ? 2.0 : 1.0) * std::ldexp(1.0, nH + nM + nN)),
@@ -285,10 +306,10 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
       int slot = timing_begin(ctx);
       cudaError_t e;
       if (tc_rows)
-        e = launch_cgemm_tc_rows(Ssm, b_src, gd, C, acc, M, N, K, H, slice_id, ctx->precision, err, ctx->sm_count,
+        e = launch_cgemm_tc_rows(Ssm, sd, b_src, gd, C, acc, M, N, K, H, slice_id, ctx->precision, err, ctx->sm_count,
                                  ctx->stream, tr_scratch, tr_avail);
       else
-        e = launch_cgemm_rows_gather(Ssm, b_src, gd, C, acc, M, N, K, H, slice_id, round_tf32, ctx->sm_count,
+        e = launch_cgemm_rows_gather(Ssm, sd, b_src, gd, C, acc, M, N, K, H, slice_id, round_tf32, ctx->sm_count,
                                      ctx->stream);
       timing_end(ctx, slot, r);
       TNQ_CUDA(e);

@@ -96,7 +96,10 @@ constexpr int TR_ENTRY_Y_LOG2 = 15;           // per-entry grids: batch bits on 
 constexpr int TR_ROWTAB_DIGITS = 7;           // 4-bit digits of a tile index (nrow <= 35)
 
 struct TrParams {
-  const float2* S;        // small operand [batch][ns][K]
+  const float2* S;        // small operand, stored bit order (see sd)
+  SmallDesc sd;
+  int log_k, log_kx;      // log2 of K and of the K values the MMAs read (zero padded beyond K)
+  int log_s, log_sx;      // log2 of ns and of npad / 2 rows (zero padded beyond ns)
   const float2* G;        // large operand, stored bit order (see gd)
   GatherDesc gd;          // rows: g bits then batch bits; K bits in contraction order
   int ns, ng, K, batch;
@@ -208,33 +211,38 @@ __device__ __forceinline__ void store_chunk(uint8_t* hi, uint8_t* lo, int r, con
 
 // Expanded small operand S' for every batch entry: rows n < npad of the reals
 // the MMAs read, hi and lo, built by the converter threads at kernel start.
-__device__ void build_bprime(const TrParams& P, const float2* S, uint8_t* bp, int tid, int nthreads) {
-  const int es = P.kind_bf16 ? 2 : 4;
-  const int reals = P.nks * (32 / es);
-  const int per_h = P.npad * reals;
+__device__ void build_bprime(const TrParams& P, uint32_t h0, uint8_t* bp, int tid, int nthreads) {
   // per batch entry and atom column: npad hi rows, then npad lo rows
   const uint32_t atom_bytes = 2u * uint32_t(P.npad) * TR_ROW_BYTES;
   const uint32_t entry_bytes = atom_bytes * P.atoms;
-  for (int e = tid; e < P.batch * per_h; e += nthreads) {
-    const int h = e / per_h, rem = e % per_h, n = rem / reals, q = rem % reals;
-    const int s = n >> 1, k = q >> 1;
-    float x = 0.f;
-    if (s < P.ns && k < P.K) {
-      const float2 a = S[(size_t(h) * P.ns + s) * P.K + k];
-      // row (s, re): [sr, -si] per k; row (s, im): [si, sr]
-      x = (n & 1) ? ((q & 1) ? a.x : a.y) : ((q & 1) ? -a.y : a.x);
-    }
+  const int log_h = P.log_kx + P.log_sx;
+  // one complex value at a time: it fills two reals of two rows, hi and lo
+  for (int e = tid; e < P.batch << log_h; e += nthreads) {
+    const int k = e & ((1 << P.log_kx) - 1), s = (e >> P.log_kx) & ((1 << P.log_sx) - 1), h = e >> log_h;
+    float2 a = make_float2(0.f, 0.f);
+    if (s < P.ns && k < P.K)
+      a = __ldg(P.S + small_dep(P.sd, ((((h0 + uint32_t(h)) << P.log_s) + s) << P.log_k) + k));
     uint8_t* hi = bp + size_t(h) * entry_bytes;
     uint8_t* lo = hi + uint32_t(P.npad) * TR_ROW_BYTES;  // row npad + n: same swizzle phase (npad % 16 == 0)
-    const uint32_t off = swz(n, (q * es) >> 4, atom_bytes) + uint32_t((q * es) & 15);
+    // row (s, re): [sr, -si] per k; row (s, im): [si, sr]
     if (P.kind_bf16) {
-      const uint32_t hb = bf16_bits(x);
-      *reinterpret_cast<unsigned short*>(hi + off) = (unsigned short)hb;
-      *reinterpret_cast<unsigned short*>(lo + off) = (unsigned short)bf16_bits(x - bf16_val(hb));
+      const uint32_t rh = bf16_bits(a.x), ih = bf16_bits(a.y);
+      const uint32_t rl = bf16_bits(a.x - bf16_val(rh)), il = bf16_bits(a.y - bf16_val(ih));
+      const uint32_t o0 = swz(2 * s, k >> 2, atom_bytes) + (uint32_t(k & 3) << 2);
+      const uint32_t o1 = swz(2 * s + 1, k >> 2, atom_bytes) + (uint32_t(k & 3) << 2);
+      *reinterpret_cast<uint32_t*>(hi + o0) = rh | ((ih ^ 0x8000u) << 16);
+      *reinterpret_cast<uint32_t*>(lo + o0) = rl | ((il ^ 0x8000u) << 16);
+      *reinterpret_cast<uint32_t*>(hi + o1) = ih | (rh << 16);
+      *reinterpret_cast<uint32_t*>(lo + o1) = il | (rl << 16);
     } else {
-      const float hv = tf32_rna(x);
-      *reinterpret_cast<float*>(hi + off) = hv;
-      *reinterpret_cast<float*>(lo + off) = tf32_rna(x - hv);
+      const float rh = tf32_rna(a.x), ih = tf32_rna(a.y);
+      const float rl = tf32_rna(a.x - rh), il = tf32_rna(a.y - ih);
+      const uint32_t o0 = swz(2 * s, k >> 1, atom_bytes) + (uint32_t(k & 1) << 3);
+      const uint32_t o1 = swz(2 * s + 1, k >> 1, atom_bytes) + (uint32_t(k & 1) << 3);
+      *reinterpret_cast<float2*>(hi + o0) = make_float2(rh, -ih);
+      *reinterpret_cast<float2*>(lo + o0) = make_float2(rl, -il);
+      *reinterpret_cast<float2*>(hi + o1) = make_float2(ih, rh);
+      *reinterpret_cast<float2*>(lo + o1) = make_float2(il, rl);
     }
   }
 }
@@ -242,7 +250,7 @@ __device__ void build_bprime(const TrParams& P, const float2* S, uint8_t* bp, in
 // S' of every batch entry expanded into global memory (streamed mode), in the
 // layout build_bprime gives it in shared memory.
 __global__ void build_bprime_kernel(const __grid_constant__ TrParams P, uint8_t* dst) {
-  build_bprime(P, P.S, dst, int(blockIdx.x * blockDim.x + threadIdx.x), int(gridDim.x * blockDim.x));
+  build_bprime(P, 0, dst, int(blockIdx.x * blockDim.x + threadIdx.x), int(gridDim.x * blockDim.x));
 }
 
 // Tile t = h * tph + gt (batch entry h, tile gt within it), stepped by the
@@ -358,7 +366,8 @@ __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const _
         if ((v >> b) & 1) o |= 1u << P.gd.rowpos[7 + 4 * n + b];
       rowtab[n][v] = o;
     }
-  if (warp < TR_CONV_WARPS && !P.stream_bp) build_bprime(P, P.S + size_t(entry()) * P.ns * P.K, bprime, threadIdx.x, 32 * TR_CONV_WARPS);
+  if (warp < TR_CONV_WARPS && !P.stream_bp)
+    build_bprime(P, entry(), bprime, threadIdx.x, 32 * TR_CONV_WARPS);
   if (warp == TR_MMA_WARP) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                  "r"(tmem_cols)
@@ -737,12 +746,13 @@ namespace {
 
 // entry_bits > 0: a per-entry grid over 2^entry_bits batch entries, whose
 // stored positions in G are entry_pos; batch and gd.nrow then exclude them.
-cudaError_t launch_tc_rows_one(const void* Ssmall, const void* Gsrc, const GatherDesc& gd, void* C, void* acc, int ns,
-                               int ng, int K, int batch, int slice_id, int precision, int* err, int sm_count,
+cudaError_t launch_tc_rows_one(const void* Ssmall, const SmallDesc& sd, const void* Gsrc, const GatherDesc& gd, void* C,
+                               void* acc, int ns, int ng, int K, int batch, int slice_id, int precision, int* err, int sm_count,
                                cudaStream_t st, void* scratch = nullptr, size_t scratch_bytes = 0, int entry_bits = 0,
                                const int* entry_pos = nullptr) {
   TrParams P;
   P.S = reinterpret_cast<const float2*>(Ssmall);
+  P.sd = sd;
   P.G = reinterpret_cast<const float2*>(Gsrc);
   P.gd = gd;
   P.ns = ns;
@@ -754,6 +764,15 @@ cudaError_t launch_tc_rows_one(const void* Ssmall, const void* Gsrc, const Gathe
   P.split = precision == TNQ_PREC_TF32 ? 0 : 1;
   const int k_step = P.kind_bf16 ? 8 : 4;  // complex values per 32-byte MMA K step
   P.nks = (K + k_step - 1) / k_step;
+  auto log2_of = [](int v) {
+    int l = 0;
+    while ((1 << l) < v) ++l;
+    return l;
+  };
+  P.log_k = log2_of(K);
+  P.log_kx = log2_of(P.nks * k_step);
+  P.log_s = log2_of(ns);
+  P.log_sx = log2_of(P.npad / 2);
   P.atoms = tr_atoms(K, P.kind_bf16 != 0);
   const size_t bp_all = tr_bprime_bytes(ns, K, batch, P.kind_bf16 != 0);
   const TrStages ts = K > TR_RESIDENT_KMAX ? tr_stages_streamed(P.atoms, P.npad) : tr_stages(P.atoms, bp_all);
@@ -824,7 +843,7 @@ cudaError_t launch_tc_rows_one(const void* Ssmall, const void* Gsrc, const Gathe
                       (P.stream_bp ? 0 : bp_all) + 1024;
   if (P.stream_bp) {
     // S' of every batch entry, expanded once into the scratch for this launch
-    const long long n = (long long)batch * P.npad * P.nks * (32 / (P.kind_bf16 ? 2 : 4));
+    const long long n = (long long)batch << (P.log_kx + P.log_sx);
     const unsigned blocks = unsigned(std::min<long long>((n + 255) / 256, 1024));
     build_bprime_kernel<<<blocks, 256, 0, st>>>(P, reinterpret_cast<uint8_t*>(scratch));
   }
@@ -843,15 +862,16 @@ bool tc_rows_shared_ok(int ns, int K, int batch, int precision) {
   return bp_all <= size_t(TR_BPRIME_BUDGET) && tr_stages(tr_atoms(K, bf16), bp_all).stages >= 2;
 }
 
-cudaError_t launch_cgemm_tc_rows(const void* Ssmall, const void* Gsrc, const GatherDesc& gd, void* C, void* acc, int ns,
+cudaError_t launch_cgemm_tc_rows(const void* Ssmall, const SmallDesc& sd, const void* Gsrc, const GatherDesc& gd, void* C,
+                                 void* acc, int ns,
                                  int ng, int K, int batch, int slice_id, int precision, int* err, int sm_count,
                                  cudaStream_t st, void* scratch, size_t scratch_bytes) {
   if (!tc_rows_supported(ns, ng, K, batch, gd.nrow, precision) || !err) return cudaErrorNotSupported;
-  if (gd.nk > 8 || gd.nrow > 32 || (1 << gd.nk) != K) return cudaErrorInvalidValue;
+  if (gd.nk > 8 || gd.nrow > 32 || (1 << gd.nk) != K || (ns & (ns - 1)) || (batch & (batch - 1))) return cudaErrorInvalidValue;
   cudaError_t pe = tc_rows_prepare();
   if (pe != cudaSuccess) return pe;
   if (tc_rows_shared_ok(ns, K, batch, precision))
-    return launch_tc_rows_one(Ssmall, Gsrc, gd, C, acc, ns, ng, K, batch, slice_id, precision, err, sm_count, st,
+    return launch_tc_rows_one(Ssmall, sd, Gsrc, gd, C, acc, ns, ng, K, batch, slice_id, precision, err, sm_count, st,
                               scratch, scratch_bytes);
   // S' of every batch entry does not fit one CTA: a per-entry grid, whose batch
   // bits (the row bits above the ng bits) come from the CTA index
@@ -861,7 +881,7 @@ cudaError_t launch_cgemm_tc_rows(const void* Ssmall, const void* Gsrc, const Gat
   if (hbits < 0 || (1 << hbits) != batch || hbits > 24) return cudaErrorNotSupported;
   GatherDesc g1 = gd;
   g1.nrow = gbits;
-  return launch_tc_rows_one(Ssmall, Gsrc, g1, C, acc, ns, ng, K, 1, slice_id, precision, err, sm_count, st, nullptr, 0,
+  return launch_tc_rows_one(Ssmall, sd, Gsrc, g1, C, acc, ns, ng, K, 1, slice_id, precision, err, sm_count, st, nullptr, 0,
                             hbits, gd.rowpos + gbits);
 }
 

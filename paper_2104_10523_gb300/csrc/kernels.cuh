@@ -81,10 +81,23 @@ struct GatherDesc {
   int n_slice;
   int slice_src[32];
 };
+// Small operand read in place: bit j of its [K][rows][batch] index (K bits
+// lowest) sits at stored position pos[j].
+struct SmallDesc {
+  int n;
+  signed char pos[32];
+};
+__device__ __forceinline__ uint32_t small_dep(const SmallDesc& d, uint32_t v) {
+  uint32_t o = 0;
+  for (int j = 0; j < d.n && (v >> j); ++j)
+    if ((v >> j) & 1) o |= 1u << d.pos[j];
+  return o;
+}
 // rows kernel with K <= 32 and ns <= 128 reading the large operand in place
-// (fused permute); output [batch][ns][ng].  round_tf32: both operands are
+// (fused permute), the small one as well; output [batch][ns][ng].  round_tf32: both operands are
 // rounded to TF32 first.
-cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const void* Gsrc, const GatherDesc& gd, void* C, void* acc,
+cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const SmallDesc& sd, const void* Gsrc, const GatherDesc& gd,
+                                     void* C, void* acc,
                                      int ns, int ng, int K, int batch, int slice_id, bool round_tf32, int sm_count,
                                      cudaStream_t st);
 

@@ -26,6 +26,7 @@ constexpr int RW_THREADS = 128;  // rows of the large operand per CTA
 constexpr int RW_KC = 32;        // K elements staged per iteration
 constexpr int RW_SMAX = 32;
 constexpr int GATHER_SMAX = 128;  // small-operand rows of the gather kernel
+constexpr int GATHER_REPS = 4;    // row blocks of a CTA
 
 __global__ void __launch_bounds__(RW_THREADS) cgemm_rows_kernel(
     const float2* __restrict__ S, const float2* __restrict__ G, float2* __restrict__ C, double2* __restrict__ acc,
@@ -228,8 +229,10 @@ __device__ __forceinline__ float2 tf32_rna2(float2 v) {
 // dep(k, kpos) further on.  One thread owns ROWS rows, held in registers; a CTA
 // owns cta_rows consecutive rows of the batch-major row index, so with short
 // rows (ng < cta_rows) it serves several batch entries, whose S rows it stages
-// together (one 16-byte pad per entry spreads the entries over the banks);
-// with ROWS = 2 a CTA stays within one entry.
+// together, gathered from their stored layout (one 16-byte pad per entry spreads the entries over the banks);
+// with ROWS = 2 a CTA stays within one entry.  A CTA of a single entry walks
+// reps blocks of rows, so that staging S (a dependent gather before the first
+// row can be used) is paid once for all of them.
 // ROUND rounds both operands to TF32 first (the products are then exact in
 // FP32: the arithmetic of the plain TF32 mode on the CUDA cores).
 //
@@ -238,28 +241,30 @@ __device__ __forceinline__ float2 tf32_rna2(float2 v) {
 // took 33.5 ms as one tensor-core launch each (8 us a launch).
 template <int K, int ROWS, bool ROUND>
 __global__ void __launch_bounds__(256) cgemm_rows_gather_kernel(const float2* __restrict__ S,
+                                                                const __grid_constant__ SmallDesc sd,
                                                                 const float2* __restrict__ G,
                                                                 const __grid_constant__ GatherDesc gd,
                                                                 float2* __restrict__ C, double2* __restrict__ acc,
                                                                 int ns, int log_per, int log_ng, int cta_rows,
-                                                                int entries, int slice_id) {
+                                                                int reps, int entries, int slice_id) {
   extern __shared__ __align__(16) float2 Ss[];  // [entries][ns * K + 2]
-  __shared__ unsigned long long blk_base;
+  __shared__ unsigned long long blk_base[GATHER_REPS];
   const int t = threadIdx.x;
-  const long long R0 = (long long)blockIdx.x * cta_rows;
-  const int h0 = int(R0 >> log_ng);
+  const long long C0 = (long long)blockIdx.x * reps * cta_rows;  // the CTA's first row
+  const int h0 = int(C0 >> log_ng);
   const int per = ns * K, pitch = per + 2;
-  for (int i = t; i < entries * per; i += 256) {
-    const float2 v = S[size_t(h0) * per + i];
-    Ss[i + 2 * (i >> log_per)] = ROUND ? tf32_rna2(v) : v;
-  }
-  if (t == 0) {
+  if (t < reps) {
+    const long long R0 = C0 + (long long)t * cta_rows;
     unsigned long long o = 0;
     for (int j = 0; j < gd.n_slice; ++j)
       if (gd.slice_src[j] >= 0 && ((slice_id >> j) & 1)) o |= 1ull << gd.slice_src[j];
     for (int j = 0; j < gd.nrow; ++j)
       if ((R0 >> j) & 1) o |= 1ull << gd.rowpos[j];
-    blk_base = o;
+    blk_base[t] = o;
+  }
+  for (int i = t; i < entries * per; i += 256) {
+    const float2 v = __ldg(S + small_dep(sd, (uint32_t(h0) << log_per) + i));
+    Ss[i + 2 * (i >> log_per)] = ROUND ? tf32_rna2(v) : v;
   }
   size_t lo = 0;
 #pragma unroll
@@ -267,97 +272,100 @@ __global__ void __launch_bounds__(256) cgemm_rows_gather_kernel(const float2* __
     if (j < gd.nrow && ((t >> j) & 1)) lo |= size_t(1) << gd.rowpos[j];
   __syncthreads();
   const bool pairs = K > 1 && gd.kpos[0] == 0;
-  bool live[ROWS];
-  float2 gv[ROWS][K];
-#pragma unroll
-  for (int r = 0; r < ROWS; ++r) {
-    live[r] = r * 256 + t < cta_rows;
-    size_t base = size_t(blk_base) | lo;
-    if (r) base |= size_t(1) << gd.rowpos[8];  // ROWS <= 2: the row bit above the thread bits
-#pragma unroll
-    for (int kk = 0; kk < K; ++kk) gv[r][kk] = make_float2(0.f, 0.f);
-    if (live[r]) {
-      const float2* p = G + base;
-      if (pairs) {
-        // the lowest K bit is the stored layout's stride-1 bit: pairs (k, k+1) are
-        // adjacent and 16-byte aligned (every other offset bit is >= 1)
-#pragma unroll
-        for (int kk = 0; kk + 1 < K; kk += 2) {
-          uint32_t ko = 0;
-#pragma unroll
-          for (int j = 1; (1 << j) < K; ++j)
-            if ((kk >> j) & 1) ko |= 1u << gd.kpos[j];
-          const float4 v = __ldg(reinterpret_cast<const float4*>(p + ko));
-          gv[r][kk] = make_float2(v.x, v.y);
-          gv[r][kk + 1] = make_float2(v.z, v.w);
-        }
-      } else {
-#pragma unroll
-        for (int kk = 0; kk < K; ++kk) {
-          uint32_t ko = 0;
-#pragma unroll
-          for (int j = 0; (1 << j) < K; ++j)
-            if ((kk >> j) & 1) ko |= 1u << gd.kpos[j];
-          gv[r][kk] = __ldg(p + ko);
-        }
-      }
-    }
-    if (ROUND) {
-#pragma unroll
-      for (int kk = 0; kk < K; ++kk) gv[r][kk] = tf32_rna2(gv[r][kk]);
-    }
-  }
-  // output [h][s][g]: the row's batch entry and g
-  size_t obase[ROWS];
-  const float2* Sr = Ss;
-#pragma unroll
-  for (int r = 0; r < ROWS; ++r) {
-    const long long R = R0 + (live[r] ? r * 256 + t : 0);
-    const size_t h = size_t(R >> log_ng);
-    obase[r] = ((h * size_t(ns)) << log_ng) + size_t(R & ((1ll << log_ng) - 1));
-    if (ROWS == 1) Sr = Ss + (int(h) - h0) * pitch;
-  }
-#pragma unroll 4
-  for (int s = 0; s < ns; ++s) {
-    float ar[ROWS], ai[ROWS];
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r) ar[r] = ai[r] = 0.f;
-    if constexpr (K == 1) {
-#pragma unroll
-      for (int r = 0; r < ROWS; ++r) {
-        const float2 a = Sr[s], b = gv[r][0];
-        ar[r] = fmaf(-a.y, b.y, a.x * b.x);
-        ai[r] = fmaf(a.y, b.x, a.x * b.y);
-      }
-    } else {
-#pragma unroll
-      for (int kk = 0; kk < K; kk += 2) {
-        const float4 a2 = *reinterpret_cast<const float4*>(Sr + s * K + kk);
-#pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
-          const float2 b0 = gv[r][kk], b1 = gv[r][kk + 1];
-          ar[r] = fmaf(a2.x, b0.x, ar[r]);
-          ar[r] = fmaf(-a2.y, b0.y, ar[r]);
-          ai[r] = fmaf(a2.x, b0.y, ai[r]);
-          ai[r] = fmaf(a2.y, b0.x, ai[r]);
-          ar[r] = fmaf(a2.z, b1.x, ar[r]);
-          ar[r] = fmaf(-a2.w, b1.y, ar[r]);
-          ai[r] = fmaf(a2.z, b1.y, ai[r]);
-          ai[r] = fmaf(a2.w, b1.x, ai[r]);
-        }
-      }
-    }
+  for (int it = 0; it < reps; ++it) {
+    const long long R0 = C0 + (long long)it * cta_rows;
+    bool live[ROWS];
+    float2 gv[ROWS][K];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
-      if (!live[r]) continue;
-      const size_t o = obase[r] + (size_t(s) << log_ng);
-      if (acc) {
-        double2 v = acc[o];
-        v.x += ar[r];
-        v.y += ai[r];
-        acc[o] = v;
+      live[r] = r * 256 + t < cta_rows;
+      size_t base = size_t(blk_base[it]) | lo;
+      if (r) base |= size_t(1) << gd.rowpos[8];  // ROWS <= 2: the row bit above the thread bits
+#pragma unroll
+      for (int kk = 0; kk < K; ++kk) gv[r][kk] = make_float2(0.f, 0.f);
+      if (live[r]) {
+        const float2* p = G + base;
+        if (pairs) {
+          // the lowest K bit is the stored layout's stride-1 bit: pairs (k, k+1) are
+          // adjacent and 16-byte aligned (every other offset bit is >= 1)
+#pragma unroll
+          for (int kk = 0; kk + 1 < K; kk += 2) {
+            uint32_t ko = 0;
+#pragma unroll
+            for (int j = 1; (1 << j) < K; ++j)
+              if ((kk >> j) & 1) ko |= 1u << gd.kpos[j];
+            const float4 v = __ldg(reinterpret_cast<const float4*>(p + ko));
+            gv[r][kk] = make_float2(v.x, v.y);
+            gv[r][kk + 1] = make_float2(v.z, v.w);
+          }
+        } else {
+#pragma unroll
+          for (int kk = 0; kk < K; ++kk) {
+            uint32_t ko = 0;
+#pragma unroll
+            for (int j = 0; (1 << j) < K; ++j)
+              if ((kk >> j) & 1) ko |= 1u << gd.kpos[j];
+            gv[r][kk] = __ldg(p + ko);
+          }
+        }
+      }
+      if (ROUND) {
+#pragma unroll
+        for (int kk = 0; kk < K; ++kk) gv[r][kk] = tf32_rna2(gv[r][kk]);
+      }
+    }
+    // output [h][s][g]: the row's batch entry and g
+    size_t obase[ROWS];
+    const float2* Sr = Ss;
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+      const long long R = R0 + (live[r] ? r * 256 + t : 0);
+      const size_t h = size_t(R >> log_ng);
+      obase[r] = ((h * size_t(ns)) << log_ng) + size_t(R & ((1ll << log_ng) - 1));
+      if (ROWS == 1) Sr = Ss + (int(h) - h0) * pitch;
+    }
+#pragma unroll 4
+    for (int s = 0; s < ns; ++s) {
+      float ar[ROWS], ai[ROWS];
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) ar[r] = ai[r] = 0.f;
+      if constexpr (K == 1) {
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+          const float2 a = Sr[s], b = gv[r][0];
+          ar[r] = fmaf(-a.y, b.y, a.x * b.x);
+          ai[r] = fmaf(a.y, b.x, a.x * b.y);
+        }
       } else {
-        C[o] = make_float2(ar[r], ai[r]);
+#pragma unroll
+        for (int kk = 0; kk < K; kk += 2) {
+          const float4 a2 = *reinterpret_cast<const float4*>(Sr + s * K + kk);
+#pragma unroll
+          for (int r = 0; r < ROWS; ++r) {
+            const float2 b0 = gv[r][kk], b1 = gv[r][kk + 1];
+            ar[r] = fmaf(a2.x, b0.x, ar[r]);
+            ar[r] = fmaf(-a2.y, b0.y, ar[r]);
+            ai[r] = fmaf(a2.x, b0.y, ai[r]);
+            ai[r] = fmaf(a2.y, b0.x, ai[r]);
+            ar[r] = fmaf(a2.z, b1.x, ar[r]);
+            ar[r] = fmaf(-a2.w, b1.y, ar[r]);
+            ai[r] = fmaf(a2.z, b1.y, ai[r]);
+            ai[r] = fmaf(a2.w, b1.x, ai[r]);
+          }
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) {
+        if (!live[r]) continue;
+        const size_t o = obase[r] + (size_t(s) << log_ng);
+        if (acc) {
+          double2 v = acc[o];
+          v.x += ar[r];
+          v.y += ai[r];
+          acc[o] = v;
+        } else {
+          C[o] = make_float2(ar[r], ai[r]);
+        }
       }
     }
   }
@@ -365,7 +373,8 @@ __global__ void __launch_bounds__(256) cgemm_rows_gather_kernel(const float2* __
 
 }  // namespace
 
-cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const void* Gsrc, const GatherDesc& gd, void* C, void* acc,
+cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const SmallDesc& sd, const void* Gsrc, const GatherDesc& gd,
+                                     void* C, void* acc,
                                      int ns, int ng, int K, int batch, int slice_id, bool round_tf32, int sm_count,
                                      cudaStream_t st) {
   if (ns < 1 || ns > GATHER_SMAX || K < 1 || K > 32 || gd.nrow > 32 || gd.nk > 5 || (1 << gd.nk) != K || (ng & (ng - 1)))
@@ -386,13 +395,17 @@ cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const void* Gsrc, const
   const int entries = int(std::max<long long>(1, cta_rows / ng));
   const size_t smem = size_t(entries) * size_t(entry_bytes);
   if (smem > 48 * 1024 || total / cta_rows > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  const unsigned grid = unsigned(total / cta_rows);
+  // several row blocks a CTA while the grid still makes a few waves
+  int reps = 1;
+  while (reps < GATHER_REPS && 2 * reps * cta_rows <= ng && total / (2 * reps * cta_rows) >= 16ll * std::max(1, sm_count))
+    reps *= 2;
+  const unsigned grid = unsigned(total / (cta_rows * reps));
   const float2* Sp = reinterpret_cast<const float2*>(Ssmall);
   const float2* Gp = reinterpret_cast<const float2*>(Gsrc);
   float2* Cp = reinterpret_cast<float2*>(C);
   double2* Ap = reinterpret_cast<double2*>(acc);
 #define TNQ_GATHER1(K_, R_, T_) \
-  cgemm_rows_gather_kernel<K_, R_, T_><<<grid, 256, smem, st>>>(Sp, Gp, gd, Cp, Ap, ns, log_per, log_ng, int(cta_rows), entries, \
+  cgemm_rows_gather_kernel<K_, R_, T_><<<grid, 256, smem, st>>>(Sp, sd, Gp, gd, Cp, Ap, ns, log_per, log_ng, int(cta_rows), reps, entries, \
                                                       slice_id)
 #define TNQ_GATHER(K_, R_)                   \
   do {                                       \

@@ -65,3 +65,9 @@ def test_batched_short_k(prec, shape):
 def test_batched_stored_order(prec, shape):
     got, ref = contract(prec, *shape, seed=5, order="stored")
     assert rel(got, ref) <= TOL[prec], rel(got, ref)
+
+
+def test_large_small_operand_is_permuted():
+    """A small operand beyond 2^22 elements leaves the in-place read."""
+    got, ref = contract("fp32", 1, 2, 2, 20, seed=3)
+    assert rel(got, ref) <= TOL["fp32"], rel(got, ref)
