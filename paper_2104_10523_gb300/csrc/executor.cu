@@ -96,6 +96,11 @@ int tc_mode_b(int prec) {
 size_t a_half_bytes(int prec, size_t n) { return prec == TNQ_PREC_BF16X3 ? 8 * n : 16 * n; }
 size_t b_half_bytes(int prec, size_t n) { return prec == TNQ_PREC_BF16X3 ? 4 * n : 8 * n; }
 
+// Largest step (complex multiply-adds) taken from the tall-skinny kernel by the
+// one-launch kernel: its prologue (barriers, TMEM, the expanded small operand)
+// makes about 10 us whatever the size.
+constexpr double kSmallTcRows = 1 << 16;
+
 struct StepOperands {
   const void* a0 = nullptr;
   const void* a1 = nullptr;
@@ -172,13 +177,43 @@ bool host_bits_ok(const Plan* p, int64_t n_bs, const int8_t* bits) {
   return true;
 }
 
+// Where a step's output goes when it may be written in another index order
+// than [N][M][H]: to C with index order `labels` (all of them), `done` telling
+// whether the step did so (else it wrote its own order to the step's C).
+struct DirectOut {
+  void* C = nullptr;
+  const std::vector<int>* labels = nullptr;
+  bool done = false;
+};
+
+// Stored position of each label of `req` in an operand with stored order `st`,
+// and the element offset its sliced labels (those not in `req`) add.
+size_t positions(const std::vector<int>& st, const std::vector<int>& req, const std::vector<int>& slice_labels,
+                 int slice_id, signed char* pos) {
+  auto at = [&](int l) { return int(std::find(st.begin(), st.end(), l) - st.begin()); };
+  for (size_t j = 0; j < req.size(); ++j) pos[j] = (signed char)at(req[j]);
+  size_t off = 0;
+  for (size_t j = 0; j < slice_labels.size(); ++j) {
+    const int q = at(slice_labels[j]);
+    // a sliced label the step keeps is an index, not fixed
+    const bool kept = std::find(req.begin(), req.end(), slice_labels[j]) != req.end();
+    if (!kept && q < (int)st.size() && ((slice_id >> j) & 1)) off |= size_t(1) << q;
+  }
+  return off;
+}
+
+// A step small enough for the one-launch kernel: at most 2^18 complex
+// multiply-adds (a 64 x 64 x 64 contraction took 45 us in four launches) and a
+// contracted extent its table holds.
+bool small_step(int nH, int nM, int nN, int nK) { return nH + nM + nN + nK <= 18 && nK <= SMALL_MAX_K; }
+
 // Prepare operands (permute / convert) and run one batched complex GEMM.
 tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_labels, bool perm_a,
                          const void* b_src, const std::vector<int>& b_labels, bool perm_b,
                          const std::vector<int>& a_req, const std::vector<int>& b_req,
                          const std::vector<int>& slice_labels, int slice_id, int nH, int nM, int nN, int nK,
                          char* scratch_a, char* scratch_b, void* C, void* acc, int* err, void* part,
-                         size_t scratch_a_bytes, int choice = -1) {
+                         size_t scratch_a_bytes, int choice = -1, DirectOut* direct = nullptr) {
   // Small, skinny or K-degenerate steps run on the CUDA cores in FP32 whatever
   // the mode: they are launch- or bandwidth-bound and a tensor-core tile would
   // idle.  An autotuned choice (0 CUDA cores, 1 tensor cores) overrides the rule.
@@ -191,6 +226,7 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   const int prec = use_tc ? ctx->precision : TNQ_PREC_FP32;
   StepOperands op;
   PermDesc d;
+  signed char pos_a[32], pos_b[32];
   const int ns = (int)slice_labels.size();
   // Tall-skinny steps in the tensor-core modes: the large operand is gathered,
   // split and multiplied on the tensor cores in one kernel (choice 2, and the
@@ -221,6 +257,50 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   // The A side is never the larger one (both hold the H and K labels), so M is
   // the small side of a skinny step.
   const bool gather = tc_rows || batched || (!use_tc && !use_dot(nM, nN, nK) && gather_bound(nM, nN, nK));
+  // Small steps of the CUDA-core path, and of the tall-skinny kernel's where a
+  // launch of it (about 10 us) is all latency, run in one launch.
+  if (!use_tc && small_step(nH, nM, nN, nK) && (!tc_rows || (choice == -1 && work <= kSmallTcRows))) {
+    SmallOp s;
+    const size_t off_a = positions(a_labels, a_req, slice_labels, slice_id, pos_a);
+    const size_t off_b = positions(b_labels, b_req, slice_labels, slice_id, pos_b);
+    s.A = reinterpret_cast<const float2*>(a_src) + off_a;
+    s.B = reinterpret_cast<const float2*>(b_src) + off_b;
+    s.C = reinterpret_cast<float2*>(C);
+    s.acc = reinterpret_cast<double2*>(acc);
+    s.nk = nK;
+    s.n_out = nN + nM + nH;
+    s.log_l = small_lanes_log2(s.n_out, nK);
+    s.round_tf32 = (tc_rows || batched) && ctx->precision == TNQ_PREC_TF32;
+    for (int j = 0; j < nK; ++j) {
+      s.ka[j] = pos_a[j];
+      s.kb[j] = pos_b[j];
+    }
+    // output bits [N][M][H]
+    for (int j = 0; j < s.n_out; ++j) {
+      const bool is_n = j < nN, is_m = !is_n && j < nN + nM;
+      s.pb[j] = is_n ? pos_b[nK + j] : is_m ? -1 : pos_b[nK + j - nM];
+      s.pa[j] = is_n ? -1 : pos_a[nK + j - nN];
+      s.pc[j] = (signed char)j;
+    }
+    if (direct) {
+      s.C = reinterpret_cast<float2*>(direct->C);
+      for (int j = 0; j < s.n_out; ++j) {
+        const int l = j < nN ? b_req[nK + j] : a_req[nK + j - nN];
+        s.pc[j] = (signed char)(std::find(direct->labels->begin(), direct->labels->end(), l) - direct->labels->begin());
+      }
+      direct->done = true;
+    }
+    KernelRecord r{nM <= 5 || use_dot(nM, nN, nK) ? 4 : 1, ctx->cur_step, nH, nM, nN, nK, 8.0 * work,
+                   8.0 * (std::ldexp(1.0, nH + nM + nK) + std::ldexp(1.0, nH + nN + nK) +
+                          (acc ? 2.0 : 1.0) * std::ldexp(1.0, nH + nM + nN)),
+                   0.f};
+    int slot = timing_begin(ctx);
+    cudaError_t e = launch_cgemm_small(s, ctx->stream);
+    timing_end(ctx, slot, r);
+    TNQ_CUDA(e);
+    ctx->launches++;
+    return TNQ_OK;
+  }
   if (gather || (!use_tc && (rows_capable(nM, nN) || use_dot(nM, nN, nK)) && part)) {
     // bandwidth-bound skinny step: complex64 operands in [h][m|n][k] order; the
     // large operand of a short-K step is read in its stored layout (fused
@@ -287,16 +367,7 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
       sd.n = (int)a_req.size();
       for (int j = 0; j < sd.n; ++j) sd.pos[j] = (signed char)j;
       if (small_gather) {
-        auto apos = [&](int l) { return int(std::find(a_labels.begin(), a_labels.end(), l) - a_labels.begin()); };
-        size_t soff = 0;
-        for (int j = 0; j < ns; ++j) {
-          const int q = apos(slice_labels[j]);
-          // a sliced label the step keeps is an index, not fixed
-          const bool kept = std::find(a_req.begin(), a_req.end(), slice_labels[j]) != a_req.end();
-          if (!kept && q < (int)a_labels.size() && ((slice_id >> j) & 1)) soff |= size_t(1) << q;
-        }
-        for (int j = 0; j < sd.n; ++j) sd.pos[j] = (signed char)apos(a_req[j]);
-        Ssm = reinterpret_cast<const float2*>(a_src) + soff;
+        Ssm = reinterpret_cast<const float2*>(a_src) + positions(a_labels, a_req, slice_labels, slice_id, sd.pos);
       }
       KernelRecord r{4, ctx->cur_step, nH, nM, nN, nK, 8.0 * work,
                      8.0 * (std::ldexp(1.0, nH + nM + nK) + std::ldexp(1.0, nH + nN + nK) +
@@ -1148,20 +1219,25 @@ tnq_status exec_contract_pair(Ctx* ctx, const void* A, int ra, const int* al, co
   char* sc = sb + ((16 * na + 4095) & ~size_t(4095));
   int* err = reinterpret_cast<int*>(sc + ((8 * (size_t(1) << rc) + 4095) & ~size_t(4095)));
   char* part = reinterpret_cast<char*>(err) + 4096;
-  TNQ_CUDA(cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
-  bool direct = out == lc;
+  // only the tensor-core kernels' bounded waits can raise the flag
+  const bool flagged = ctx->precision != TNQ_PREC_FP32;
+  if (flagged) TNQ_CUDA(cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
+  const bool direct = out == lc;
+  DirectOut dout;
+  dout.C = C;
+  dout.labels = &lc;
   std::vector<int> none;
   tnq_status st = run_gemm_step(ctx, pa, xa, xa != a_req, pb, xb, xb != b_req, a_req, b_req, none, 0,
                                 (int)Hh.size(), (int)M.size(), (int)N.size(), (int)K.size(), sa, sb,
-                                direct ? C : (void*)sc, nullptr, err, part, size_t(sb - sa));
+                                direct ? C : (void*)sc, nullptr, err, part, size_t(sb - sa), -1, &dout);
   if (st != TNQ_OK) return st;
-  if (!direct) {
+  if (!direct && !dout.done) {
     PermDesc d;
     build_perm_desc(out.data(), (int)out.size(), lc.data(), rc, nullptr, 0, PM_C64, 0, &d);
     TNQ_CUDA(perm(ctx, d, sc, C, nullptr, 0, 16.0 * std::ldexp(1.0, rc)));
   }
   int herr = 0;
-  TNQ_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  if (flagged) TNQ_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
   if (ctx->timing) {
     tnq_status ts = timing_collect(ctx);

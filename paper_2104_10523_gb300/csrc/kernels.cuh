@@ -101,6 +101,25 @@ cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const SmallDesc& sd, co
                                      int ns, int ng, int K, int batch, int slice_id, bool round_tf32, int sm_count,
                                      cudaStream_t st);
 
+// One small contraction reading both operands in place (see small.cu): bit j of
+// an output index (2^n_out of them) sits at stored position pa[j] of A, pb[j]
+// of B (-1: not an index of that operand) and pc[j] of C; bit j of the
+// contracted index at ka[j], kb[j].  With acc the result is added in FP64.
+constexpr int SMALL_MAX_K = 10;  // log2 of the longest contracted extent
+struct SmallOp {
+  const float2* A;   // slice offsets already added
+  const float2* B;
+  float2* C;
+  double2* acc;
+  int n_out, nk;
+  int log_l;         // log2 of the lanes sharing an output (small_lanes_log2)
+  int round_tf32;    // round the operands to TF32 first
+  signed char pa[32], pb[32], pc[32];
+  signed char ka[SMALL_MAX_K], kb[SMALL_MAX_K];
+};
+int small_lanes_log2(int n_out, int nk);
+cudaError_t launch_cgemm_small(const SmallOp& op, cudaStream_t st);
+
 // Projection leaves j < n_proj at leaves_base + j * stride_bytes:
 // P_j[(b << 1) | x] = [bits[b * row_len + tab[j]] == x] for b < n_valid, else 0.
 // tab (device) also lists, after the n_proj entries, the n_open row entries
