@@ -236,10 +236,10 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   // layout too, while it stays in L2 (32 MB): each value is read by few CTAs,
   // and a permute of its own is a launch (6 to 13 us for the gate-sized ones).
   const bool small_in_place = a_labels.size() <= 22;
-  // Long-K tall-skinny steps expand the small operand into scratch A (after
-  // the small operand itself when that one is permuted into scratch A)
-  const size_t tr_used =
-      perm_a && !small_in_place ? ((8 * (size_t(1) << a_req.size()) + 4095) & ~size_t(4095)) : 0;
+  // Long-K tall-skinny steps expand the small operand into scratch A, after the
+  // place of its permuted copy (kept free where the operand is read in place,
+  // so that which kernel a step takes does not hang on that)
+  const size_t tr_used = perm_a ? ((8 * (size_t(1) << a_req.size()) + 4095) & ~size_t(4095)) : 0;
   char* tr_scratch = scratch_a + tr_used;
   const size_t tr_avail = scratch_a_bytes > tr_used ? scratch_a_bytes - tr_used : 0;
   const bool tc_rows_ok = choice != 0 && choice != 1 && ctx->precision != TNQ_PREC_FP32 && n_small <= 7 &&
@@ -259,7 +259,40 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   const bool gather = tc_rows || batched || (!use_tc && !use_dot(nM, nN, nK) && gather_bound(nM, nN, nK));
   // Small steps of the CUDA-core path, and of the tall-skinny kernel's where a
   // launch of it (about 10 us) is all latency, run in one launch.
-  if (!use_tc && small_step(nH, nM, nN, nK) && (!tc_rows || (choice == -1 && work <= kSmallTcRows))) {
+  const bool small = !use_tc && small_step(nH, nM, nN, nK) && (!tc_rows || (choice == -1 && work <= kSmallTcRows));
+  const bool kdot = !small && !gather && !use_tc && use_kdot(nM, nN, nK) && part;
+  signed char pos_c[32];  // positions in C of the output bits [N][M][H]
+  for (int j = 0; j < nN + nM + nH && j < 32; ++j) pos_c[j] = (signed char)j;
+  if ((small || kdot) && direct) {
+    for (int j = 0; j < nN + nM + nH; ++j) {
+      const int l = j < nN ? b_req[nK + j] : a_req[nK + j - nN];
+      pos_c[j] = (signed char)(std::find(direct->labels->begin(), direct->labels->end(), l) - direct->labels->begin());
+    }
+    C = direct->C;
+    direct->done = true;
+  }
+  if (kdot) {
+    KdotDesc kd;
+    const size_t off_a = positions(a_labels, a_req, slice_labels, slice_id, pos_a);
+    const size_t off_b = positions(b_labels, b_req, slice_labels, slice_id, pos_b);
+    if (!build_kdot(nM, nN, nK, nH, pos_a, pos_b, pos_c, &kd))
+      return fail(TNQ_ERR_NOT_SUPPORTED, "contraction too large for the long-K kernel");
+    const int splits = kdot_splits(nH, nM, nN, nK);
+    KernelRecord r{4, ctx->cur_step, nH, nM, nN, nK, 8.0 * work,
+                   8.0 * (std::ldexp(1.0, nH + nM + nK) + std::ldexp(1.0, nH + nN + nK) +
+                          (acc ? 2.0 : 1.0) * std::ldexp(1.0, nH + nM + nN)),
+                   0.f};
+    int slot = timing_begin(ctx);
+    cudaError_t e = launch_cgemm_kdot(kd, reinterpret_cast<const float2*>(a_src) + off_a,
+                                      reinterpret_cast<const float2*>(b_src) + off_b, C, acc, part, splits, ctx->stream);
+    if (e == cudaSuccess && splits > 1)
+      e = launch_reduce_splits(part, splits, out_elems, C, acc, ctx->sm_count, ctx->stream);
+    timing_end(ctx, slot, r);
+    TNQ_CUDA(e);
+    ctx->launches += splits > 1 ? 2 : 1;
+    return TNQ_OK;
+  }
+  if (small) {
     SmallOp s;
     const size_t off_a = positions(a_labels, a_req, slice_labels, slice_id, pos_a);
     const size_t off_b = positions(b_labels, b_req, slice_labels, slice_id, pos_b);
@@ -280,15 +313,7 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
       const bool is_n = j < nN, is_m = !is_n && j < nN + nM;
       s.pb[j] = is_n ? pos_b[nK + j] : is_m ? -1 : pos_b[nK + j - nM];
       s.pa[j] = is_n ? -1 : pos_a[nK + j - nN];
-      s.pc[j] = (signed char)j;
-    }
-    if (direct) {
-      s.C = reinterpret_cast<float2*>(direct->C);
-      for (int j = 0; j < s.n_out; ++j) {
-        const int l = j < nN ? b_req[nK + j] : a_req[nK + j - nN];
-        s.pc[j] = (signed char)(std::find(direct->labels->begin(), direct->labels->end(), l) - direct->labels->begin());
-      }
-      direct->done = true;
+      s.pc[j] = pos_c[j];
     }
     KernelRecord r{nM <= 5 || use_dot(nM, nN, nK) ? 4 : 1, ctx->cur_step, nH, nM, nN, nK, 8.0 * work,
                    8.0 * (std::ldexp(1.0, nH + nM + nK) + std::ldexp(1.0, nH + nN + nK) +
@@ -301,117 +326,50 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
     ctx->launches++;
     return TNQ_OK;
   }
-  if (gather || (!use_tc && (rows_capable(nM, nN) || use_dot(nM, nN, nK)) && part)) {
-    // bandwidth-bound skinny step: complex64 operands in [h][m|n][k] order; the
-    // large operand of a short-K step is read in its stored layout (fused
-    // gather) instead of being permuted first.
-    // Dot steps read an operand in place when its stored layout starts with at
-    // least 2^5 K values in the required K order (one contiguous run) and keeps
-    // every K bit above the run in K order too (the kernel steps its K offset
-    // by adding in the deposited domain, which needs increasing positions).
-    auto inplace_dot = [&](const void* src, const std::vector<int>& st, const std::vector<int>& req, DotOp* d) {
-      if (!use_dot(nM, nN, nK) || nK > 40 || (int)req.size() - nK > 24) return false;
-      auto spos = [&](int l) { return int(std::find(st.begin(), st.end(), l) - st.begin()); };
-      *d = DotOp{};
-      d->nk = nK;
-      d->kmask = 0;
-      for (int j = 0; j < nK; ++j) {
-        const int q = spos(req[j]);
-        if (q >= (int)st.size() || (j < 5 && q != j) || (j > 0 && q <= d->kpos[j - 1])) return false;
-        d->kpos[j] = (signed char)q;
-        d->kmask |= 1ull << q;
-      }
-      d->nrow = (int)req.size() - nK;
-      for (int j = 0; j < d->nrow; ++j) {
-        const int q = spos(req[nK + j]);
-        if (q >= (int)st.size()) return false;
-        d->rowpos[j] = (signed char)q;
-      }
-      size_t soff = 0;
-      for (int j = 0; j < ns; ++j) {
-        const int q = spos(slice_labels[j]);
-        if (q < (int)st.size() && ((slice_id >> j) & 1)) soff |= size_t(1) << q;
-      }
-      d->p = reinterpret_cast<const float2*>(src) + soff;
-      return true;
-    };
-    DotOp dot_a, dot_b;
-    const bool inpl_a = perm_a && inplace_dot(a_src, a_labels, a_req, &dot_a);
-    const bool inpl_b = perm_b && inplace_dot(b_src, b_labels, b_req, &dot_b);
-    const bool small_gather = gather && perm_a && small_in_place;
-    if (perm_a && !inpl_a && !small_gather) {
+  if (gather) {
+    // bandwidth-bound short-K step: both operands are read in their stored
+    // layouts (fused permutes) unless the small one outgrows L2
+    const bool small_gather = perm_a && small_in_place;
+    if (perm_a && !small_gather) {
       build_perm_desc(a_labels.data(), (int)a_labels.size(), a_req.data(), (int)a_req.size(), slice_labels.data(),
                       ns, PM_C64, nK, &d);
       TNQ_CUDA(perm(ctx, d, a_src, scratch_a, nullptr, slice_id, 16.0 * std::ldexp(1.0, (int)a_req.size())));
     }
-    if (perm_b && !inpl_b && !gather) {
-      build_perm_desc(b_labels.data(), (int)b_labels.size(), b_req.data(), (int)b_req.size(), slice_labels.data(),
-                      ns, PM_C64, nK, &d);
-      TNQ_CUDA(perm(ctx, d, b_src, scratch_b, nullptr, slice_id, 16.0 * std::ldexp(1.0, (int)b_req.size())));
-    }
-    if (gather) {
-      // large operand: required order [K][rows][H]; find each bit in its stored labels
-      auto spos = [&](int l) { return int(std::find(b_labels.begin(), b_labels.end(), l) - b_labels.begin()); };
-      GatherDesc gd;
-      gd.nk = nK;
-      for (int j = 0; j < nK; ++j) gd.kpos[j] = spos(b_req[j]);
-      gd.nrow = (int)b_req.size() - nK;
-      for (int j = 0; j < gd.nrow; ++j) gd.rowpos[j] = spos(b_req[nK + j]);
-      gd.n_slice = ns;
-      for (int j = 0; j < 32; ++j) gd.slice_src[j] = j < ns ? spos(slice_labels[j]) : -1;
-      for (int j = 0; j < ns; ++j)
-        if (gd.slice_src[j] >= (int)b_labels.size()) gd.slice_src[j] = -1;
-      const int M = 1 << nM, N = 1 << nN, K = 1 << nK, H = 1 << nH;
-      const void* Ssm = perm_a ? (const void*)scratch_a : a_src;
-      SmallDesc sd;
-      sd.n = (int)a_req.size();
-      for (int j = 0; j < sd.n; ++j) sd.pos[j] = (signed char)j;
-      if (small_gather) {
-        Ssm = reinterpret_cast<const float2*>(a_src) + positions(a_labels, a_req, slice_labels, slice_id, sd.pos);
-      }
-      KernelRecord r{4, ctx->cur_step, nH, nM, nN, nK, 8.0 * work,
-                     8.0 * (std::ldexp(1.0, nH + nM + nK) + std::ldexp(1.0, nH + nN + nK) +
-                            (acc ? 2.0 : 1.0) * std::ldexp(1.0, nH + nM + nN)),
-                     0.f};
-      if (tc_rows) r.kind = 5;
-      int slot = timing_begin(ctx);
-      cudaError_t e;
-      if (tc_rows)
-        e = launch_cgemm_tc_rows(Ssm, sd, b_src, gd, C, acc, M, N, K, H, slice_id, ctx->precision, err, ctx->sm_count,
-                                 ctx->stream, tr_scratch, tr_avail);
-      else
-        e = launch_cgemm_rows_gather(Ssm, sd, b_src, gd, C, acc, M, N, K, H, slice_id, round_tf32, ctx->sm_count,
-                                     ctx->stream);
-      timing_end(ctx, slot, r);
-      TNQ_CUDA(e);
-      ctx->launches++;
-      return TNQ_OK;
-    }
-    const void* A = perm_a ? (const void*)scratch_a : a_src;
-    const void* B = perm_b ? (const void*)scratch_b : b_src;
+    // large operand: required order [K][rows][H]; find each bit in its stored labels
+    auto spos = [&](int l) { return int(std::find(b_labels.begin(), b_labels.end(), l) - b_labels.begin()); };
+    GatherDesc gd;
+    gd.nk = nK;
+    for (int j = 0; j < nK; ++j) gd.kpos[j] = spos(b_req[j]);
+    gd.nrow = (int)b_req.size() - nK;
+    for (int j = 0; j < gd.nrow; ++j) gd.rowpos[j] = spos(b_req[nK + j]);
+    gd.n_slice = ns;
+    for (int j = 0; j < 32; ++j) gd.slice_src[j] = j < ns ? spos(slice_labels[j]) : -1;
+    for (int j = 0; j < ns; ++j)
+      if (gd.slice_src[j] >= (int)b_labels.size()) gd.slice_src[j] = -1;
     const int M = 1 << nM, N = 1 << nN, K = 1 << nK, H = 1 << nH;
+    const void* Ssm = perm_a ? (const void*)scratch_a : a_src;
+    SmallDesc sd;
+    sd.n = (int)a_req.size();
+    for (int j = 0; j < sd.n; ++j) sd.pos[j] = (signed char)j;
+    if (small_gather) {
+      Ssm = reinterpret_cast<const float2*>(a_src) + positions(a_labels, a_req, slice_labels, slice_id, sd.pos);
+    }
     KernelRecord r{4, ctx->cur_step, nH, nM, nN, nK, 8.0 * work,
                    8.0 * (std::ldexp(1.0, nH + nM + nK) + std::ldexp(1.0, nH + nN + nK) +
                           (acc ? 2.0 : 1.0) * std::ldexp(1.0, nH + nM + nN)),
                    0.f};
+    if (tc_rows) r.kind = 5;
     int slot = timing_begin(ctx);
     cudaError_t e;
-    int splits;
-    if (use_dot(nM, nN, nK)) {
-      splits = dot_splits(nH, nM, nN, nK);
-      if (!inpl_a) dot_a = dot_contiguous(A, M, K, H);
-      if (!inpl_b) dot_b = dot_contiguous(B, N, K, H);
-      e = launch_cdot_ops(dot_a, dot_b, part, splits, M, N, K, H, ctx->stream);
-      if (e == cudaSuccess) e = launch_reduce_splits(part, splits, out_elems, C, acc, ctx->sm_count, ctx->stream);
-    } else {
-      splits = rows_splits(nH, nM, nN, nK);
-      e = launch_cgemm_rows(A, B, C, acc, part, splits, M, N, K, H, ctx->stream);
-      if (e == cudaSuccess && splits > 1)
-        e = launch_reduce_splits(part, splits, out_elems, C, acc, ctx->sm_count, ctx->stream);
-    }
+    if (tc_rows)
+      e = launch_cgemm_tc_rows(Ssm, sd, b_src, gd, C, acc, M, N, K, H, slice_id, ctx->precision, err, ctx->sm_count,
+                               ctx->stream, tr_scratch, tr_avail);
+    else
+      e = launch_cgemm_rows_gather(Ssm, sd, b_src, gd, C, acc, M, N, K, H, slice_id, round_tf32, ctx->sm_count,
+                                   ctx->stream);
     timing_end(ctx, slot, r);
     TNQ_CUDA(e);
-    ctx->launches += (use_dot(nM, nN, nK) || splits > 1) ? 2 : 1;
+    ctx->launches++;
     return TNQ_OK;
   }
   if (prec == TNQ_PREC_FP32) {

@@ -513,8 +513,44 @@ __global__ void reduce_splits_kernel(const float2* __restrict__ part, int splits
   }
 }
 
+// Few outputs of many splits: a warp per output, lanes over the splits (each
+// sums its splits in order, the lanes meet in a fixed tree), so that the loads
+// of an output are in flight together instead of one after the other.
+__global__ void reduce_splits_warp_kernel(const float2* __restrict__ part, int splits, size_t n, float2* __restrict__ C,
+                                          double2* __restrict__ acc) {
+  const size_t i = (blockIdx.x * size_t(blockDim.x) + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (i >= n) return;
+  double re = 0, im = 0;
+  for (int s = lane; s < splits; s += 32) {
+    const float2 v = part[size_t(s) * n + i];
+    re += v.x;
+    im += v.y;
+  }
+  for (int d = 16; d; d >>= 1) {
+    re += __shfl_xor_sync(0xffffffffu, re, d);
+    im += __shfl_xor_sync(0xffffffffu, im, d);
+  }
+  if (lane) return;
+  if (acc) {
+    double2 t = acc[i];
+    t.x += re;
+    t.y += im;
+    acc[i] = t;
+  } else {
+    C[i] = make_float2(float(re), float(im));
+  }
+}
+
 cudaError_t launch_reduce_splits(const void* part, int splits, size_t n, void* C, void* acc, int sm_count,
                                  cudaStream_t st) {
+  // a warp each while the warps are few (reading 32 splits of one output is
+  // uncoalesced, which a small partial array in L2 does not mind)
+  if (splits >= 16 && n <= 4096) {
+    reduce_splits_warp_kernel<<<unsigned((n * 32 + 255) / 256), 256, 0, st>>>(
+        reinterpret_cast<const float2*>(part), splits, n, reinterpret_cast<float2*>(C), reinterpret_cast<double2*>(acc));
+    return cudaGetLastError();
+  }
   size_t blocks = std::min<size_t>((n + 255) / 256, size_t(sm_count) * 8);
   if (blocks < 1) blocks = 1;
   reduce_splits_kernel<<<(unsigned)blocks, 256, 0, st>>>(reinterpret_cast<const float2*>(part), splits, n,

@@ -49,27 +49,27 @@ cudaError_t launch_cgemm_simt(const void* A, const void* B, void* C, void* acc, 
 cudaError_t launch_reduce_splits(const void* part, int splits, size_t n, void* C, void* acc, int sm_count,
                                  cudaStream_t st);
 
-// Skinny steps (see skinny.cu).  rows: C = S x G^T for a small operand S of
-// ns <= 32 rows and ng rows of the large operand; output [batch][ns][ng].
-// dot: M, N <= 8; always writes FP32 partials [splits][batch][M][N].
-cudaError_t launch_cgemm_rows(const void* Ssmall, const void* Gbig, void* C, void* acc, void* part, int splits,
-                              int ns, int ng, int K, int batch, cudaStream_t st);
-cudaError_t launch_cdot(const void* A, const void* B, void* part, int splits, int M, int N, int K, int batch,
-                        cudaStream_t st);
-// Operand of the dot kernel addressed through bit deposits: element (row r of
-// batch entry h, k) sits at p + dep(h * rows + r, rowpos) + dep(k, kpos), with
-// kmask = OR of 1 << kpos[j].  kpos[0] must be 0 (16-byte pair loads) and
-// kpos must increase.
-struct DotOp {
-  const float2* p;              // slice offset already added
-  unsigned long long kmask;
-  int nk, nrow;
-  signed char kpos[40];
-  signed char rowpos[24];
+// Long-K step with at most 32 rows on its small side (see kdot.cu).  The tile
+// lists hold its stored bits in increasing position with their place in the
+// tile (K bit i of the tile, or -1 - i for row bit i); ko: K bits outside the
+// tile; u: batch bits (nh of them), then N bits outside the tile.
+constexpr int KD_DIGITS = 7;  // 4-bit digits of a K tile index
+struct KdotDesc {
+  int na, nb;          // tile bits of A and B
+  int tm, tn, tk;      // log2 of M rows, N rows and K values of a tile
+  int nko, nh, nu;
+  int nc;              // log2 of the output elements (stride of a split's partials)
+  signed char a_pos[16], a_to[16], b_pos[16], b_to[16];
+  signed char ko_a[28], ko_b[28];
+  signed char u_a[32], u_b[32], u_c[32];
+  signed char m_c[8], n_c[8];
 };
-DotOp dot_contiguous(const void* p, int rows, int K, int batch);
-cudaError_t launch_cdot_ops(const DotOp& A, const DotOp& B, void* part, int splits, int M, int N, int K, int batch,
-                            cudaStream_t st);
+// pos_a / pos_b: stored positions of [K][M][H] and [K][N][H]; pos_c: positions
+// in C of the output bits [N][M][H].
+bool build_kdot(int nM, int nN, int nK, int nH, const signed char* pos_a, const signed char* pos_b,
+                const signed char* pos_c, KdotDesc* d);
+cudaError_t launch_cgemm_kdot(const KdotDesc& d, const void* A, const void* B, void* C, void* acc, void* part,
+                              int splits, cudaStream_t st);
 
 // Bit positions (in the large operand's stored layout) of its row index (the
 // N or M bits, then the batch bits) and of its K bits, plus sliced labels.

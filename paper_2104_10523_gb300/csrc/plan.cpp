@@ -271,9 +271,9 @@ void layout_steps(Plan* p) {
   size_t max_part = 0;
   for (auto& s : p->steps) {
     int sp = std::max({simt_splits(s.nH, s.nM, s.nN, s.nK), tc_splits(s.nH, s.nM, s.nN, s.nK, true),
-                       tc_splits(s.nH, s.nM, s.nN, s.nK, false), rows_splits(s.nH, s.nM, s.nN, s.nK)});
-    if (use_dot(s.nM, s.nN, s.nK)) sp = std::max(sp, dot_splits(s.nH, s.nM, s.nN, s.nK));
-    if (sp > 1 || use_dot(s.nM, s.nN, s.nK))
+                       tc_splits(s.nH, s.nM, s.nN, s.nK, false)});
+    if (use_kdot(s.nM, s.nN, s.nK)) sp = std::max(sp, kdot_splits(s.nH, s.nM, s.nN, s.nK));
+    if (sp > 1)
       max_part = std::max(max_part, size_t(sp) * 8 * (size_t(1) << (s.nH + s.nM + s.nN)));
   }
   p->ws_partial = off;

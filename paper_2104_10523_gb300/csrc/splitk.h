@@ -25,9 +25,6 @@ inline bool skinny(int nM, int nN, int nK) {
   return s <= 4;
 }
 
-// Whether the rows kernel can run the step (small side <= 32 rows).
-inline bool rows_capable(int nM, int nN) { return (nM < nN ? nM : nN) <= 5; }
-
 // Whether the short-K gather kernel runs the step near the memory bound: K of at
 // most 32 (a row sits in registers) and a small side of at most 128 rows whose
 // 8 M K flops per row of the large operand stay below about 10 flops per byte
@@ -40,7 +37,8 @@ inline bool gather_bound(int nM, int nN, int nK) {
   return m * k <= 10.0 * (m + k);
 }
 
-// Tiny outputs (M, N <= 8) with a long contracted dimension: the dot kernel.
+// Tiny outputs (M, N <= 8) with a long contracted dimension never fill a
+// tensor-core tile.
 inline bool use_dot(int nM, int nN, int nK) { return nM <= 3 && nN <= 3 && nK >= 10; }
 
 // tiles: CTAs without splitting; kunits: K extent in units the split may cut
@@ -58,18 +56,23 @@ inline int simt_splits(int nH, int nM, int nN, int nK) {
   return split_factor(tiles, std::ceil(std::ldexp(1.0, nK) / 16.0), 16.0, std::ldexp(1.0, nH + nM + nN));
 }
 
-// rows kernel: 128 rows of the large operand per CTA, K staged 32 at a time;
-// short K (<= 32) runs unsplit with the row in registers.
-inline int rows_splits(int nH, int nM, int nN, int nK) {
-  if (nK <= 5) return 1;
-  int big = std::max(nM, nN);
-  double tiles = std::ldexp(1.0, nH) * std::ceil(std::ldexp(1.0, big) / 128.0);
-  return split_factor(tiles, std::ceil(std::ldexp(1.0, nK) / 32.0), 8.0, std::ldexp(1.0, nH + nM + nN));
+// Long-K kernel with a small side of at most 32 rows (kdot.cu): its tile holds
+// every M index, 2^tn N values (16, 32 beside 16 or more rows) and as many K
+// values as one of two 48 KB buffers takes beside them.
+constexpr int kKdotTileElems = 6144;
+inline bool use_kdot(int nM, int nN, int nK) { return (nM < nN ? nM : nN) <= 5 && nK >= 6; }
+inline void kdot_tile(int nM, int nN, int nK, int* tn, int* tk) {
+  *tn = std::min(nN, nM >= 4 ? 5 : 4);
+  *tk = 6;
+  while (*tk < nK && *tk < 11 && (((1 << nM) + (1 << *tn)) << (*tk + 1)) <= kKdotTileElems) ++*tk;
 }
-
-// dot kernel: one CTA per (split, batch entry); each split keeps >= 2048 K elements.
-inline int dot_splits(int nH, int nM, int nN, int nK) {
-  return split_factor(std::ldexp(1.0, nH), std::ldexp(1.0, nK) / 512.0, 4.0, std::ldexp(1.0, nH + nM + nN));
+// K tiles are shared out over CTAs until two of them run on every SM.
+inline int kdot_splits(int nH, int nM, int nN, int nK) {
+  int tn, tk;
+  kdot_tile(nM, nN, nK, &tn, &tk);
+  const double units = std::ldexp(1.0, nH + nN - tn), tiles = std::ldexp(1.0, nK - tk);
+  const double cap = kPartialCapElems / std::ldexp(1.0, nH + nM + nN);
+  return int(std::max(1.0, std::min({std::floor(kSplitTargetCtas / units), tiles, cap})));
 }
 
 // bf16: 64 complex elements per 128-byte K block of A'; tf32: 16.
