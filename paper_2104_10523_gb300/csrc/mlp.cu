@@ -126,21 +126,305 @@ __global__ void colsum_kernel(const float* X, int R, int Cn, int ld, float* out,
   }
 }
 
+// BF16 copy of a weight matrix entry of the flat parameter vector (W1 b1 W2 b2
+// W3 b3); biases have none.
+struct Bf16Copies {
+  size_t w1_end, w2, w2_end, w3, w3_end;
+  __nv_bfloat16 *W1, *W2, *W3;
+  __device__ __forceinline__ void set(size_t i, float v) const {
+    const __nv_bfloat16 b = __float2bfloat16_rn(v);
+    if (i < w1_end) W1[i] = b;
+    else if (i >= w2 && i < w2_end) W2[i - w2] = b;
+    else if (i >= w3 && i < w3_end) W3[i - w3] = b;
+  }
+};
+
+__global__ void to_bf16_kernel(const float* p, size_t n, Bf16Copies c) {
+  for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
+    c.set(i, p[i]);
+}
+
+// Adam update of the FP32 parameters, their BF16 copies refreshed with it.
 __global__ void adam_kernel(float* p, const float* g, float* m, float* v, size_t n, float lr, float b1, float b2,
-                            float eps, float c1, float c2) {
+                            float eps, float c1, float c2, Bf16Copies c) {
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    p[i] = pi;
+    c.set(i, pi);
   }
 }
 
-__global__ void to_bf16_kernel(const float* src, __nv_bfloat16* dst, size_t n) {
-  for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
-    dst[i] = __float2bfloat16_rn(src[i]);
+// ---------------------------------------------------------------- fused rows
+// Everything of a training pass that is local to a row: z1, a1, z2, a2, y and,
+// with BACK, dy, dz2, dz1.  A CTA takes MR_ROWS rows and keeps W2 (BF16, at most
+// 256 x 256) in shared memory, where the forward pass reads its columns and the
+// backward pass its rows; a thread owns a hidden unit for all rows of the CTA.
+// The three layers and their gradients were ten launches of 64 x 64-tiled GEMMs
+// and elementwise passes, each too small to fill the chip: 1024 rows of the
+// 16-256-256-1 model took 466 us a call, now bound by the copies of the call.
+constexpr int MR_ROWS = 8, MR_THREADS = 256;
+
+struct MlpRows {
+  int B, d_in, h;
+  const float *x, *t, *b1, *b2, *b3;
+  const __nv_bfloat16 *W1, *W2, *W3;
+  float *a1, *a2, *y, *dy, *sq, *dz1, *dz2;
+};
+
+__host__ __device__ inline int mr_pitch(int h) { return h + 8; }  // BF16 values a W2 row takes: 16-byte phases spread
+
+__host__ __device__ inline size_t mr_smem(int d_in, int h) {
+  return size_t(h) * mr_pitch(h) * 2 + sizeof(float) * MR_ROWS * (size_t(d_in) + 2 * h + MR_THREADS / 32 + 2);
+}
+
+__device__ __forceinline__ void fma_rows(float (&acc)[MR_ROWS], const float* v, float w) {
+  const float4 p = *reinterpret_cast<const float4*>(v), q = *reinterpret_cast<const float4*>(v + 4);
+  acc[0] = fmaf(p.x, w, acc[0]);
+  acc[1] = fmaf(p.y, w, acc[1]);
+  acc[2] = fmaf(p.z, w, acc[2]);
+  acc[3] = fmaf(p.w, w, acc[3]);
+  acc[4] = fmaf(q.x, w, acc[4]);
+  acc[5] = fmaf(q.y, w, acc[5]);
+  acc[6] = fmaf(q.z, w, acc[6]);
+  acc[7] = fmaf(q.w, w, acc[7]);
+}
+
+template <bool BACK>
+__global__ void __launch_bounds__(MR_THREADS) mlp_rows_kernel(const __grid_constant__ MlpRows P) {
+  extern __shared__ __align__(16) unsigned char mr_raw[];
+  const int h = P.h, d_in = P.d_in, pitch = mr_pitch(h);
+  __nv_bfloat16* w2 = reinterpret_cast<__nv_bfloat16*>(mr_raw);     // [h][pitch]
+  float* a1s = reinterpret_cast<float*>(w2 + size_t(h) * pitch);    // [h][MR_ROWS]
+  float* dz2s = a1s + h * MR_ROWS;                                  // [h][MR_ROWS]
+  float* xs = dz2s + h * MR_ROWS;                                   // [d_in][MR_ROWS]
+  float* red = xs + d_in * MR_ROWS;                                 // [warps][MR_ROWS]
+  float* dys = red + (MR_THREADS / 32) * MR_ROWS;                   // [MR_ROWS]
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int r0 = blockIdx.x * MR_ROWS, nr = min(MR_ROWS, P.B - r0);
+  for (int i = t; i < h * (h / 8); i += MR_THREADS) {
+    const int k = i / (h / 8), c8 = i % (h / 8);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(w2 + size_t(k) * pitch + 8 * c8))),
+                 "l"(P.W2 + size_t(k) * h + 8 * c8)
+                 : "memory");
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  for (int i = t; i < MR_ROWS * d_in; i += MR_THREADS) {
+    const int r = i / d_in, d = i % d_in;
+    xs[d * MR_ROWS + r] = r < nr ? P.x[size_t(r0 + r) * d_in + d] : 0.f;
+  }
+  __syncthreads();
+  const bool on = t < h;
+  float acc[MR_ROWS];
+  if (on) {
+    const float b = P.b1[t];
+#pragma unroll
+    for (int r = 0; r < MR_ROWS; ++r) acc[r] = 0.f;
+#pragma unroll 4
+    for (int d = 0; d < d_in; ++d) fma_rows(acc, xs + d * MR_ROWS, __bfloat162float(P.W1[size_t(d) * h + t]));
+#pragma unroll
+    for (int r = 0; r < MR_ROWS; ++r) {
+      const float v = fmaxf(acc[r] + b, 0.f);
+      a1s[t * MR_ROWS + r] = v;
+      if (BACK && r < nr) P.a1[size_t(r0 + r) * h + t] = v;
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  float a2[MR_ROWS], yp[MR_ROWS];
+  const float w3 = on ? __bfloat162float(P.W3[t]) : 0.f;
+#pragma unroll
+  for (int r = 0; r < MR_ROWS; ++r) acc[r] = a2[r] = yp[r] = 0.f;
+  if (on) {
+    const float b = P.b2[t];
+#pragma unroll 8
+    for (int k = 0; k < h; ++k) fma_rows(acc, a1s + k * MR_ROWS, __bfloat162float(w2[size_t(k) * pitch + t]));
+#pragma unroll
+    for (int r = 0; r < MR_ROWS; ++r) {
+      a2[r] = fmaxf(acc[r] + b, 0.f);
+      yp[r] = a2[r] * w3;
+      if (BACK && r < nr) P.a2[size_t(r0 + r) * h + t] = a2[r];
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < MR_ROWS; ++r) {
+    for (int d = 16; d; d >>= 1) yp[r] += __shfl_xor_sync(0xffffffffu, yp[r], d);
+    if (lane == 0) red[warp * MR_ROWS + r] = yp[r];
+  }
+  __syncthreads();
+  if (t < MR_ROWS) {
+    float y = 0.f;
+    for (int w = 0; w < MR_THREADS / 32; ++w) y += red[w * MR_ROWS + t];
+    y += P.b3[0];
+    float dy = 0.f;
+    if (t < nr) {
+      P.y[r0 + t] = y;
+      if (BACK) {
+        const float e = y - P.t[r0 + t];
+        dy = 2.f * e / float(P.B);
+        P.dy[r0 + t] = dy;
+        P.sq[r0 + t] = e * e;
+      }
+    }
+    dys[t] = dy;
+  }
+  if (!BACK) return;
+  __syncthreads();
+  if (on) {
+#pragma unroll
+    for (int r = 0; r < MR_ROWS; ++r) {
+      const float g = a2[r] > 0.f ? dys[r] * w3 : 0.f;
+      dz2s[t * MR_ROWS + r] = g;
+      if (r < nr) P.dz2[size_t(r0 + r) * h + t] = g;
+    }
+  }
+  __syncthreads();
+  if (on) {
+#pragma unroll
+    for (int r = 0; r < MR_ROWS; ++r) acc[r] = 0.f;
+    for (int c = 0; c < h; c += 8) {
+      const uint4 w = *reinterpret_cast<const uint4*>(w2 + size_t(t) * pitch + c);
+      const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        fma_rows(acc, dz2s + (c + 2 * j) * MR_ROWS, __uint_as_float(u[j] << 16));
+        fma_rows(acc, dz2s + (c + 2 * j + 1) * MR_ROWS, __uint_as_float(u[j] & 0xffff0000u));
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < MR_ROWS; ++r)
+      if (r < nr) P.dz1[size_t(r0 + r) * h + t] = a1s[t * MR_ROWS + r] > 0.f ? acc[r] : 0.f;
+  }
+}
+
+// Parameter gradients as partial sums over `rows` rows each (blockIdx.y):
+// 64 x 64 tiles of W2 = a1^T dz2 and W1 = x^T dz1 (both operands are stored with
+// the summed row index slowest, so a stage of 16 rows is two coalesced copies),
+// then the column sums of W3, b2, b1 and the sums of b3 and the loss.  One CTA
+// per tile over all rows would fill 20 of 152 SMs; the partials are added in
+// order by mlp_reduce_kernel.
+constexpr int MW_T = 64, MW_K = 16;
+
+struct MlpGrads {
+  int B, d_in, h, rows;
+  const float *x, *a1, *a2, *dy, *sq, *dz1, *dz2;
+  float* part;  // [splits][n_params + 1]; the last entry is the sum of squared errors
+  size_t stride, w1, b1, w2, b2, w3, b3;
+};
+
+__global__ void __launch_bounds__(256) mlp_grads_kernel(const __grid_constant__ MlpGrads P) {
+  __shared__ float As[MW_K][MW_T], Bs[MW_K][MW_T];
+  const int tid = threadIdx.x, h = P.h;
+  const int r0 = blockIdx.y * P.rows, r1 = min(P.B, r0 + P.rows);
+  float* part = P.part + blockIdx.y * P.stride;
+  const int tn = (h + MW_T - 1) / MW_T, t2 = tn * tn, t1 = ((P.d_in + MW_T - 1) / MW_T) * tn;
+  int role = blockIdx.x;
+  if (role >= t2 + t1) {
+    role -= t2 + t1;
+    if (role == 0) {  // b3 and the loss
+      if (tid < 64) {
+        const float* v = tid < 32 ? P.dy : P.sq;
+        float s = 0.f;
+        for (int r = r0 + (tid & 31); r < r1; r += 32) s += v[r];
+        for (int d = 16; d; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        if ((tid & 31) == 0) part[tid < 32 ? P.b3 : P.stride - 1] = s;
+      }
+      return;
+    }
+    const int c = (role - 1) * 64 + (tid & 63), g = tid >> 6;  // four row groups per column
+    float s3 = 0.f, s2 = 0.f, s1 = 0.f;
+    if (c < h) {
+#pragma unroll 4
+      for (int r = r0 + g; r < r1; r += 4) {
+        s3 = fmaf(P.a2[size_t(r) * h + c], P.dy[r], s3);
+        s2 += P.dz2[size_t(r) * h + c];
+        s1 += P.dz1[size_t(r) * h + c];
+      }
+    }
+    float* sh = &As[0][0];  // [3][4][64]
+    sh[(0 + g) * 64 + (tid & 63)] = s3;
+    sh[(4 + g) * 64 + (tid & 63)] = s2;
+    sh[(8 + g) * 64 + (tid & 63)] = s1;
+    __syncthreads();
+    if (tid < 192) {
+      const int q = tid >> 6, col = (role - 1) * 64 + (tid & 63);
+      if (col < h) {
+        float s = 0.f;
+        for (int j = 0; j < 4; ++j) s += sh[(4 * q + j) * 64 + (tid & 63)];
+        part[(q == 0 ? P.w3 : q == 1 ? P.b2 : P.b1) + col] = s;
+      }
+    }
+    return;
+  }
+  const bool second = role < t2;
+  if (!second) role -= t2;
+  const float* A = second ? P.a1 : P.x;
+  const float* Bm = second ? P.dz2 : P.dz1;
+  const int M = second ? h : P.d_in;
+  const int m0 = (role / tn) * MW_T, n0 = (role % tn) * MW_T;
+  const int tx = tid & 15, ty = tid >> 4, lr = tid >> 6, lc = tid & 63;
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  float pa[4], pb[4];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const int r = k0 + lr + 4 * l;
+      pa[l] = r < r1 && m0 + lc < M ? A[size_t(r) * M + m0 + lc] : 0.f;
+      pb[l] = r < r1 && n0 + lc < h ? Bm[size_t(r) * h + n0 + lc] : 0.f;
+    }
+  };
+  fetch(r0);
+  for (int k0 = r0; k0 < r1; k0 += MW_K) {
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      As[lr + 4 * l][lc] = pa[l];
+      Bs[lr + 4 * l][lc] = pb[l];
+    }
+    __syncthreads();
+    if (k0 + MW_K < r1) fetch(k0 + MW_K);
+#pragma unroll
+    for (int kk = 0; kk < MW_K; ++kk) {
+      float a[4], b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+  const size_t off = second ? P.w2 : P.w1;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int m = m0 + ty + 16 * i, n = n0 + tx + 16 * j;
+      if (m < M && n < h) part[off + size_t(m) * h + n] = acc[i][j];
+    }
+}
+
+// grads = partials added in split order; the last entry becomes the mean loss.
+__global__ void mlp_reduce_kernel(const float* __restrict__ part, int splits, size_t stride, float* grads, float* loss,
+                                  float inv_b) {
+  const size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x;
+  if (i >= stride) return;
+  float s = 0.f;
+#pragma unroll 8
+  for (int k = 0; k < splits; ++k) s += part[size_t(k) * stride + i];
+  if (i + 1 < stride) grads[i] = s;
+  else *loss = s * inv_b;
 }
 
 unsigned nblk(size_t n) { return unsigned(std::max<size_t>(1, std::min<size_t>((n + 255) / 256, 2048))); }
@@ -148,6 +432,9 @@ unsigned nblk(size_t n) { return unsigned(std::max<size_t>(1, std::min<size_t>((
 }  // namespace
 
 // ---------------------------------------------------------------- model
+// partial gradients of a pass: at least 64 rows each, at most this many
+constexpr int kGradSplits = 16;
+
 size_t CostModel::n_params() const { return size_t(d_in) * h + h + size_t(h) * h + h + h + 1; }
 
 void CostModel::layout() {
@@ -178,6 +465,7 @@ void CostModel::layout() {
   o_dz1 = take(4 * B * h);
   o_dz2 = take(4 * B * h);
   o_loss = take(8);
+  o_part = take(fused() ? 4 * (P + 1) * kGradSplits : 0);
   ws_bytes = off;
 }
 
@@ -197,21 +485,101 @@ static void param_offsets(const CostModel& m, size_t* w1, size_t* b1, size_t* w2
     if (_e != cudaSuccess) return cuda_fail(_e, #call); \
   } while (0)
 
+static Bf16Copies bf16_copies(const CostModel& m) {
+  char* ws = static_cast<char*>(m.ws);
+  size_t w1, b1, w2, b2, w3, b3;
+  param_offsets(m, &w1, &b1, &w2, &b2, &w3, &b3);
+  Bf16Copies c;
+  c.w1_end = b1;
+  c.w2 = w2;
+  c.w2_end = b2;
+  c.w3 = w3;
+  c.w3_end = b3;
+  c.W1 = reinterpret_cast<__nv_bfloat16*>(ws + m.o_w1b);
+  c.W2 = reinterpret_cast<__nv_bfloat16*>(ws + m.o_w2b);
+  c.W3 = reinterpret_cast<__nv_bfloat16*>(ws + m.o_w3b);
+  return c;
+}
+
 static tnq_status refresh_bf16(Ctx* ctx, CostModel* m) {
+  const size_t P = m->n_params();
+  to_bf16_kernel<<<nblk(P), 256, 0, ctx->stream>>>(
+      reinterpret_cast<const float*>(static_cast<char*>(m->ws) + m->o_params), P, bf16_copies(*m));
+  MLP_CUDA(cudaGetLastError());
+  ctx->launches++;
+  return TNQ_OK;
+}
+
+// The fused row kernel on B rows already in the x (and, with `back`, t) region:
+// leaves y, or what the parameter gradients need as well.
+static tnq_status rows_pass(Ctx* ctx, CostModel* m, int B, bool back) {
   char* ws = static_cast<char*>(m->ws);
   size_t w1, b1, w2, b2, w3, b3;
   param_offsets(*m, &w1, &b1, &w2, &b2, &w3, &b3);
-  const float* P = reinterpret_cast<const float*>(ws + m->o_params);
-  to_bf16_kernel<<<nblk(size_t(m->d_in) * m->h), 256, 0, ctx->stream>>>(P + w1, reinterpret_cast<__nv_bfloat16*>(ws + m->o_w1b), size_t(m->d_in) * m->h);
-  to_bf16_kernel<<<nblk(size_t(m->h) * m->h), 256, 0, ctx->stream>>>(P + w2, reinterpret_cast<__nv_bfloat16*>(ws + m->o_w2b), size_t(m->h) * m->h);
-  to_bf16_kernel<<<nblk(m->h), 256, 0, ctx->stream>>>(P + w3, reinterpret_cast<__nv_bfloat16*>(ws + m->o_w3b), size_t(m->h));
+  auto f = [&](size_t o) { return reinterpret_cast<float*>(ws + o); };
+  const float* P = f(m->o_params);
+  const Bf16Copies c = bf16_copies(*m);
+  MlpRows a;
+  a.B = B;
+  a.d_in = m->d_in;
+  a.h = m->h;
+  a.x = f(m->o_x);
+  a.t = f(m->o_t);
+  a.b1 = P + b1;
+  a.b2 = P + b2;
+  a.b3 = P + b3;
+  a.W1 = c.W1;
+  a.W2 = c.W2;
+  a.W3 = c.W3;
+  a.a1 = f(m->o_a1);
+  a.a2 = f(m->o_a2);
+  a.y = f(m->o_y);
+  a.dy = f(m->o_dy);
+  a.sq = f(m->o_sq);
+  a.dz1 = f(m->o_dz1);
+  a.dz2 = f(m->o_dz2);
+  const size_t smem = mr_smem(m->d_in, m->h);
+  const unsigned grid = unsigned((B + MR_ROWS - 1) / MR_ROWS);
+  auto k = back ? mlp_rows_kernel<true> : mlp_rows_kernel<false>;
+  MLP_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+  k<<<grid, MR_THREADS, smem, ctx->stream>>>(a);
   MLP_CUDA(cudaGetLastError());
-  ctx->launches += 3;
+  ctx->launches++;
+  return TNQ_OK;
+}
+
+static tnq_status grads_pass(Ctx* ctx, CostModel* m, int B) {
+  char* ws = static_cast<char*>(m->ws);
+  auto f = [&](size_t o) { return reinterpret_cast<float*>(ws + o); };
+  MlpGrads a;
+  param_offsets(*m, &a.w1, &a.b1, &a.w2, &a.b2, &a.w3, &a.b3);
+  a.B = B;
+  a.d_in = m->d_in;
+  a.h = m->h;
+  a.rows = std::max(64, (B + kGradSplits - 1) / kGradSplits);
+  a.x = f(m->o_x);
+  a.a1 = f(m->o_a1);
+  a.a2 = f(m->o_a2);
+  a.dy = f(m->o_dy);
+  a.sq = f(m->o_sq);
+  a.dz1 = f(m->o_dz1);
+  a.dz2 = f(m->o_dz2);
+  a.part = f(m->o_part);
+  a.stride = m->n_params() + 1;
+  const int tn = (m->h + MW_T - 1) / MW_T, splits = (B + a.rows - 1) / a.rows;
+  const dim3 grid{unsigned(tn * tn + ((m->d_in + MW_T - 1) / MW_T) * tn + 1 + tn), unsigned(splits), 1u};
+  mlp_grads_kernel<<<grid, 256, 0, ctx->stream>>>(a);
+  mlp_reduce_kernel<<<unsigned((a.stride + 255) / 256), 256, 0, ctx->stream>>>(a.part, splits, a.stride, f(m->o_grads),
+                                                                             f(m->o_loss), 1.f / float(B));
+  MLP_CUDA(cudaGetLastError());
+  ctx->launches += 2;
   return TNQ_OK;
 }
 
 // Forward on B rows already in the x region; leaves y (and z/a for backward).
-static tnq_status forward(Ctx* ctx, CostModel* m, int B) {
+// Wider models than the fused kernel holds run layer by layer.
+static tnq_status forward(Ctx* ctx, CostModel* m, int B, bool back) {
+  if (m->fused()) return rows_pass(ctx, m, B, back);
   char* ws = static_cast<char*>(m->ws);
   size_t w1, b1, w2, b2, w3, b3;
   param_offsets(*m, &w1, &b1, &w2, &b2, &w3, &b3);
@@ -230,6 +598,7 @@ static tnq_status forward(Ctx* ctx, CostModel* m, int B) {
 
 // Backward for B rows with targets in the t region; writes the gradient vector.
 static tnq_status backward(Ctx* ctx, CostModel* m, int B) {
+  if (m->fused()) return grads_pass(ctx, m, B);
   char* ws = static_cast<char*>(m->ws);
   size_t w1, b1, w2, b2, w3, b3;
   param_offsets(*m, &w1, &b1, &w2, &b2, &w3, &b3);
@@ -267,10 +636,10 @@ static tnq_status adam(Ctx* ctx, CostModel* m, float lr) {
   adam_kernel<<<nblk(P), 256, 0, ctx->stream>>>(reinterpret_cast<float*>(ws + m->o_params),
                                                 reinterpret_cast<const float*>(ws + m->o_grads),
                                                 reinterpret_cast<float*>(ws + m->o_m), reinterpret_cast<float*>(ws + m->o_v),
-                                                P, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
+                                                P, lr, 0.9f, 0.999f, 1e-8f, c1, c2, bf16_copies(*m));
   MLP_CUDA(cudaGetLastError());
   ctx->launches++;
-  return refresh_bf16(ctx, m);
+  return TNQ_OK;
 }
 
 tnq_status mlp_bind(Ctx* ctx, CostModel* m, void* ws, size_t bytes) {
@@ -311,7 +680,7 @@ tnq_status mlp_gradients(Ctx* ctx, CostModel* m, const float* X, const float* t,
   char* ws = static_cast<char*>(m->ws);
   MLP_CUDA(cudaMemcpyAsync(ws + m->o_x, X, 4 * size_t(n) * m->d_in, cudaMemcpyHostToDevice, ctx->stream));
   MLP_CUDA(cudaMemcpyAsync(ws + m->o_t, t, 4 * size_t(n), cudaMemcpyHostToDevice, ctx->stream));
-  tnq_status s = forward(ctx, m, int(n));
+  tnq_status s = forward(ctx, m, int(n), true);
   if (s == TNQ_OK) s = backward(ctx, m, int(n));
   if (s != TNQ_OK) return s;
   if (grads)
@@ -344,7 +713,7 @@ tnq_status mlp_train(Ctx* ctx, CostModel* m, const float* X, const float* t, int
       }
       MLP_CUDA(cudaMemcpyAsync(ws + m->o_x, xb.data(), 4 * size_t(B) * m->d_in, cudaMemcpyHostToDevice, ctx->stream));
       MLP_CUDA(cudaMemcpyAsync(ws + m->o_t, tb.data(), 4 * size_t(B), cudaMemcpyHostToDevice, ctx->stream));
-      tnq_status s = forward(ctx, m, B);
+      tnq_status s = forward(ctx, m, B, true);
       if (s == TNQ_OK) s = backward(ctx, m, B);
       if (s == TNQ_OK) s = adam(ctx, m, lr);
       if (s != TNQ_OK) return s;
@@ -367,7 +736,7 @@ tnq_status mlp_predict(Ctx* ctx, CostModel* m, const float* X, int64_t n, float*
     const int B = int(std::min<int64_t>(m->max_batch, n - s0));
     MLP_CUDA(cudaMemcpyAsync(ws + m->o_x, X + s0 * m->d_in, 4 * size_t(B) * m->d_in, cudaMemcpyHostToDevice,
                              ctx->stream));
-    tnq_status s = forward(ctx, m, B);
+    tnq_status s = forward(ctx, m, B, false);
     if (s != TNQ_OK) return s;
     MLP_CUDA(cudaMemcpyAsync(y + s0, ws + m->o_y, 4 * size_t(B), cudaMemcpyDeviceToHost, ctx->stream));
     MLP_CUDA(cudaStreamSynchronize(ctx->stream));

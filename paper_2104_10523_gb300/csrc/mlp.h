@@ -19,7 +19,9 @@ struct CostModel {
   long adam_t = 0;
   // workspace offsets (bytes)
   size_t o_params = 0, o_grads = 0, o_m = 0, o_v = 0, o_w1b = 0, o_w2b = 0, o_w3b = 0, o_x = 0, o_t = 0, o_z1 = 0,
-         o_a1 = 0, o_z2 = 0, o_a2 = 0, o_y = 0, o_dy = 0, o_sq = 0, o_dz1 = 0, o_dz2 = 0, o_loss = 0;
+         o_a1 = 0, o_z2 = 0, o_a2 = 0, o_y = 0, o_dy = 0, o_sq = 0, o_dz1 = 0, o_dz2 = 0, o_loss = 0, o_part = 0;
+  // whether the fused row kernel holds the hidden weights (mlp.cu)
+  bool fused() const { return h <= 256 && h % 8 == 0; }
   size_t n_params() const;
   void layout();
 };
