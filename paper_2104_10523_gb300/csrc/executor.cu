@@ -207,6 +207,12 @@ size_t positions(const std::vector<int>& st, const std::vector<int>& req, const 
 // contracted extent its table holds.
 bool small_step(int nH, int nM, int nN, int nK) { return nH + nM + nN + nK <= 18 && nK <= SMALL_MAX_K; }
 
+// Scratch A bytes kept free before the expanded small operand of a long-K
+// tall-skinny step.
+size_t long_k_reserve(bool perm_a, size_t rank_a) {
+  return perm_a ? ((8 * (size_t(1) << rank_a) + 4095) & ~size_t(4095)) : 0;
+}
+
 // Prepare operands (permute / convert) and run one batched complex GEMM.
 tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_labels, bool perm_a,
                          const void* b_src, const std::vector<int>& b_labels, bool perm_b,
@@ -239,7 +245,7 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   // Long-K tall-skinny steps expand the small operand into scratch A, after the
   // place of its permuted copy (kept free where the operand is read in place,
   // so that which kernel a step takes does not hang on that)
-  const size_t tr_used = perm_a ? ((8 * (size_t(1) << a_req.size()) + 4095) & ~size_t(4095)) : 0;
+  const size_t tr_used = long_k_reserve(perm_a, a_req.size());
   char* tr_scratch = scratch_a + tr_used;
   const size_t tr_avail = scratch_a_bytes > tr_used ? scratch_a_bytes - tr_used : 0;
   const bool tc_rows_ok = choice != 0 && choice != 1 && ctx->precision != TNQ_PREC_FP32 && n_small <= 7 &&
@@ -250,7 +256,14 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   // cores unless a row's arithmetic would bound the CUDA cores: each batch
   // entry would fill its own S' and few tiles.  The plain TF32 mode keeps its
   // operand rounding.
-  const bool batched = tc_rows_ok && choice == -1 && gather_bound(nM, nN, nK) &&
+  //
+  // In a plan the modes whose operands are rounded coarsely (2^-11, or 2^-17 for
+  // the BF16 split) keep the tensor cores there and the order of every sum
+  // (`ordered`): a last-bit difference of an earlier sum moves the rounding of
+  // later operands and grows to the mode's own error within a few steps, so the
+  // choice of kernel would show in the amplitudes (1e-4 in TF32).
+  const bool ordered = !direct && (ctx->precision == TNQ_PREC_TF32 || ctx->precision == TNQ_PREC_BF16X3);
+  const bool batched = tc_rows_ok && choice == -1 && !ordered && gather_bound(nM, nN, nK) &&
                        !tc_rows_shared_ok(1 << n_small, 1 << nK, 1 << nH, ctx->precision);
   const bool tc_rows = tc_rows_ok && !batched;
   const bool round_tf32 = batched && ctx->precision == TNQ_PREC_TF32;
@@ -259,7 +272,11 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   const bool gather = tc_rows || batched || (!use_tc && !use_dot(nM, nN, nK) && gather_bound(nM, nN, nK));
   // Small steps of the CUDA-core path, and of the tall-skinny kernel's where a
   // launch of it (about 10 us) is all latency, run in one launch.
-  const bool small = !use_tc && small_step(nH, nM, nN, nK) && (!tc_rows || (choice == -1 && work <= kSmallTcRows));
+  // `ordered` long-K steps run there too, one lane an output.
+  const bool long_ordered = ordered && !use_tc && !gather && use_kdot(nM, nN, nK) && !use_dot(nM, nN, nK) && part &&
+                            nM + nN + nH <= SMALL_MAX_OUT;
+  const bool small = long_ordered || (!use_tc && small_step(nH, nM, nN, nK) &&
+                                      (!tc_rows || (choice == -1 && !ordered && work <= kSmallTcRows)));
   const bool kdot = !small && !gather && !use_tc && use_kdot(nM, nN, nK) && part;
   signed char pos_c[32];  // positions in C of the output bits [N][M][H]
   for (int j = 0; j < nN + nM + nH && j < 32; ++j) pos_c[j] = (signed char)j;
@@ -302,7 +319,12 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
     s.acc = reinterpret_cast<double2*>(acc);
     s.nk = nK;
     s.n_out = nN + nM + nH;
-    s.log_l = small_lanes_log2(s.n_out, nK);
+    // steps of a step program's size use its lanes, so that a step gives the same
+    // bits inside a program and on its own
+    s.log_l = ordered ? 0
+              : s.n_out <= PROG_MAX_OUT && nH + nM + nN + nK <= PROG_MAX_WORK ? prog_lanes_log2(s.n_out, nK)
+                                                                             : small_lanes_log2(s.n_out, nK);
+    const int splits = long_ordered ? ordered_splits(nH, nM, nN, nK) : 1;
     s.round_tf32 = (tc_rows || batched) && ctx->precision == TNQ_PREC_TF32;
     for (int j = 0; j < nK; ++j) {
       s.ka[j] = pos_a[j];
@@ -320,7 +342,11 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
                           (acc ? 2.0 : 1.0) * std::ldexp(1.0, nH + nM + nN)),
                    0.f};
     int slot = timing_begin(ctx);
-    cudaError_t e = launch_cgemm_small(s, ctx->stream);
+    cudaError_t e = launch_cgemm_small(s, part, splits, ctx->stream);
+    if (e == cudaSuccess && splits > 1) {
+      e = launch_reduce_splits(part, splits, out_elems, C, acc, ctx->sm_count, ctx->stream, true);
+      ctx->launches++;
+    }
     timing_end(ctx, slot, r);
     TNQ_CUDA(e);
     ctx->launches++;
@@ -397,7 +423,7 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
     int slot = timing_begin(ctx);
     TNQ_CUDA(launch_cgemm_simt(op.a0, op.b0, C, acc, part, splits, 1 << nM, 1 << nN, 1 << nK, 1 << nH, ctx->stream));
     if (splits > 1) {
-      TNQ_CUDA(launch_reduce_splits(part, splits, out_elems, C, acc, ctx->sm_count, ctx->stream));
+      TNQ_CUDA(launch_reduce_splits(part, splits, out_elems, C, acc, ctx->sm_count, ctx->stream, ordered));
       ctx->launches++;
     }
     timing_end(ctx, slot, r);
@@ -448,7 +474,7 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   int slot = timing_begin(ctx);
   cudaError_t e = launch_cgemm_tc(g, ctx->sm_count, ctx->stream);
   if (e == cudaSuccess && used > 1) {
-    e = launch_reduce_splits(part, used, out_elems, C, acc, ctx->sm_count, ctx->stream);
+    e = launch_reduce_splits(part, used, out_elems, C, acc, ctx->sm_count, ctx->stream, ordered);
     ctx->launches++;
   }
   timing_end(ctx, slot, r);
@@ -487,18 +513,105 @@ int forced_tc_choice(const Ctx* ctx, const Step& s) {
   return -1;
 }
 
+// Step programs run in the modes that leave the order of a sum free (see
+// run_gemm_step).
+bool programs_allowed(const Ctx* ctx) { return ctx->precision == TNQ_PREC_FP32 || ctx->precision == TNQ_PREC_TF32X3; }
+
+// Records of the plan's step programs for the bound workspace.
+tnq_status upload_programs(Ctx* ctx, Plan* p, char* ws) {
+  if (p->groups.empty()) return TNQ_OK;
+  static const std::vector<int> kNoSlices;
+  std::vector<ProgOp> recs;
+  std::vector<uint2> ktab;
+  recs.reserve(p->prog_records);
+  ktab.reserve(p->prog_k_entries);
+  for (const StepGroup& g : p->groups) {
+    for (size_t l = 0; l + 1 < g.level_begin.size(); ++l) {
+      uint32_t units = 0;
+      for (int q = g.level_begin[l]; q < g.level_begin[l + 1]; ++q) {
+        const Step& s = p->steps[g.steps[q]];
+        const auto &ta = p->tensors[s.a], &tb = p->tensors[s.b];
+        const std::vector<int>& sl = s.sliced_batch ? kNoSlices : p->slice_labels;
+        signed char pa[32], pb[32];
+        positions(ta.labels, s.a_req, kNoSlices, 0, pa);
+        positions(tb.labels, s.b_req, kNoSlices, 0, pb);
+        ProgOp r{};
+        r.a = reinterpret_cast<unsigned long long>(ws + ta.offset);
+        r.b = reinterpret_cast<unsigned long long>(ws + tb.offset);
+        r.acc = s.out == p->root;
+        r.c = reinterpret_cast<unsigned long long>(ws + (r.acc ? p->ws_acc : p->tensors[s.out].offset));
+        r.n_out = short(s.nN + s.nM + s.nH);
+        r.nk = short(s.nK);
+        r.log_l = short(prog_lanes_log2(r.n_out, r.nk));
+        r.warp_begin = units;
+        const int lt = r.n_out + r.log_l;
+        units += lt > 5 ? 1u << (lt - 5) : 1u;
+        for (int j = 0; j < r.n_out; ++j) {
+          const bool is_n = j < s.nN, is_m = !is_n && j < s.nN + s.nM;
+          r.bit[j] = make_uint4(is_n ? 0u : 1u << pa[s.nK + j - s.nN],
+                                is_m ? 0u : 1u << pb[is_n ? s.nK + j : s.nK + j - s.nM], 1u << j, 0u);
+        }
+        for (int j = 0; j < 32; ++j) r.sa[j] = r.sb[j] = -1;
+        for (size_t j = 0; j < sl.size() && j < 32; ++j) {
+          auto at = [&](const std::vector<int>& st, const std::vector<int>& req) {
+            const auto it = std::find(st.begin(), st.end(), sl[j]);
+            const bool kept = std::find(req.begin(), req.end(), sl[j]) != req.end();
+            return kept || it == st.end() ? -1 : int(it - st.begin());
+          };
+          r.sa[j] = (signed char)at(ta.labels, s.a_req);
+          r.sb[j] = (signed char)at(tb.labels, s.b_req);
+        }
+        r.ktab = uint32_t(ktab.size());
+        for (uint32_t k = 0; k < 1u << s.nK; ++k) {
+          uint2 o = make_uint2(0, 0);
+          for (int j = 0; j < s.nK; ++j)
+            if ((k >> j) & 1) {
+              o.x |= 1u << pa[j];
+              o.y |= 1u << pb[j];
+            }
+          ktab.push_back(o);
+        }
+        recs.push_back(r);
+      }
+    }
+  }
+  TNQ_CUDA(cudaMemcpyAsync(ws + p->ws_prog, recs.data(), sizeof(ProgOp) * recs.size(), cudaMemcpyHostToDevice, ctx->stream));
+  TNQ_CUDA(cudaMemcpyAsync(ws + p->ws_prog_k, ktab.data(), 8 * ktab.size(), cudaMemcpyHostToDevice, ctx->stream));
+  TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
+  return TNQ_OK;
+}
+
 // One slice of a batch; slice-invariant steps run only in the batch's first
-// slice (their outputs persist for the batch).
+// slice (their outputs persist for the batch).  Groups of small steps run as
+// one launch each, unless their steps are timed one by one, forced onto the
+// tensor cores or summed in a fixed order.
 tnq_status run_pass(Ctx* ctx, Plan* p, int slice_id, char* ws, bool first) {
   const bool tuned = p->tuned_precision == ctx->precision && p->kernel_choice.size() == p->steps.size();
   const bool forced = ctx->kernel_policy == TNQ_KERNELS_TENSOR_CORES;
-  for (size_t si = 0; si < p->steps.size(); ++si) {
-    if (p->steps[si].fold) continue;  // contracted when the plan was bound
-    if (p->steps[si].once() && !first) continue;
-    ctx->cur_step = (int)si;
-    const int choice = forced ? forced_tc_choice(ctx, p->steps[si]) : tuned ? p->kernel_choice[si] : -1;
-    tnq_status st = run_step(ctx, p, si, slice_id, ws, choice);
-    if (st != TNQ_OK) return st;
+  const bool programs = !forced && !ctx->timing && p->slice_labels.size() <= 32 && programs_allowed(ctx);
+  for (int e : p->exec) {
+    std::vector<int> one;
+    if (e >= 0) one.push_back(e);
+    const std::vector<int>& members = e < 0 ? p->groups[-1 - e].steps : one;
+    const Step& s0 = p->steps[members[0]];
+    if (s0.fold) continue;  // contracted when the plan was bound
+    if (s0.once() && !first) continue;
+    if (e < 0 && programs) {
+      const StepGroup& g = p->groups[-1 - e];
+      ctx->cur_step = -1;
+      TNQ_CUDA(launch_prog(reinterpret_cast<const ProgOp*>(ws + p->ws_prog) + g.rec_begin,
+                           reinterpret_cast<const uint2*>(ws + p->ws_prog_k), g.level_begin.data(),
+                           (int)g.level_begin.size() - 1, (int)g.steps.size(), (int)p->slice_labels.size(), slice_id,
+                           ctx->stream));
+      ctx->launches++;
+      continue;
+    }
+    for (int si : members) {
+      ctx->cur_step = si;
+      const int choice = forced ? forced_tc_choice(ctx, p->steps[si]) : tuned ? p->kernel_choice[si] : -1;
+      tnq_status st = run_step(ctx, p, si, slice_id, ws, choice);
+      if (st != TNQ_OK) return st;
+    }
   }
   ctx->cur_step = -1;
   return TNQ_OK;
@@ -650,6 +763,10 @@ tnq_status exec_bind(Ctx* ctx, Plan* p, void* ws, size_t bytes) {
       TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
     }
   }
+  {
+    tnq_status st = upload_programs(ctx, p, base);
+    if (st != TNQ_OK) return st;
+  }
   p->bound_ws = ws;
   p->bound_bytes = bytes;
   p->folded_precision = -1;
@@ -759,7 +876,13 @@ tnq_status exec_autotune(Ctx* ctx, Plan* p, int reps, int* n_tc, int* n_cuda) {
   ctx->timing = false;
   int ntc = 0, ncc = 0;
   tnq_status result = TNQ_OK;
+  // small steps that run in a step program have one choice
+  std::vector<char> grouped(n, 0);
+  if (programs_allowed(ctx))
+    for (const StepGroup& g : p->groups)
+      for (int si : g.steps) grouped[si] = 1;
   for (size_t si = 0; si < n && result == TNQ_OK; ++si) {
+    if (grouped[si]) continue;
     const Step& s = p->steps[si];
     const bool tc_ok = ctx->precision != TNQ_PREC_FP32 &&
                        tc_gemm_supported(1 << s.nM, 1 << s.nN, 1 << s.nK, ctx->precision) &&

@@ -143,6 +143,15 @@ struct Step {
   bool once() const { return invariant || sliced_batch; }
 };
 
+// Small steps (of one lifetime class) that run as one launch, in levels: a step
+// depends only on earlier levels, on steps executed before and on leaves.
+struct StepGroup {
+  std::vector<int> steps;        // by level
+  std::vector<int> level_begin;  // n_levels + 1 entries into steps
+  int cls = 2;
+  size_t rec_begin = 0;          // first record of the group in the program region
+};
+
 struct TensorSlot {
   std::vector<int> labels;        // effective labels (sliced removed), storage order for outputs
   int rank = 0;
@@ -157,6 +166,9 @@ struct Plan {
   std::vector<char> sliced;       // per label
   std::vector<int> slice_labels;  // bit j of the slice id = value of slice_labels[j]
   std::vector<Step> steps;
+  // execution order: step indices, and -1 - g for step group g
+  std::vector<int> exec;
+  std::vector<StepGroup> groups;
   std::vector<TensorSlot> tensors;
   TreeCost cost;
   double search_ms = 0;
@@ -174,6 +186,8 @@ struct Plan {
   int kept_gates = 0;             // gates of the circuit inside the observable's light cone
   std::vector<int8_t> picks;
   size_t ws_picks = 0;
+  // step programs: records of every group's steps, then their K offset tables
+  size_t ws_prog = 0, ws_prog_k = 0, prog_records = 0, prog_k_entries = 0;
   // workspace layout (bytes)
   // persist: outputs of slice-invariant steps read by slice-dependent steps
   // (kept for the whole batch, outside the reusable arena)

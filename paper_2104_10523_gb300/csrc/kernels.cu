@@ -543,10 +543,10 @@ __global__ void reduce_splits_warp_kernel(const float2* __restrict__ part, int s
 }
 
 cudaError_t launch_reduce_splits(const void* part, int splits, size_t n, void* C, void* acc, int sm_count,
-                                 cudaStream_t st) {
+                                 cudaStream_t st, bool in_order) {
   // a warp each while the warps are few (reading 32 splits of one output is
   // uncoalesced, which a small partial array in L2 does not mind)
-  if (splits >= 16 && n <= 4096) {
+  if (splits >= 16 && n <= 4096 && !in_order) {
     reduce_splits_warp_kernel<<<unsigned((n * 32 + 255) / 256), 256, 0, st>>>(
         reinterpret_cast<const float2*>(part), splits, n, reinterpret_cast<float2*>(C), reinterpret_cast<double2*>(acc));
     return cudaGetLastError();

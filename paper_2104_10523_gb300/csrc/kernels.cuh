@@ -46,8 +46,9 @@ cudaError_t launch_permute(const PermDesc& d, const void* src, void* dst0, void*
 // products go to part[s][h][m][n]; launch_reduce_splits then forms C or acc.
 cudaError_t launch_cgemm_simt(const void* A, const void* B, void* C, void* acc, void* part, int splits, int M,
                               int N, int K, int batch, cudaStream_t st);
+// in_order: the splits of an output are always added one after the other
 cudaError_t launch_reduce_splits(const void* part, int splits, size_t n, void* C, void* acc, int sm_count,
-                                 cudaStream_t st);
+                                 cudaStream_t st, bool in_order = false);
 
 // Long-K step with at most 32 rows on its small side (see kdot.cu).  The tile
 // lists hold its stored bits in increasing position with their place in the
@@ -105,7 +106,8 @@ cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const SmallDesc& sd, co
 // an output index (2^n_out of them) sits at stored position pa[j] of A, pb[j]
 // of B (-1: not an index of that operand) and pc[j] of C; bit j of the
 // contracted index at ka[j], kb[j].  With acc the result is added in FP64.
-constexpr int SMALL_MAX_K = 10;  // log2 of the longest contracted extent
+constexpr int SMALL_MAX_K = 10;    // log2 of the longest contracted extent taken for latency's sake
+constexpr int SMALL_MAX_OUT = 30;  // log2 of the most output elements
 struct SmallOp {
   const float2* A;   // slice offsets already added
   const float2* B;
@@ -115,10 +117,34 @@ struct SmallOp {
   int log_l;         // log2 of the lanes sharing an output (small_lanes_log2)
   int round_tf32;    // round the operands to TF32 first
   signed char pa[32], pb[32], pc[32];
-  signed char ka[SMALL_MAX_K], kb[SMALL_MAX_K];
+  signed char ka[32], kb[32];
 };
+// A step of a step program: operands and output by byte address, index bits as
+// element offsets.  An output bit's entry holds its offset in A, B and C (0:
+// not an index of that tensor).
+constexpr int PROG_MAX_OUT = 14;   // log2 of the largest output of a program step
+constexpr int PROG_MAX_K = 10;     // log2 of its longest contracted extent
+constexpr int PROG_MAX_WORK = 15;  // log2 of its complex multiply-adds
+constexpr int PROG_MAX_OPS = 160;  // steps per launch (their records sit in shared memory)
+struct ProgOp {
+  unsigned long long a, b, c;      // byte addresses (c of the FP64 accumulator when acc is set)
+  uint32_t warp_begin;             // first warp-sized unit of the step within its level
+  uint32_t ktab;                   // first entry of the step's (A, B) offsets per K value
+  short n_out, nk, log_l;
+  short acc;                       // add in FP64
+  short pad[4];
+  uint4 bit[PROG_MAX_OUT];
+  signed char sa[32], sb[32];      // stored positions of the sliced labels the slice id fixes (-1: none)
+};
+static_assert(sizeof(ProgOp) % 16 == 0, "records are copied 16 bytes at a time");
+// Runs ops[0 .. n_ops) of a program, level by level: level l is ops
+// [levels[l], levels[l + 1]), whose steps depend on earlier levels only.
+cudaError_t launch_prog(const ProgOp* ops, const uint2* ktab, const int* levels, int n_levels, int n_ops, int n_slices,
+                        int slice_id, cudaStream_t st);
+int prog_lanes_log2(int n_out, int nk);
 int small_lanes_log2(int n_out, int nk);
-cudaError_t launch_cgemm_small(const SmallOp& op, cudaStream_t st);
+// splits > 1 (a power of two): FP32 sums of equal K ranges go to part[split][2^n_out].
+cudaError_t launch_cgemm_small(const SmallOp& op, void* part, int splits, cudaStream_t st);
 
 // Projection leaves j < n_proj at leaves_base + j * stride_bytes:
 // P_j[(b << 1) | x] = [bits[b * row_len + tab[j]] == x] for b < n_valid, else 0.

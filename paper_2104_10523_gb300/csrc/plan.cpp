@@ -22,6 +22,7 @@
 #include "internal.h"
 #include "splitk.h"
 #include "gemm_tc.cuh"
+#include "kernels.cuh"
 #include "mlp.h"
 
 namespace tnq {
@@ -30,6 +31,11 @@ namespace {
 
 // Largest slice-batched output (log2 elements, sliced indices included).
 constexpr int kSliceBatchMaxLog2 = 16;
+
+// Steps that may join a step program: sizes at which a launch of their own on
+// the whole chip is still mostly latency.
+constexpr int kProgMaxOut = PROG_MAX_OUT, kProgMaxK = PROG_MAX_K, kProgMaxWork = PROG_MAX_WORK;
+constexpr size_t kProgMaxOps = PROG_MAX_OPS, kProgRecordBytes = sizeof(ProgOp);
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -205,6 +211,81 @@ void layout_steps(Plan* p) {
     if (s.b >= L && out_cls[s.b] < cls(s)) pinned[s.b] = 1;
   }
 
+  // ---- execution order: folded steps, then the once-per-batch ones, then the
+  // per-slice ones.  Within a class the small steps that depend on no larger
+  // step of it go first, as one group; later runs of small steps form groups of
+  // their own.
+  p->exec.clear();
+  p->groups.clear();
+  p->prog_records = p->prog_k_entries = 0;
+  const int n_steps_all = (int)p->steps.size();
+  auto prog_step = [&](const Step& s) {
+    return !s.fold && s.nH + s.nM + s.nN <= kProgMaxOut && s.nK <= kProgMaxK &&
+           s.nH + s.nM + s.nN + s.nK <= kProgMaxWork;
+  };
+  auto add_group = [&](const std::vector<int>& members, int c) {
+    // levels by dependence within the group; groups are cut at the launch's limit
+    for (size_t at = 0; at < members.size();) {
+      const size_t end = std::min(members.size(), at + kProgMaxOps);
+      std::map<int, int> level;  // tensor id -> level of the group step producing it
+      std::vector<std::vector<int>> by;
+      for (size_t i = at; i < end; ++i) {
+        const Step& s = p->steps[members[i]];
+        int l = 0;
+        for (int id : {s.a, s.b}) {
+          auto it = level.find(id);
+          if (it != level.end()) l = std::max(l, it->second + 1);
+        }
+        level[s.out] = l;
+        if ((int)by.size() <= l) by.resize(l + 1);
+        by[l].push_back(members[i]);
+      }
+      if (end - at == 1) {
+        p->exec.push_back(members[at]);
+      } else {
+        StepGroup g;
+        g.cls = c;
+        for (auto& v : by) {
+          g.level_begin.push_back((int)g.steps.size());
+          g.steps.insert(g.steps.end(), v.begin(), v.end());
+        }
+        g.level_begin.push_back((int)g.steps.size());
+        g.rec_begin = p->prog_records;
+        p->prog_records += g.steps.size();
+        for (int si : g.steps) p->prog_k_entries += size_t(1) << p->steps[si].nK;
+        p->exec.push_back(-1 - (int)p->groups.size());
+        p->groups.push_back(g);
+      }
+      at = end;
+    }
+  };
+  for (int c = 0; c < 3; ++c) {
+    std::vector<int> early, rest;
+    std::vector<char> late(p->tensors.size(), 0);  // outputs of this class outside the early group
+    for (int i = 0; i < n_steps_all; ++i) {
+      const Step& s = p->steps[i];
+      if (cls(s) != c) continue;
+      if (prog_step(s) && !late[s.a] && !late[s.b]) {
+        early.push_back(i);
+      } else {
+        late[s.out] = 1;
+        rest.push_back(i);
+      }
+    }
+    add_group(early, c);
+    std::vector<int> run;
+    for (int i : rest) {
+      if (prog_step(p->steps[i])) {
+        run.push_back(i);
+        continue;
+      }
+      add_group(run, c);
+      run.clear();
+      p->exec.push_back(i);
+    }
+    add_group(run, c);
+  }
+
   // ---- workspace: [leaves][arena of intermediates][scratch A][scratch B][acc][misc]
   size_t off = 0;
   for (int i = 0; i < L; ++i) {
@@ -247,10 +328,20 @@ void layout_steps(Plan* p) {
     live.erase(std::remove_if(live.begin(), live.end(), [&](const Blk& bk) { return bk.owner == owner; }),
                live.end());
   };
-  for (auto& s : p->steps) {
-    if (!pinned[s.out]) p->tensors[s.out].offset = arena_base + alloc(size_t(8) << p->tensors[s.out].rank, s.out);
-    if (s.a >= L) release(s.a);
-    if (s.b >= L) release(s.b);
+  // in execution order; a group's steps run concurrently, so all its outputs
+  // are placed before any operand of the group is given back
+  for (int e : p->exec) {
+    std::vector<int> one{e};
+    const std::vector<int>& members = e < 0 ? p->groups[-1 - e].steps : one;
+    for (int i : members) {
+      const Step& s = p->steps[i];
+      if (!pinned[s.out]) p->tensors[s.out].offset = arena_base + alloc(size_t(8) << p->tensors[s.out].rank, s.out);
+    }
+    for (int i : members) {
+      const Step& s = p->steps[i];
+      if (s.a >= L) release(s.a);
+      if (s.b >= L) release(s.b);
+    }
   }
   p->ws_arena = arena_base;
   p->ws_arena_bytes = arena_top;
@@ -272,7 +363,8 @@ void layout_steps(Plan* p) {
   for (auto& s : p->steps) {
     int sp = std::max({simt_splits(s.nH, s.nM, s.nN, s.nK), tc_splits(s.nH, s.nM, s.nN, s.nK, true),
                        tc_splits(s.nH, s.nM, s.nN, s.nK, false)});
-    if (use_kdot(s.nM, s.nN, s.nK)) sp = std::max(sp, kdot_splits(s.nH, s.nM, s.nN, s.nK));
+    if (use_kdot(s.nM, s.nN, s.nK))
+      sp = std::max({sp, kdot_splits(s.nH, s.nM, s.nN, s.nK), ordered_splits(s.nH, s.nM, s.nN, s.nK)});
     if (sp > 1)
       max_part = std::max(max_part, size_t(sp) * 8 * (size_t(1) << (s.nH + s.nM + s.nN)));
   }
@@ -294,6 +386,10 @@ void layout_steps(Plan* p) {
   off = align_up(off + (p->chan_cumq.size() << p->traj_log2), 256);
   p->ws_dedup_w = off;
   off = align_up(off + (p->chan_cumq.empty() ? 0 : size_t(8) << p->traj_log2), 256);
+  p->ws_prog = off;
+  off = align_up(off + kProgRecordBytes * p->prog_records, 256);
+  p->ws_prog_k = off;
+  off = align_up(off + 8 * p->prog_k_entries, 256);
   p->ws_misc = off;
   const size_t per = size_t(1) << p->batch_log2;
   const size_t n_open = p->net.open_qubits.size();

@@ -23,53 +23,65 @@ __device__ __forceinline__ float2 tf32_rna2(float2 v) {
 
 // 2^log_l lanes share an output element (each takes every 2^log_l-th K value;
 // their sums meet by shuffles), so that few outputs with a longer K still fill
-// warps.  Offsets of the K values are tabulated in shared memory.
-__global__ void __launch_bounds__(SM_THREADS) cgemm_small_kernel(const __grid_constant__ SmallOp op) {
-  __shared__ uint2 ktab[1 << SMALL_MAX_K];
+// warps.  Offsets of the K values are tabulated in shared memory, 2^SMALL_TAB_K
+// at a time.  The grid's y cuts the K range into splits whose sums go to part.
+constexpr int SMALL_TAB_K = 10;
+
+__global__ void __launch_bounds__(SM_THREADS) cgemm_small_kernel(const __grid_constant__ SmallOp op,
+                                                                 float2* __restrict__ part) {
+  __shared__ uint2 ktab[1 << SMALL_TAB_K];
   __shared__ uint3 otab[32];
   const int t = threadIdx.x;
-  for (int k = t; k < 1 << op.nk; k += SM_THREADS) {
-    uint32_t a = 0, b = 0;
-    for (int j = 0; j < op.nk; ++j)
-      if ((k >> j) & 1) {
-        a |= 1u << op.ka[j];
-        b |= 1u << op.kb[j];
-      }
-    ktab[k] = make_uint2(a, b);
-  }
+  const uint32_t K = 1u << op.nk, kchunk = K / gridDim.y, kbeg = blockIdx.y * kchunk;
   if (t < op.n_out) {
     auto bit = [](int p) { return p < 0 ? 0u : 1u << p; };
     otab[t] = make_uint3(bit(op.pa[t]), bit(op.pb[t]), bit(op.pc[t]));
   }
-  __syncthreads();
   const uint32_t idx = blockIdx.x * SM_THREADS + t;
   const uint32_t o = idx >> op.log_l, L = 1u << op.log_l;
   const bool live = o < 1u << op.n_out;
   uint32_t oa = 0, ob = 0, oc = 0;
-  for (int j = 0; j < op.n_out; ++j) {
-    const uint3 w = otab[j];
-    if ((o >> j) & 1) {
-      oa |= w.x;
-      ob |= w.y;
-      oc |= w.z;
-    }
-  }
   float re = 0.f, im = 0.f;
-  if (live) {
-    const float2* A = op.A + oa;
-    const float2* B = op.B + ob;
-#pragma unroll 8
-    for (uint32_t k = idx & (L - 1); k < 1u << op.nk; k += L) {
-      const uint2 q = ktab[k];
-      float2 a = __ldg(A + q.x), b = __ldg(B + q.y);
-      if (op.round_tf32) {
-        a = tf32_rna2(a);
-        b = tf32_rna2(b);
+  for (uint32_t k0 = 0; k0 < kchunk; k0 += 1u << SMALL_TAB_K) {
+    const uint32_t kn = min(kchunk - k0, 1u << SMALL_TAB_K);
+    if (k0) __syncthreads();
+    for (uint32_t k = t; k < kn; k += SM_THREADS) {
+      const uint32_t kk = kbeg + k0 + k;
+      uint32_t a = 0, b = 0;
+      for (int j = 0; j < op.nk; ++j)
+        if ((kk >> j) & 1) {
+          a |= 1u << op.ka[j];
+          b |= 1u << op.kb[j];
+        }
+      ktab[k] = make_uint2(a, b);
+    }
+    __syncthreads();
+    if (!k0) {
+      for (int j = 0; j < op.n_out; ++j) {
+        const uint3 w = otab[j];
+        if ((o >> j) & 1) {
+          oa |= w.x;
+          ob |= w.y;
+          oc |= w.z;
+        }
       }
-      re = fmaf(a.x, b.x, re);
-      re = fmaf(-a.y, b.y, re);
-      im = fmaf(a.x, b.y, im);
-      im = fmaf(a.y, b.x, im);
+    }
+    if (live) {
+      const float2* A = op.A + oa;
+      const float2* B = op.B + ob;
+#pragma unroll 8
+      for (uint32_t k = idx & (L - 1); k < kn; k += L) {
+        const uint2 q = ktab[k];
+        float2 a = __ldg(A + q.x), b = __ldg(B + q.y);
+        if (op.round_tf32) {
+          a = tf32_rna2(a);
+          b = tf32_rna2(b);
+        }
+        re = fmaf(a.x, b.x, re);
+        re = fmaf(-a.y, b.y, re);
+        im = fmaf(a.x, b.y, im);
+        im = fmaf(a.y, b.x, im);
+      }
     }
   }
   for (uint32_t d = 1; d < L; d <<= 1) {
@@ -77,7 +89,9 @@ __global__ void __launch_bounds__(SM_THREADS) cgemm_small_kernel(const __grid_co
     im += __shfl_xor_sync(0xffffffffu, im, d);
   }
   if (live && (idx & (L - 1)) == 0) {
-    if (op.acc) {
+    if (part) {
+      part[(size_t(blockIdx.y) << op.n_out) + oc] = make_float2(re, im);
+    } else if (op.acc) {
       double2 v = op.acc[oc];
       v.x += re;
       v.y += im;
@@ -88,18 +102,142 @@ __global__ void __launch_bounds__(SM_THREADS) cgemm_small_kernel(const __grid_co
   }
 }
 
+// ------------------------------------------------------------------ step program
+// A run of small steps in one launch: one cluster of CTAs walks the steps level
+// by level, a cluster barrier between levels (the barrier's release and acquire
+// order the intermediates, which stay in L2).  Each step alone is a launch whose
+// 2 to 3 us are latency; a level costs about one, whatever its number of steps.
+// The records of the steps are copied to shared memory first; a warp finds its
+// step by its place among the level's warp-sized units.
+constexpr int PROG_CTAS = 8, PROG_THREADS = 512, PROG_WARPS = PROG_CTAS * PROG_THREADS / 32;
+
+struct ProgLevels {
+  int n;
+  short begin[PROG_MAX_OPS + 1];
+};
+
+__global__ void __cluster_dims__(PROG_CTAS, 1, 1) __launch_bounds__(PROG_THREADS)
+    prog_kernel(const ProgOp* __restrict__ gops, const uint2* __restrict__ ktab, const __grid_constant__ ProgLevels lv,
+                int n_ops, int n_slices, int slice_id) {
+  extern __shared__ __align__(16) unsigned char prog_raw[];
+  ProgOp* ops = reinterpret_cast<ProgOp*>(prog_raw);
+  const int t = threadIdx.x, lane = t & 31;
+  {
+    const uint4* src = reinterpret_cast<const uint4*>(gops);
+    uint4* dst = reinterpret_cast<uint4*>(prog_raw);
+    for (int i = t; i < n_ops * int(sizeof(ProgOp) / 16); i += PROG_THREADS) dst[i] = __ldg(src + i);
+  }
+  __syncthreads();
+  for (int i = t; i < n_ops; i += PROG_THREADS) {
+    unsigned long long a = 0, b = 0;
+    for (int j = 0; j < n_slices; ++j)
+      if ((slice_id >> j) & 1) {
+        if (ops[i].sa[j] >= 0) a |= 8ull << ops[i].sa[j];
+        if (ops[i].sb[j] >= 0) b |= 8ull << ops[i].sb[j];
+      }
+    ops[i].a += a;
+    ops[i].b += b;
+  }
+  __syncthreads();
+  const uint32_t warp = blockIdx.x * (PROG_THREADS / 32) + (t >> 5);
+  for (int l = 0; l < lv.n; ++l) {
+    const int o0 = lv.begin[l], o1 = lv.begin[l + 1];
+    const ProgOp& last = ops[o1 - 1];
+    const int lt = last.n_out + last.log_l;
+    const uint32_t units = last.warp_begin + (lt > 5 ? 1u << (lt - 5) : 1u);
+    for (uint32_t u = warp; u < units; u += PROG_WARPS) {
+      int at = o0 - 1;  // the last step of the level that begins at or before u
+      for (int q = o0; q < o1; q += 32) {
+        const unsigned m = __ballot_sync(0xffffffffu, q + lane < o1 && ops[q + lane].warp_begin <= u);
+        at += __popc(m);
+      }
+      const ProgOp& op = ops[at];
+      const uint32_t idx = (u - op.warp_begin) * 32 + lane;
+      const uint32_t o = idx >> op.log_l, L = 1u << op.log_l, K = 1u << op.nk;
+      const bool live = o < 1u << op.n_out;
+      uint32_t oa = 0, ob = 0, oc = 0;
+      for (int j = 0; j < op.n_out; ++j) {
+        const uint4 w = op.bit[j];
+        if ((o >> j) & 1) {
+          oa |= w.x;
+          ob |= w.y;
+          oc |= w.z;
+        }
+      }
+      float re = 0.f, im = 0.f;
+      if (live) {
+        const float2* A = reinterpret_cast<const float2*>(op.a) + oa;
+        const float2* B = reinterpret_cast<const float2*>(op.b) + ob;
+        const uint2* kt = ktab + op.ktab;
+#pragma unroll 4
+        for (uint32_t k = idx & (L - 1); k < K; k += L) {
+          const uint2 q = __ldg(kt + k);
+          // plain loads: earlier levels of this launch may have written them
+          const float2 a = A[q.x], b = B[q.y];
+          re = fmaf(a.x, b.x, re);
+          re = fmaf(-a.y, b.y, re);
+          im = fmaf(a.x, b.y, im);
+          im = fmaf(a.y, b.x, im);
+        }
+      }
+      for (uint32_t d = 1; d < L; d <<= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, d);
+        im += __shfl_xor_sync(0xffffffffu, im, d);
+      }
+      if (live && (idx & (L - 1)) == 0) {
+        if (op.acc) {
+          double2* p = reinterpret_cast<double2*>(op.c) + oc;
+          double2 v = *p;
+          v.x += re;
+          v.y += im;
+          *p = v;
+        } else {
+          reinterpret_cast<float2*>(op.c)[oc] = make_float2(re, im);
+        }
+      }
+    }
+    if (l + 1 < lv.n) {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+  }
+}
+
 }  // namespace
+
+int prog_lanes_log2(int n_out, int nk) {
+  // two K values a lane while the step stays within the cluster's threads
+  return std::max(0, std::min({5, nk - 1, 12 - n_out}));
+}
+
+cudaError_t launch_prog(const ProgOp* ops, const uint2* ktab, const int* levels, int n_levels, int n_ops, int n_slices,
+                        int slice_id, cudaStream_t st) {
+  if (n_ops < 1 || n_ops > PROG_MAX_OPS || n_levels < 1 || n_levels > n_ops || n_slices > 32)
+    return cudaErrorInvalidConfiguration;
+  static const cudaError_t ok = cudaFuncSetAttribute(prog_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     int(PROG_MAX_OPS * sizeof(ProgOp)));
+  if (ok != cudaSuccess) return ok;
+  ProgLevels lv;
+  lv.n = n_levels;
+  for (int i = 0; i <= n_levels; ++i) lv.begin[i] = short(levels[i]);
+  prog_kernel<<<PROG_CTAS, PROG_THREADS, size_t(n_ops) * sizeof(ProgOp), st>>>(ops, ktab, lv, n_ops, n_slices,
+                                                                              slice_id);
+  return cudaGetLastError();
+}
 
 int small_lanes_log2(int n_out, int nk) {
   // enough threads to fill the chip (2^16) while lanes have a K value each
   return std::max(0, std::min({5, nk, 16 - n_out}));
 }
 
-cudaError_t launch_cgemm_small(const SmallOp& op, cudaStream_t st) {
-  if (op.n_out < 0 || op.n_out > 24 || op.nk < 0 || op.nk > SMALL_MAX_K || op.log_l < 0 || op.log_l > 5)
+cudaError_t launch_cgemm_small(const SmallOp& op, void* part, int splits, cudaStream_t st) {
+  if (op.n_out < 0 || op.n_out > SMALL_MAX_OUT || op.nk < 0 || op.nk > 31 || op.log_l < 0 || op.log_l > 5 ||
+      splits < 1 || splits > 65535 || (splits & (splits - 1)) || splits > (1 << std::min(op.nk, 16)) ||
+      (splits > 1 && !part))
     return cudaErrorInvalidConfiguration;
   const long long threads = 1ll << (op.n_out + op.log_l);
-  cgemm_small_kernel<<<unsigned((threads + SM_THREADS - 1) / SM_THREADS), SM_THREADS, 0, st>>>(op);
+  const dim3 grid{unsigned((threads + SM_THREADS - 1) / SM_THREADS), unsigned(splits), 1u};
+  cgemm_small_kernel<<<grid, SM_THREADS, 0, st>>>(op, splits > 1 ? reinterpret_cast<float2*>(part) : nullptr);
   return cudaGetLastError();
 }
 

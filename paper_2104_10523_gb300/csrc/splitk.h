@@ -75,6 +75,14 @@ inline int kdot_splits(int nH, int nM, int nN, int nK) {
   return int(std::max(1.0, std::min({std::floor(kSplitTargetCtas / units), tiles, cap})));
 }
 
+// K splits of a long-K step whose sums keep a fixed order (one lane per output,
+// ascending K): at least 256 K values a split.
+inline int ordered_splits(int nH, int nM, int nN, int nK) {
+  if (nK <= 5) return 1;
+  double tiles = std::ldexp(1.0, nH) * std::ceil(std::ldexp(1.0, std::max(nM, nN)) / 128.0);
+  return split_factor(tiles, std::ceil(std::ldexp(1.0, nK) / 32.0), 8.0, std::ldexp(1.0, nH + nM + nN));
+}
+
 // bf16: 64 complex elements per 128-byte K block of A'; tf32: 16.
 inline int tc_splits(int nH, int nM, int nN, int nK, bool bf16) {
   double tiles = std::ldexp(1.0, nH) * std::ceil(std::ldexp(2.0, nM) / 128.0) *
