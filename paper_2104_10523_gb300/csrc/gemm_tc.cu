@@ -46,7 +46,8 @@ constexpr int TC_THREADS = 320;  // warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
 constexpr int TC_BM = 128;            // rows of A' per tile (64 complex rows)
 constexpr int TC_ROW_BYTES = 128;     // one 128B swizzle atom of K per stage
 constexpr int TC_MAX_STAGES = 8;
-constexpr int TC_SMEM_BUDGET = 200 * 1024;
+constexpr int TC_SMEM_BUDGET = 192 * 1024;  // stages
+constexpr int TC_STAGE_OUT = 4096;          // output staging of an epilogue warp: 16 rows of 32 complex values
 constexpr int TC_GROUP_M = 16;         // m-tiles per launch-order group
 
 struct TcParams {
@@ -234,20 +235,87 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int q0 = half * nq_half;
     const int nq = min(nq_all - q0, nq_half);  // groups owned by this warp (0..4)
     const uint32_t lane_addr = uint32_t(quarter * 32) << 16;
-    const int row = quarter * 32 + lane;
-    const bool odd = lane & 1;
+    float* stage_out = reinterpret_cast<float*>(smem + size_t(P.stages) * stage_bytes + size_t(warp - 2) * TC_STAGE_OUT);
     long long chunk = 0;
     bool ok = true;
     for (long long t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
       int mt, nt, split, h, kb0, nkb;
       decode(t, &mt, &nt, &split, &h, &kb0, &nkb);
       const int nchunks = (nkb + P.chunk_kb - 1) / P.chunk_kb;
-      const int grow = mt * TC_BM + row;  // row of A' within the batch
-      const int m = grow >> 1;
-      const size_t cbase = (size_t(h) * P.M + m) * size_t(P.N);
-      float acc[128];
+      const int mb = mt * (TC_BM / 2) + quarter * 16;  // the warp's first complex row
+      const int rows = min(16, P.M - mb);
+      const int n00 = nt * P.BN + q0 * 32 + lane;
+      const size_t o00 = (size_t(h) * P.M + mb) * size_t(P.N) + n00;
+      float2* out = P.part ? P.part + size_t(split) * P.batch * P.M * P.N : P.C;
+      // Column group q of the tile: a lane holds 32 reals of one row of A' (even
+      // lanes Re, odd lanes Im of a complex row); written as they are, a store
+      // instruction would touch 32 lines (256 store cycles a group; the tile's
+      // share of the memory rate is about 200).  The warp's 16 complex rows x 32
+      // values go through shared memory (XOR-swizzled: neither side has bank
+      // conflicts) and out as 256-byte row pieces.
+      auto put = [&](int q, const float (&x)[32]) {
+        const int r = lane >> 1;
+        __syncwarp();
 #pragma unroll
-      for (int j = 0; j < 128; ++j) acc[j] = 0.f;
+        for (int j = 0; j < 32; ++j) stage_out[2 * (r * 32 + (j ^ r)) + (lane & 1)] = x[j];
+        __syncwarp();
+        if (n00 + q * 32 >= P.N) return;
+        const float2* st = reinterpret_cast<const float2*>(stage_out);
+        const size_t o = o00 + q * 32;
+        if (P.acc && !P.part) {
+          for (int i = 0; i < rows; ++i) {
+            const float2 v = st[i * 32 + (lane ^ i)];
+            double2 tt = P.acc[o + size_t(i) * P.N];
+            tt.x += double(v.x);
+            tt.y += double(v.y);
+            P.acc[o + size_t(i) * P.N] = tt;
+          }
+        } else if (rows == 16) {
+          float2* dst = out + o;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            *dst = st[i * 32 + (lane ^ i)];
+            dst += P.N;
+          }
+        } else {
+          for (int i = 0; i < rows; ++i) out[o + size_t(i) * P.N] = st[i * 32 + (lane ^ i)];
+        }
+      };
+      auto drained = [&](int b) {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[b])) : "memory");
+      };
+      const uint32_t tcol = tmem + lane_addr + uint32_t(q0 * 32);
+      if (nchunks == 1) {
+        // one chunk (short K): from tensor memory straight to the output
+        const int b = int(chunk & 1);
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_full[b]), uint32_t(chunk >> 1) & 1));
+        if (!ok) {
+          if (lane == 0) atomicOr(P.err, 1);
+          break;
+        }
+        ++chunk;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        for (int q = 0; q < nq; ++q) {
+          uint32_t v[32];
+          TC_LD32(tcol + uint32_t(b) * buf_cols + uint32_t(q * 32), v);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          TC_PIN32(v);
+          if (q + 1 == nq) drained(b);
+          float x[32];
+#pragma unroll
+          for (int j = 0; j < 32; ++j) x[j] = __uint_as_float(v[j]);
+          put(q, x);
+        }
+        if (nq <= 0) drained(b);
+        continue;
+      }
+      float acc[4][32];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[q][j] = 0.f;
       for (int c = 0; c < nchunks; ++c, ++chunk) {
         const int b = int(chunk & 1);
         ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_full[b]), uint32_t(chunk >> 1) & 1));
@@ -256,60 +324,26 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           if (q < nq) {
-            uint32_t v[32];
-            TC_LD32(tmem + lane_addr + uint32_t(b) * buf_cols + uint32_t((q0 + q) * 32), v);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int j = 0; j < 32; ++j) acc[q * 32 + j] += __uint_as_float(v[j]);
+            for (int hq = 0; hq < 2; ++hq) {
+              uint32_t v[16];
+              TC_LD16(tcol + uint32_t(b) * buf_cols + uint32_t(q * 32 + 16 * hq), v);
+              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+              TC_PIN16(v);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) acc[q][16 * hq + j] += __uint_as_float(v[j]);
+            }
           }
         }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[b])) : "memory");
+        drained(b);
       }
       if (!ok) {
         if (lane == 0) atomicOr(P.err, 1);
         break;
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (q >= nq) break;
-        float re[16], im[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float mine_lo = acc[q * 32 + j], mine_hi = acc[q * 32 + 16 + j];
-          const float other = __shfl_xor_sync(0xffffffffu, odd ? mine_lo : mine_hi, 1);
-          // even lane (re row) keeps columns 0..15, odd lane (im row) keeps 16..31
-          re[j] = odd ? other : mine_lo;
-          im[j] = odd ? mine_hi : other;
-        }
-        if (m < P.M) {
-          const int n0 = nt * P.BN + (q0 + q) * 32 + (odd ? 16 : 0);
-          if (P.part) {
-            float2* dst = P.part + size_t(split) * P.batch * P.M * P.N + cbase;
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (n0 + j < P.N) dst[n0 + j] = make_float2(re[j], im[j]);
-          } else if (P.acc) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (n0 + j < P.N) {
-                double2 tt = P.acc[cbase + n0 + j];
-                tt.x += double(re[j]);
-                tt.y += double(im[j]);
-                P.acc[cbase + n0 + j] = tt;
-              }
-          } else if (n0 + 16 <= P.N) {
-            float4* dst = reinterpret_cast<float4*>(P.C + cbase + n0);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) dst[j] = make_float4(re[2 * j], im[2 * j], re[2 * j + 1], im[2 * j + 1]);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (n0 + j < P.N) P.C[cbase + n0 + j] = make_float2(re[j], im[j]);
-          }
-        }
-      }
+      for (int q = 0; q < 4; ++q)
+        if (q < nq) put(q, acc[q]);
     }
   }
   __syncthreads();
@@ -367,7 +401,8 @@ cudaError_t tc_gemm_prepare() {
   std::call_once(once, [] {
     result = encode_fn() ? cudaSuccess : cudaErrorNotSupported;
     if (result == cudaSuccess)
-      result = cudaFuncSetAttribute(cgemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BUDGET + 1024);
+      result = cudaFuncSetAttribute(cgemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    TC_SMEM_BUDGET + 8 * TC_STAGE_OUT + 1024);
     if (result == cudaSuccess) result = tc_rows_prepare();
   });
   return result;
@@ -430,7 +465,7 @@ cudaError_t launch_cgemm_tc(const TcGemmArgs& g, int sm_count, cudaStream_t st) 
     ma_lo = ma_hi;
     mb_lo = mb_hi;
   }
-  const int smem = int(P.stages * stage_bytes) + 1024;
+  const int smem = int(P.stages * stage_bytes) + 8 * TC_STAGE_OUT + 1024;
   cudaError_t pe = tc_gemm_prepare();
   if (pe != cudaSuccess) return pe;
   // Short-K tiles: persistent CTAs (one per SM) loop over their tiles so the
