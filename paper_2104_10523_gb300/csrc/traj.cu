@@ -24,84 +24,109 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 }
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 
-__global__ void traj_leaf_kernel(const TrajLeafDesc* __restrict__ leaves, int n_leaves,
-                                 const TrajFactor* __restrict__ factors, const double2* __restrict__ mats,
-                                 const double* __restrict__ cumq, char* ws, uint64_t seed, uint64_t traj_base,
-                                 int traj_log2, const int8_t* __restrict__ picks, int n_sel, int64_t n_terms) {
-  const long long T = 1ll << traj_log2;
-  const long long total = (long long)n_leaves * T;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int leaf = int(idx / T);
-    const long long tau = idx % T;
-    const TrajLeafDesc L = leaves[leaf];
-    const int ns = L.n_slots, D = 1 << ns;
-    double2 M[16];
-    for (int i = 0; i < 16; ++i) M[i] = make_double2(0.0, 0.0);
-    for (int i = 0; i < D; ++i) M[i * D + i] = make_double2(1.0, 0.0);
+// Index of the operator factor F applies in trajectory (term) tau of the pass.
+__device__ __forceinline__ int pick_of(const TrajFactor& F, long long tau, uint64_t seed, uint64_t traj_base,
+                                       const double* __restrict__ cumq, const int8_t* __restrict__ picks, int n_sel,
+                                       int64_t n_terms) {
+  if (F.channel == 2 || (F.channel == 1 && picks)) {
+    // pick table: per term (observables) or per distinct trajectory (noise)
+    const int64_t term = int64_t(traj_base) + tau;
+    return term < n_terms ? int(picks[term * n_sel + F.chan_index]) : 0;
+  }
+  if (!F.channel) return 0;
+  const double u = draw_uniform(seed, traj_base + uint64_t(tau), uint64_t(F.chan_index));
+  int k = F.n_ops - 1;
+  for (int j = 0; j < F.n_ops; ++j)
+    if (u < cumq[F.cum_off + j]) {
+      k = j;
+      break;
+    }
+  return k;
+}
+
+// A CTA builds one leaf for a block of trajectories.  Most of them pick operator
+// 0 of every channel of the leaf: that product is computed once and copied, and
+// only the others (listed in shared memory) are multiplied up, 16 lanes to a
+// 4x4 product (FP64 runs at a small fraction of the FP32 rate, and a thread
+// holding whole matrices indexes local memory).  256 trajectories of 78 leaves
+// with about 8 factors each took 411 us a pass, one thread per matrix.
+constexpr int TL_THREADS = 256;
+
+__global__ void __launch_bounds__(TL_THREADS) traj_leaf_kernel(
+    const TrajLeafDesc* __restrict__ leaves, const TrajFactor* __restrict__ factors, const double2* __restrict__ mats,
+    const double* __restrict__ cumq, char* ws, uint64_t seed, uint64_t traj_base, int traj_log2,
+    const int8_t* __restrict__ picks, int n_sel, int64_t n_terms) {
+  __shared__ double2 prod[TL_THREADS / 16][16];  // running product of a half-warp
+  __shared__ float2 def[16];                     // product of picks 0, as stored
+  __shared__ unsigned short todo[TL_THREADS];
+  __shared__ int n_todo;
+  const int t = threadIdx.x, hw = t >> 4, e = t & 15;
+  const long long T = 1ll << traj_log2, tau0 = (long long)blockIdx.y * TL_THREADS;
+  const TrajLeafDesc L = leaves[blockIdx.x];
+  const int ns = L.n_slots, D = 1 << ns, rank_op = L.nfree + ns, n_out = 1 << rank_op;
+  if (t == 0) n_todo = 0;
+  __syncthreads();
+  const long long tau = tau0 + t;
+  bool plain = true;
+  if (tau < T)
+    for (int f = 0; f < L.n_factors && plain; ++f)
+      plain = pick_of(factors[L.factor_off + f], tau, seed, traj_base, cumq, picks, n_sel, n_terms) == 0;
+  if (tau < T && !plain) todo[atomicAdd(&n_todo, 1)] = (unsigned short)t;
+  // product for trajectory `tt` (picks 0 when tt < 0) by the 16 lanes of a
+  // half-warp, lane e holding entry e; stored entries (rows x free-input
+  // columns, closed inputs take column entry 0) go to `out`
+  auto build = [&](long long tt, float2* out) {
+    double2(&M)[16] = prod[hw];
+    const unsigned mask = 0xffffu << (t & 16);
+    const bool on = e < D * D;
+    const int r = e / D, c = e % D;
+    M[e] = make_double2(on && r == c ? 1.0 : 0.0, 0.0);
+    __syncwarp(mask);
     for (int f = 0; f < L.n_factors; ++f) {
       const TrajFactor F = factors[L.factor_off + f];
-      int mi = F.mat_off;
-      if (F.channel == 2 || (F.channel == 1 && picks)) {
-        // pick table: per term (observables) or per distinct trajectory (noise)
-        const int64_t term = int64_t(traj_base) + tau;
-        mi += term < n_terms ? int(picks[term * n_sel + F.chan_index]) : 0;
-      } else if (F.channel) {
-        const double u = draw_uniform(seed, traj_base + uint64_t(tau), uint64_t(F.chan_index));
-        int k = F.n_ops - 1;
-        for (int j = 0; j < F.n_ops; ++j)
-          if (u < cumq[F.cum_off + j]) {
-            k = j;
-            break;
+      const int k = tt < 0 ? 0 : pick_of(F, tt, seed, traj_base, cumq, picks, n_sel, n_terms);
+      const double2* U = mats + size_t(F.mat_off + k) * 16;
+      double2 s = make_double2(0.0, 0.0);
+      if (on) {
+        if (ns == 1) {  // 2x2 group, one-qubit op
+          s = cadd(cmul(U[r * 2 + 0], M[0 * 2 + c]), cmul(U[r * 2 + 1], M[1 * 2 + c]));
+        } else if (F.arity == 2) {  // 4x4 op on both slots (indices swapped if listed reversed)
+          const int rr = F.swap ? (((r & 1) << 1) | (r >> 1)) : r;
+          for (int k2 = 0; k2 < 4; ++k2) {
+            const int kk = F.swap ? (((k2 & 1) << 1) | (k2 >> 1)) : k2;
+            s = cadd(s, cmul(U[rr * 4 + kk], M[k2 * 4 + c]));
           }
-        mi += k;
-      }
-      const double2* U = mats + size_t(mi) * 16;
-      double2 R[16];
-      if (ns == 1) {  // 2x2 group, one-qubit op
-        for (int r = 0; r < 2; ++r)
-          for (int c = 0; c < 2; ++c)
-            R[r * 2 + c] = cadd(cmul(U[r * 2 + 0], M[0 * 2 + c]), cmul(U[r * 2 + 1], M[1 * 2 + c]));
-      } else if (F.arity == 2) {  // 4x4 op on both slots (indices swapped if listed reversed)
-        for (int r = 0; r < 4; ++r)
-          for (int c = 0; c < 4; ++c) {
-            double2 s = make_double2(0.0, 0.0);
-            for (int k2 = 0; k2 < 4; ++k2) {
-              const int rr = F.swap ? (((r & 1) << 1) | (r >> 1)) : r;
-              const int kk = F.swap ? (((k2 & 1) << 1) | (k2 >> 1)) : k2;
-              s = cadd(s, cmul(U[rr * 4 + kk], M[k2 * 4 + c]));
-            }
-            R[r * 4 + c] = s;
-          }
-      } else {  // one-qubit op on slot 0 (most significant) or slot 1
-        const int s0 = F.slot_mask == 1 ? 0 : 1;
-        for (int r = 0; r < 4; ++r) {
+        } else {  // one-qubit op on slot 0 (most significant) or slot 1
           const int a = r >> 1, b = r & 1;
-          for (int c = 0; c < 4; ++c) {
-            double2 s;
-            if (s0 == 0) s = cadd(cmul(U[a * 2 + 0], M[(0 << 1 | b) * 4 + c]), cmul(U[a * 2 + 1], M[(1 << 1 | b) * 4 + c]));
-            else s = cadd(cmul(U[b * 2 + 0], M[(a << 1 | 0) * 4 + c]), cmul(U[b * 2 + 1], M[(a << 1 | 1) * 4 + c]));
-            R[r * 4 + c] = s;
-          }
+          if (F.slot_mask == 1)
+            s = cadd(cmul(U[a * 2 + 0], M[b * 4 + c]), cmul(U[a * 2 + 1], M[(2 | b) * 4 + c]));
+          else
+            s = cadd(cmul(U[b * 2 + 0], M[(a << 1) * 4 + c]), cmul(U[b * 2 + 1], M[(a << 1 | 1) * 4 + c]));
         }
       }
-      for (int i = 0; i < D * D; ++i) M[i] = R[i];
+      __syncwarp(mask);
+      if (on) M[e] = s;
+      __syncwarp(mask);
     }
-    // write rows x free-input columns (closed inputs take column entry 0)
-    const int rank_op = L.nfree + ns;
-    float2* out = reinterpret_cast<float2*>(ws + L.out_offset) + (size_t(tau) << rank_op);
-    for (int row = 0; row < D; ++row)
-      for (int cf = 0; cf < (1 << L.nfree); ++cf) {
-        int col = 0, bit = 0;
-        for (int s = ns - 1; s >= 0; --s) {
-          if ((L.in_fixed_mask >> s) & 1) continue;
-          col |= ((cf >> bit) & 1) << (ns - 1 - s);
-          ++bit;
-        }
-        const double2 v = M[row * D + col];
-        out[(row << L.nfree) | cf] = make_float2(float(v.x), float(v.y));
+    if (e < n_out) {
+      const int row = e >> L.nfree, cf = e & ((1 << L.nfree) - 1);
+      int col = 0, bit = 0;
+      for (int s = ns - 1; s >= 0; --s) {
+        if ((L.in_fixed_mask >> s) & 1) continue;
+        col |= ((cf >> bit) & 1) << (ns - 1 - s);
+        ++bit;
       }
-  }
+      const double2 v = M[row * D + col];
+      out[e] = make_float2(float(v.x), float(v.y));
+    }
+    __syncwarp(mask);
+  };
+  if (hw == 0) build(-1, def);
+  __syncthreads();
+  float2* out = reinterpret_cast<float2*>(ws + L.out_offset) + (size_t(tau0) << rank_op);
+  for (int i = hw; i < n_todo; i += TL_THREADS / 16) build(tau0 + todo[i], out + (size_t(todo[i]) << rank_op));
+  if (tau < T && plain)
+    for (int j = 0; j < n_out; ++j) out[(size_t(t) << rank_op) + j] = def[j];
 }
 
 struct Pos {
@@ -116,20 +141,45 @@ __device__ __forceinline__ size_t scatter(long long v, const Pos& P) {
   return r;
 }
 
-__global__ void noisy_accumulate_kernel(const double2* __restrict__ acc, int64_t nb, int64_t nt, Pos bp, Pos tp,
-                                        double* psum, double* p2sum, const double* __restrict__ weights) {
-  for (int64_t b = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; b < nb; b += int64_t(gridDim.x) * blockDim.x) {
+// A CTA per bitstring: its threads share the trajectories out and meet in a
+// fixed tree.  (16 bitstrings of a pass used 16 threads, each a chain of 256
+// dependent sums: 182 us.)
+constexpr int NA_THREADS = 256;
+
+__global__ void __launch_bounds__(NA_THREADS) noisy_accumulate_kernel(const double2* __restrict__ acc, int64_t nb,
+                                                                      int64_t nt, Pos bp, Pos tp, double* psum,
+                                                                      double* p2sum,
+                                                                      const double* __restrict__ weights) {
+  __shared__ double sh[2][NA_THREADS / 32];
+  for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) {
     const size_t base = scatter(b, bp);
     double s = 0.0, s2 = 0.0;
-    for (int64_t t = 0; t < nt; ++t) {
+    for (int64_t t = threadIdx.x; t < nt; t += NA_THREADS) {
       const double2 a = acc[base | scatter(t, tp)];
       const double p = a.x * a.x + a.y * a.y;
       const double w = weights ? weights[t] : 1.0;
       s += w * p;
       s2 += w * p * p;
     }
-    psum[b] += s;
-    p2sum[b] += s2;
+    for (int d = 16; d; d >>= 1) {
+      s += __shfl_xor_sync(0xffffffffu, s, d);
+      s2 += __shfl_xor_sync(0xffffffffu, s2, d);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      sh[0][threadIdx.x >> 5] = s;
+      sh[1][threadIdx.x >> 5] = s2;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double u = 0.0, u2 = 0.0;
+      for (int w = 0; w < NA_THREADS / 32; ++w) {
+        u += sh[0][w];
+        u2 += sh[1][w];
+      }
+      psum[b] += u;
+      p2sum[b] += u2;
+    }
+    __syncthreads();
   }
 }
 
@@ -170,18 +220,19 @@ cudaError_t launch_traj_leaves(const TrajLeafDesc* leaves, int n_leaves, const T
                                uint64_t traj_base, int traj_log2, cudaStream_t st, const int8_t* picks, int n_sel,
                                int64_t n_terms) {
   if (n_leaves == 0) return cudaSuccess;
-  const int64_t total = int64_t(n_leaves) << traj_log2;
-  traj_leaf_kernel<<<blocks_for(total), 256, 0, st>>>(leaves, n_leaves, factors, mats, cumq, ws, seed, traj_base,
-                                                      traj_log2, picks, n_sel, n_terms);
+  const long long blocks = ((1ll << traj_log2) + TL_THREADS - 1) / TL_THREADS;
+  traj_leaf_kernel<<<dim3(unsigned(n_leaves), unsigned(blocks), 1u), TL_THREADS, 0, st>>>(
+      leaves, factors, mats, cumq, ws, seed, traj_base, traj_log2, picks, n_sel, n_terms);
   return cudaGetLastError();
 }
 
 cudaError_t launch_noisy_accumulate(const void* acc, int64_t nb, int64_t nt, const int* bpos, int nbpos,
                                     const int* tpos, int ntpos, double* psum, double* p2sum, cudaStream_t st,
                                     const double* weights) {
-  noisy_accumulate_kernel<<<blocks_for(nb), 256, 0, st>>>(reinterpret_cast<const double2*>(acc), nb, nt,
-                                                          make_pos(bpos, nbpos), make_pos(tpos, ntpos), psum, p2sum,
-                                                          weights);
+  const unsigned grid = unsigned(std::max<int64_t>(1, std::min<int64_t>(nb, 65535)));
+  noisy_accumulate_kernel<<<grid, NA_THREADS, 0, st>>>(reinterpret_cast<const double2*>(acc), nb, nt,
+                                                       make_pos(bpos, nbpos), make_pos(tpos, ntpos), psum, p2sum,
+                                                       weights);
   return cudaGetLastError();
 }
 

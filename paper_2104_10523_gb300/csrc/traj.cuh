@@ -50,8 +50,8 @@ cudaError_t launch_traj_leaves(const TrajLeafDesc* leaves, int n_leaves, const T
                                int n_sel = 0, int64_t n_terms = 0);
 
 // For b < nb: psum[b] += sum_{t < nt} w_t |amp(b, t)|^2, p2sum[b] += sum_t w_t |amp|^4,
-// with amp(b, t) = acc[pdep(b, bpos) | pdep(t, tpos)] (FP64, trajectories in
-// order) and w_t = weights[t] (device; NULL: every weight 1).
+// with amp(b, t) = acc[pdep(b, bpos) | pdep(t, tpos)] (FP64, a fixed
+// tree over the trajectories) and w_t = weights[t] (device; NULL: every weight 1).
 cudaError_t launch_noisy_accumulate(const void* acc, int64_t nb, int64_t nt, const int* bpos, int nbpos,
                                     const int* tpos, int ntpos, double* psum, double* p2sum, cudaStream_t st,
                                     const double* weights = nullptr);
