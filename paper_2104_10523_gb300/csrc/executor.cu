@@ -522,10 +522,9 @@ tnq_status upload_programs(Ctx* ctx, Plan* p, char* ws) {
   if (p->groups.empty()) return TNQ_OK;
   static const std::vector<int> kNoSlices;
   std::vector<ProgOp> recs;
-  std::vector<uint2> ktab;
   recs.reserve(p->prog_records);
-  ktab.reserve(p->prog_k_entries);
-  for (const StepGroup& g : p->groups) {
+  for (StepGroup& g : p->groups) {
+    g.max_units = 0;
     for (size_t l = 0; l + 1 < g.level_begin.size(); ++l) {
       uint32_t units = 0;
       for (int q = g.level_begin[l]; q < g.level_begin[l + 1]; ++q) {
@@ -561,22 +560,13 @@ tnq_status upload_programs(Ctx* ctx, Plan* p, char* ws) {
           r.sa[j] = (signed char)at(ta.labels, s.a_req);
           r.sb[j] = (signed char)at(tb.labels, s.b_req);
         }
-        r.ktab = uint32_t(ktab.size());
-        for (uint32_t k = 0; k < 1u << s.nK; ++k) {
-          uint2 o = make_uint2(0, 0);
-          for (int j = 0; j < s.nK; ++j)
-            if ((k >> j) & 1) {
-              o.x |= 1u << pa[j];
-              o.y |= 1u << pb[j];
-            }
-          ktab.push_back(o);
-        }
+        for (int j = 0; j < s.nK; ++j) r.kbit[j] = make_uint2(1u << pa[j], 1u << pb[j]);
         recs.push_back(r);
       }
+      g.max_units = std::max(g.max_units, int(units));
     }
   }
   TNQ_CUDA(cudaMemcpyAsync(ws + p->ws_prog, recs.data(), sizeof(ProgOp) * recs.size(), cudaMemcpyHostToDevice, ctx->stream));
-  TNQ_CUDA(cudaMemcpyAsync(ws + p->ws_prog_k, ktab.data(), 8 * ktab.size(), cudaMemcpyHostToDevice, ctx->stream));
   TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
   return TNQ_OK;
 }
@@ -600,9 +590,8 @@ tnq_status run_pass(Ctx* ctx, Plan* p, int slice_id, char* ws, bool first) {
       const StepGroup& g = p->groups[-1 - e];
       ctx->cur_step = -1;
       TNQ_CUDA(launch_prog(reinterpret_cast<const ProgOp*>(ws + p->ws_prog) + g.rec_begin,
-                           reinterpret_cast<const uint2*>(ws + p->ws_prog_k), g.level_begin.data(),
-                           (int)g.level_begin.size() - 1, (int)g.steps.size(), (int)p->slice_labels.size(), slice_id,
-                           ctx->stream));
+                           g.level_begin.data(), (int)g.level_begin.size() - 1, (int)g.steps.size(), g.max_units,
+                           (int)p->slice_labels.size(), slice_id, ctx->stream));
       ctx->launches++;
       continue;
     }

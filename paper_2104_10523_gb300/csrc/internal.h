@@ -150,6 +150,7 @@ struct StepGroup {
   std::vector<int> level_begin;  // n_levels + 1 entries into steps
   int cls = 2;
   size_t rec_begin = 0;          // first record of the group in the program region
+  int max_units = 0;             // warp-sized units of its largest level (set when the records are made)
 };
 
 struct TensorSlot {
@@ -186,8 +187,8 @@ struct Plan {
   int kept_gates = 0;             // gates of the circuit inside the observable's light cone
   std::vector<int8_t> picks;
   size_t ws_picks = 0;
-  // step programs: records of every group's steps, then their K offset tables
-  size_t ws_prog = 0, ws_prog_k = 0, prog_records = 0, prog_k_entries = 0;
+  // step programs: records of every group's steps
+  size_t ws_prog = 0, prog_records = 0;
   // workspace layout (bytes)
   // persist: outputs of slice-invariant steps read by slice-dependent steps
   // (kept for the whole batch, outside the reusable arena)

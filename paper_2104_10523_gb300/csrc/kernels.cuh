@@ -129,17 +129,19 @@ constexpr int PROG_MAX_OPS = 160;  // steps per launch (their records sit in sha
 struct ProgOp {
   unsigned long long a, b, c;      // byte addresses (c of the FP64 accumulator when acc is set)
   uint32_t warp_begin;             // first warp-sized unit of the step within its level
-  uint32_t ktab;                   // first entry of the step's (A, B) offsets per K value
+  uint32_t pad0;
   short n_out, nk, log_l;
   short acc;                       // add in FP64
   short pad[4];
   uint4 bit[PROG_MAX_OUT];
+  uint2 kbit[PROG_MAX_K];          // (A, B) offset of a contracted index's bit
   signed char sa[32], sb[32];      // stored positions of the sliced labels the slice id fixes (-1: none)
 };
 static_assert(sizeof(ProgOp) % 16 == 0, "records are copied 16 bytes at a time");
 // Runs ops[0 .. n_ops) of a program, level by level: level l is ops
 // [levels[l], levels[l + 1]), whose steps depend on earlier levels only.
-cudaError_t launch_prog(const ProgOp* ops, const uint2* ktab, const int* levels, int n_levels, int n_ops, int n_slices,
+// max_units: warp-sized units of the largest level.
+cudaError_t launch_prog(const ProgOp* ops, const int* levels, int n_levels, int n_ops, int max_units, int n_slices,
                         int slice_id, cudaStream_t st);
 int prog_lanes_log2(int n_out, int nk);
 int small_lanes_log2(int n_out, int nk);

@@ -217,7 +217,7 @@ void layout_steps(Plan* p) {
   // their own.
   p->exec.clear();
   p->groups.clear();
-  p->prog_records = p->prog_k_entries = 0;
+  p->prog_records = 0;
   const int n_steps_all = (int)p->steps.size();
   auto prog_step = [&](const Step& s) {
     return !s.fold && s.nH + s.nM + s.nN <= kProgMaxOut && s.nK <= kProgMaxK &&
@@ -252,7 +252,6 @@ void layout_steps(Plan* p) {
         g.level_begin.push_back((int)g.steps.size());
         g.rec_begin = p->prog_records;
         p->prog_records += g.steps.size();
-        for (int si : g.steps) p->prog_k_entries += size_t(1) << p->steps[si].nK;
         p->exec.push_back(-1 - (int)p->groups.size());
         p->groups.push_back(g);
       }
@@ -388,8 +387,6 @@ void layout_steps(Plan* p) {
   off = align_up(off + (p->chan_cumq.empty() ? 0 : size_t(8) << p->traj_log2), 256);
   p->ws_prog = off;
   off = align_up(off + kProgRecordBytes * p->prog_records, 256);
-  p->ws_prog_k = off;
-  off = align_up(off + 8 * p->prog_k_entries, 256);
   p->ws_misc = off;
   const size_t per = size_t(1) << p->batch_log2;
   const size_t n_open = p->net.open_qubits.size();

@@ -103,32 +103,36 @@ __global__ void __launch_bounds__(SM_THREADS) cgemm_small_kernel(const __grid_co
 }
 
 // ------------------------------------------------------------------ step program
-// A run of small steps in one launch: one cluster of CTAs walks the steps level
+// A run of small steps in one launch: one cluster (the grid) of CTAs walks the steps level
 // by level, a cluster barrier between levels (the barrier's release and acquire
 // order the intermediates, which stay in L2).  Each step alone is a launch whose
 // 2 to 3 us are latency; a level costs about one, whatever its number of steps.
 // The records of the steps are copied to shared memory first; a warp finds its
 // step by its place among the level's warp-sized units.
-constexpr int PROG_CTAS = 8, PROG_THREADS = 512, PROG_WARPS = PROG_CTAS * PROG_THREADS / 32;
+// The cluster grows with the largest level: one CTA for at most 2^10 outputs (a
+// block barrier is cheaper than a cluster's), eight of 16 warps for at most 2^13,
+// sixteen of 32 warps above (eight where a cluster of sixteen cannot be placed;
+// a level of 2^14 outputs is then one round of the warps).  A 4x5 noisy pass
+// (levels of 2^14) took 132 us with eight of 16 warps, 48 with sixteen of 32.
+constexpr int PROG_CTAS = 16, PROG_CTAS_PORTABLE = 8, PROG_THREADS = 1024;
 
 struct ProgLevels {
   int n;
   short begin[PROG_MAX_OPS + 1];
 };
 
-__global__ void __cluster_dims__(PROG_CTAS, 1, 1) __launch_bounds__(PROG_THREADS)
-    prog_kernel(const ProgOp* __restrict__ gops, const uint2* __restrict__ ktab, const __grid_constant__ ProgLevels lv,
-                int n_ops, int n_slices, int slice_id) {
+__global__ void __launch_bounds__(PROG_THREADS)
+    prog_kernel(const ProgOp* __restrict__ gops, const __grid_constant__ ProgLevels lv, int n_ops, int n_slices, int slice_id) {
   extern __shared__ __align__(16) unsigned char prog_raw[];
   ProgOp* ops = reinterpret_cast<ProgOp*>(prog_raw);
   const int t = threadIdx.x, lane = t & 31;
   {
     const uint4* src = reinterpret_cast<const uint4*>(gops);
     uint4* dst = reinterpret_cast<uint4*>(prog_raw);
-    for (int i = t; i < n_ops * int(sizeof(ProgOp) / 16); i += PROG_THREADS) dst[i] = __ldg(src + i);
+    for (int i = t; i < n_ops * int(sizeof(ProgOp) / 16); i += blockDim.x) dst[i] = __ldg(src + i);
   }
   __syncthreads();
-  for (int i = t; i < n_ops; i += PROG_THREADS) {
+  for (int i = t; i < n_ops; i += blockDim.x) {
     unsigned long long a = 0, b = 0;
     for (int j = 0; j < n_slices; ++j)
       if ((slice_id >> j) & 1) {
@@ -139,13 +143,13 @@ __global__ void __cluster_dims__(PROG_CTAS, 1, 1) __launch_bounds__(PROG_THREADS
     ops[i].b += b;
   }
   __syncthreads();
-  const uint32_t warp = blockIdx.x * (PROG_THREADS / 32) + (t >> 5);
+  const uint32_t per = blockDim.x >> 5, warp = blockIdx.x * per + (t >> 5), warps = gridDim.x * per;
   for (int l = 0; l < lv.n; ++l) {
     const int o0 = lv.begin[l], o1 = lv.begin[l + 1];
     const ProgOp& last = ops[o1 - 1];
     const int lt = last.n_out + last.log_l;
     const uint32_t units = last.warp_begin + (lt > 5 ? 1u << (lt - 5) : 1u);
-    for (uint32_t u = warp; u < units; u += PROG_WARPS) {
+    for (uint32_t u = warp; u < units; u += warps) {
       int at = o0 - 1;  // the last step of the level that begins at or before u
       for (int q = o0; q < o1; q += 32) {
         const unsigned m = __ballot_sync(0xffffffffu, q + lane < o1 && ops[q + lane].warp_begin <= u);
@@ -168,12 +172,18 @@ __global__ void __cluster_dims__(PROG_CTAS, 1, 1) __launch_bounds__(PROG_THREADS
       if (live) {
         const float2* A = reinterpret_cast<const float2*>(op.a) + oa;
         const float2* B = reinterpret_cast<const float2*>(op.b) + ob;
-        const uint2* kt = ktab + op.ktab;
 #pragma unroll 4
         for (uint32_t k = idx & (L - 1); k < K; k += L) {
-          const uint2 q = __ldg(kt + k);
+          uint32_t ka = 0, kb = 0;
+          for (int j = 0; j < op.nk; ++j) {
+            const uint2 w = op.kbit[j];
+            if ((k >> j) & 1) {
+              ka |= w.x;
+              kb |= w.y;
+            }
+          }
           // plain loads: earlier levels of this launch may have written them
-          const float2 a = A[q.x], b = B[q.y];
+          const float2 a = A[ka], b = B[kb];
           re = fmaf(a.x, b.x, re);
           re = fmaf(-a.y, b.y, re);
           im = fmaf(a.x, b.y, im);
@@ -196,7 +206,9 @@ __global__ void __cluster_dims__(PROG_CTAS, 1, 1) __launch_bounds__(PROG_THREADS
         }
       }
     }
-    if (l + 1 < lv.n) {
+    if (l + 1 < lv.n && gridDim.x == 1) {
+      __syncthreads();
+    } else if (l + 1 < lv.n) {
       asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
       asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
@@ -210,19 +222,44 @@ int prog_lanes_log2(int n_out, int nk) {
   return std::max(0, std::min({5, nk - 1, 12 - n_out}));
 }
 
-cudaError_t launch_prog(const ProgOp* ops, const uint2* ktab, const int* levels, int n_levels, int n_ops, int n_slices,
+cudaError_t launch_prog(const ProgOp* ops, const int* levels, int n_levels, int n_ops, int max_units, int n_slices,
                         int slice_id, cudaStream_t st) {
   if (n_ops < 1 || n_ops > PROG_MAX_OPS || n_levels < 1 || n_levels > n_ops || n_slices > 32)
     return cudaErrorInvalidConfiguration;
-  static const cudaError_t ok = cudaFuncSetAttribute(prog_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     int(PROG_MAX_OPS * sizeof(ProgOp)));
-  if (ok != cudaSuccess) return ok;
   ProgLevels lv;
   lv.n = n_levels;
   for (int i = 0; i <= n_levels; ++i) lv.begin[i] = short(levels[i]);
-  prog_kernel<<<PROG_CTAS, PROG_THREADS, size_t(n_ops) * sizeof(ProgOp), st>>>(ops, ktab, lv, n_ops, n_slices,
-                                                                              slice_id);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  auto shape = [&](int ctas, int threads, size_t smem) {
+    cfg.blockDim = dim3(unsigned(threads));
+    attr[0].val.clusterDim.x = unsigned(ctas);
+    cfg.gridDim = dim3(unsigned(ctas));
+    cfg.dynamicSmemBytes = smem;
+  };
+  static const int ctas = [&] {
+    if (cudaFuncSetAttribute(prog_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(PROG_MAX_OPS * sizeof(ProgOp))) != cudaSuccess)
+      return 0;
+    int n = 0;
+    shape(PROG_CTAS, PROG_THREADS, PROG_MAX_OPS * sizeof(ProgOp));
+    if (cudaFuncSetAttribute(prog_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, prog_kernel, &cfg) == cudaSuccess && n >= 1)
+      return PROG_CTAS;
+    cudaGetLastError();
+    return PROG_CTAS_PORTABLE;
+  }();
+  if (!ctas) return cudaErrorInvalidConfiguration;
+  const size_t smem = size_t(n_ops) * sizeof(ProgOp);
+  if (max_units <= 32) shape(1, PROG_THREADS, smem);
+  else if (max_units <= 256) shape(PROG_CTAS_PORTABLE, PROG_THREADS / 2, smem);
+  else shape(ctas, PROG_THREADS, smem);
+  cfg.stream = st;
+  return cudaLaunchKernelEx(&cfg, prog_kernel, ops, lv, n_ops, n_slices, slice_id);
 }
 
 int small_lanes_log2(int n_out, int nk) {
