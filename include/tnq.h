@@ -18,6 +18,8 @@
  *     says so; the library checks which with cudaPointerGetAttributes;
  *   - device memory: the library allocates none on its own; every byte it
  *     uses on the GPU lives in the workspace the caller binds to a plan;
+ *   - host memory: error flags sit in one 256 KB block of pinned memory, made
+ *     by the first call that needs one and kept until the process exits;
  *   - calls never throw; on failure they return a status other than TNQ_OK
  *     and leave a message for tnq_last_error();
  *   - GPU calls are ordered on the context's stream and return after the
@@ -328,12 +330,12 @@ tnq_status tnq_contract_pair_noalloc(tnq_ctx* ctx, const void* A, int ra, const 
  * precision's bound).  Optional outputs: steps placed on each kind of core. */
 tnq_status tnq_plan_autotune(tnq_ctx* ctx, tnq_plan* p, int reps, int* n_tensor_core, int* n_cuda_core);
 
-/* Replay full batches from a CUDA graph (1, the default) or launch every kernel
- * directly (0).  With graphs on, the first full batch of a plan at a given
- * precision captures every slice and step of one batch into a graph (on a
- * private stream) and later batches replay it on the context's stream.  The
- * results are identical either way.  Ragged last batches and timed runs
- * (tnq_ctx_set_timing) always launch directly. */
+/* Replay batches from a CUDA graph (1, the default) or launch every kernel
+ * directly (0).  With graphs on, the first batch of a plan at a given precision
+ * captures every slice and step of one batch into a graph (on a private stream);
+ * it and later batches, ragged ones included, replay the graph on the context's
+ * stream.  The results are identical either way.  Timed runs
+ * (tnq_ctx_set_timing) and partial slice ranges always launch directly. */
 tnq_status tnq_ctx_set_graphs(tnq_ctx* ctx, int enable);
 
 /* Which kernels run the steps of a plan.  TNQ_KERNELS_DEFAULT: the plan's

@@ -348,6 +348,7 @@ tnq_status tnq_expectation(tnq_ctx* c, tnq_plan* p, const double* coeffs, double
 void tnq_plan_destroy(tnq_plan* p) {
   if (!p) return;
   plan_release_graph(&p->p);
+  plan_release_flags(&p->p);
   delete p;
 }
 

@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "executor.h"
+#include "flags.h"
 #include "kernels.cuh"
 #include "gemm_tc.cuh"
 #include "traj.cuh"
@@ -496,7 +497,7 @@ tnq_status run_step(Ctx* ctx, Plan* p, size_t si, int slice_id, char* ws, int ch
   const std::vector<int>& sl = s.sliced_batch ? kNoSlices : p->slice_labels;
   return run_gemm_step(ctx, ws + ta.offset, ta.labels, s.perm_a, ws + tb.offset, tb.labels, s.perm_b, s.a_req,
                        s.b_req, sl, s.sliced_batch ? 0 : slice_id, s.nH, s.nM, s.nN, s.nK, ws + p->ws_scratch_a,
-                       ws + p->ws_scratch_b, C, acc, reinterpret_cast<int*>(ws + p->ws_misc + 4),
+                       ws + p->ws_scratch_b, C, acc, p->flags + kFlagWait,
                        ws + p->ws_partial, p->ws_scratch_b - p->ws_scratch_a, choice);
 }
 
@@ -635,30 +636,35 @@ void plan_release_graph(Plan* p) {
   p->graph_policy = -1;
 }
 
+void plan_release_flags(Plan* p) {
+  flags_put(p->flags);
+  p->flags = nullptr;
+}
+
 namespace {
 
-// Enqueue one full batch that reads its bitstrings from the staging buffer and
-// leaves its amplitudes (bitstring order) in the output staging buffer.
-tnq_status enqueue_batch(Ctx* ctx, Plan* p, int64_t nv) {
+// Enqueue every slice of a batch whose projection leaves are filled; leaves its
+// amplitudes in the FP64 accumulator.
+tnq_status enqueue_slices(Ctx* ctx, Plan* p, int64_t slice_begin, int64_t slice_count) {
   char* ws = static_cast<char*>(p->bound_ws);
-  const int w = p->batch_log2;
-  std::vector<int> bpos, opos;
-  root_positions(p, &bpos, &opos);
-  TNQ_CUDA(fill_projections(ctx, proj_leaves(p, ws), w, reinterpret_cast<const int8_t*>(ws + p->ws_bits), nv,
-                            reinterpret_cast<int*>(ws + p->ws_misc)));
   TNQ_CUDA(launch_zero(ws + p->ws_acc, 16 * (size_t(1) << p->tensors[p->root].rank), ctx->stream));
-  const int n_slices = 1 << p->slice_labels.size();
-  for (int s = 0; s < n_slices; ++s) {
-    tnq_status st = run_pass(ctx, p, s, ws, s == 0);
+  for (int64_t s = slice_begin; s < slice_begin + slice_count; ++s) {
+    tnq_status st = run_pass(ctx, p, int(s), ws, s == slice_begin);
     if (st != TNQ_OK) return st;
   }
-  TNQ_CUDA(launch_finalize(ws + p->ws_acc, ws + p->ws_out_stage, nv, bpos.data(), w, opos.data(), (int)opos.size(),
-                           p->density, ctx->stream));
-  ctx->launches++;
   return TNQ_OK;
 }
 
-// Capture enqueue_batch for a full batch into a graph (once per plan and precision).
+// Kernels of an abandoned call may still run and raise the plan's flags: wait
+// for them, so that the next call starts with flags of its own.
+tnq_status abandon(Ctx* ctx, Plan* p, tnq_status st) {
+  cudaStreamSynchronize(ctx->stream);
+  if (p->flags) flags_take(p->flags);
+  return st;
+}
+
+// Capture every slice of a batch into a graph (once per plan and precision);
+// what depends on the caller's buffers and the number of bitstrings stays outside.
 tnq_status ensure_graph(Ctx* ctx, Plan* p) {
   if (p->graph_exec && p->graph_precision == ctx->precision && p->graph_policy == ctx->kernel_policy) return TNQ_OK;
   plan_release_graph(p);
@@ -675,7 +681,7 @@ tnq_status ensure_graph(Ctx* ctx, Plan* p) {
     ctx->stream = user_stream;
     return cuda_fail(e, "cudaStreamBeginCapture");
   }
-  tnq_status st = enqueue_batch(ctx, p, int64_t(1) << p->batch_log2);
+  tnq_status st = enqueue_slices(ctx, p, 0, int64_t(1) << p->slice_labels.size());
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(ctx->stream, &g);
   ctx->stream = user_stream;
@@ -752,6 +758,8 @@ tnq_status exec_bind(Ctx* ctx, Plan* p, void* ws, size_t bytes) {
       TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
     }
   }
+  if (!p->flags && !(p->flags = flags_get()))
+    return fail(TNQ_ERR_CUDA, "no mapped host memory for the plan's error flags");
   {
     tnq_status st = upload_programs(ctx, p, base);
     if (st != TNQ_OK) return st;
@@ -784,67 +792,57 @@ tnq_status exec_amplitudes_range(Ctx* ctx, Plan* p, int64_t n_bs, const int8_t* 
     return fail(TNQ_ERR_INVALID_ARG, p->net.open_qubits.empty()
                                          ? "bitstring entries must be 0 or 1"
                                          : "bitstring entries must be -1 at the plan's open qubits and 0 or 1 elsewhere");
-  int* err_flag = reinterpret_cast<int*>(ws + p->ws_misc);
   int8_t* bits_stage = reinterpret_cast<int8_t*>(ws + p->ws_bits);
   double* out_stage = reinterpret_cast<double*>(ws + p->ws_out_stage);
   const ProjLeaves pl = proj_leaves(p, ws);
   std::vector<int> bpos, opos;
   root_positions(p, &bpos, &opos);
-  TNQ_CUDA(cudaMemsetAsync(err_flag, 0, 2 * sizeof(int), ctx->stream));
-  const size_t acc_bytes = 16 * (size_t(1) << p->tensors[p->root].rank);
   const int64_t n_slices = int64_t(1) << p->slice_labels.size();
   if (slice_begin < 0 || slice_count < 0 || slice_begin + slice_count > n_slices)
     return fail(TNQ_ERR_INVALID_ARG, "slice range outside [0, 2^n_sliced)");
   // the captured graph covers every slice; partial ranges launch directly
   const bool graphs = ctx->use_graphs && !ctx->timing && slice_begin == 0 && slice_count == n_slices;
-  {
+  // results are written where the caller wants them when that is device memory
+  // the kernel's 16-byte (complex) or 8-byte stores can address
+  const bool out_direct = out_dev && reinterpret_cast<uintptr_t>(out) % (p->density ? 8 : 16) == 0;
+  auto enqueue = [&]() -> tnq_status {
     tnq_status st = ensure_folded(ctx, p);
     if (st != TNQ_OK) return st;
-  }
-  for (int64_t base = 0; base < n_bs; base += per) {
-    int64_t nv = std::min<int64_t>(per, n_bs - base);
-    const size_t out_bytes = size_t(nv * n_out * vals) * 8;
-    if (graphs && nv == per) {
-      // full batch: stage the bitstrings, replay the captured graph, copy out
-      TNQ_CUDA(cudaMemcpyAsync(bits_stage, bits + base * rl, size_t(nv) * rl,
-                               bits_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, ctx->stream));
-      tnq_status st = ensure_graph(ctx, p);
-      if (st != TNQ_OK) return st;
-      TNQ_CUDA(cudaGraphLaunch(static_cast<cudaGraphExec_t>(p->graph_exec), ctx->stream));
-      ctx->launches += uint64_t(p->graph_nodes);
-      TNQ_CUDA(cudaMemcpyAsync(out + vals * base * n_out, out_stage, out_bytes,
-                               out_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, ctx->stream));
-      continue;
+    for (int64_t base = 0; base < n_bs; base += per) {
+      int64_t nv = std::min<int64_t>(per, n_bs - base);
+      const int8_t* bsrc = bits_dev ? bits + base * rl : bits_stage;
+      if (!bits_dev)
+        TNQ_CUDA(cudaMemcpyAsync(bits_stage, bits + base * rl, size_t(nv) * rl, cudaMemcpyHostToDevice, ctx->stream));
+      TNQ_CUDA(fill_projections(ctx, pl, w, bsrc, nv, p->flags + kFlagInput));
+      if (graphs) {
+        st = ensure_graph(ctx, p);
+        if (st != TNQ_OK) return st;
+        TNQ_CUDA(cudaGraphLaunch(static_cast<cudaGraphExec_t>(p->graph_exec), ctx->stream));
+        ctx->launches += uint64_t(p->graph_nodes);
+      } else {
+        st = enqueue_slices(ctx, p, slice_begin, slice_count);
+        if (st != TNQ_OK) return st;
+      }
+      double* user = out + vals * base * n_out;
+      TNQ_CUDA(launch_finalize(ws + p->ws_acc, out_direct ? user : out_stage, nv, bpos.data(), w, opos.data(),
+                               (int)opos.size(), p->density, ctx->stream));
+      ctx->launches++;
+      if (!out_direct)
+        TNQ_CUDA(cudaMemcpyAsync(user, out_stage, size_t(nv * n_out * vals) * 8,
+                                 out_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, ctx->stream));
     }
-    const int8_t* bsrc;
-    if (bits_dev) {
-      bsrc = bits + base * rl;
-    } else {
-      TNQ_CUDA(cudaMemcpyAsync(bits_stage, bits + base * rl, size_t(nv) * rl, cudaMemcpyHostToDevice, ctx->stream));
-      bsrc = bits_stage;
-    }
-    TNQ_CUDA(fill_projections(ctx, pl, w, bsrc, nv, err_flag));
-    TNQ_CUDA(launch_zero(ws + p->ws_acc, acc_bytes, ctx->stream));
-    for (int64_t s = slice_begin; s < slice_begin + slice_count; ++s) {
-      tnq_status st = run_pass(ctx, p, int(s), ws, s == slice_begin);
-      if (st != TNQ_OK) return st;
-    }
-    double* dst = out_dev ? out + vals * base * n_out : out_stage;
-    TNQ_CUDA(launch_finalize(ws + p->ws_acc, dst, nv, bpos.data(), w, opos.data(), (int)opos.size(), p->density,
-                             ctx->stream));
-    ctx->launches++;
-    if (!out_dev)
-      TNQ_CUDA(cudaMemcpyAsync(out + vals * base * n_out, out_stage, out_bytes, cudaMemcpyDeviceToHost, ctx->stream));
-  }
-  int herr[2] = {0, 0};
-  TNQ_CUDA(cudaMemcpyAsync(herr, err_flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-  TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
+    TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
+    return TNQ_OK;
+  };
+  tnq_status st = enqueue();
+  if (st != TNQ_OK) return abandon(ctx, p, st);
+  const FlagValues herr = flags_take(p->flags);
   if (ctx->timing) {
     tnq_status ts = timing_collect(ctx);
     if (ts != TNQ_OK) return ts;
   }
-  if (herr[1]) return fail(TNQ_ERR_TIMEOUT, "a tensor-core GEMM wait expired; results are invalid");
-  if (herr[0])
+  if (herr.wait) return fail(TNQ_ERR_TIMEOUT, "a tensor-core GEMM wait expired; results are invalid");
+  if (herr.input)
     return fail(TNQ_ERR_INVALID_ARG, p->net.open_qubits.empty()
                                          ? "bitstring entries must be 0 or 1"
                                          : "bitstring entries must be -1 at the plan's open qubits and 0 or 1 elsewhere");
@@ -917,10 +915,9 @@ tnq_status exec_autotune(Ctx* ctx, Plan* p, int reps, int* n_tc, int* n_cuda) {
   ctx->timing = timing;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (result != TNQ_OK) return result;
-  int herr = 0;
-  TNQ_CUDA(cudaMemcpy(&herr, ws + p->ws_misc + 4, sizeof(int), cudaMemcpyDeviceToHost));
-  if (herr) return fail(TNQ_ERR_TIMEOUT, "a tensor-core GEMM wait expired during autotuning");
+  if (result != TNQ_OK) return abandon(ctx, p, result);
+  TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
+  if (flags_take(p->flags).wait) return fail(TNQ_ERR_TIMEOUT, "a tensor-core GEMM wait expired during autotuning");
   p->kernel_choice = choice;
   p->tuned_precision = ctx->precision;
   p->folded_precision = -1;  // the timing runs overwrote the folded outputs
@@ -992,14 +989,12 @@ tnq_status noisy_driver(Ctx* ctx, Plan* p, int64_t traj_begin, int64_t n_traj, u
   const bool bits_dev = is_device_ptr(bits);
   if (!bits_dev && !host_bits_ok(p, n_bs, bits))
     return fail(TNQ_ERR_INVALID_ARG, "bitstring entries must be 0 or 1");
-  int* err_flag = reinterpret_cast<int*>(ws + p->ws_misc);
   int8_t* bits_stage = reinterpret_cast<int8_t*>(ws + p->ws_bits);
   const ProjLeaves pl = proj_leaves(p, ws);
   const auto& rl = p->tensors[p->root].labels;
   std::vector<int> bpos(w), tpos(t);
   for (int j = 0; j < w; ++j) bpos[j] = int(std::find(rl.begin(), rl.end(), p->net.batch_labels[j]) - rl.begin());
   for (int j = 0; j < t; ++j) tpos[j] = int(std::find(rl.begin(), rl.end(), p->net.traj_labels[j]) - rl.begin());
-  TNQ_CUDA(cudaMemsetAsync(err_flag, 0, 2 * sizeof(int), ctx->stream));
   const size_t acc_bytes = 16 * (size_t(1) << p->tensors[p->root].rank);
   const int n_slices = 1 << p->slice_labels.size();
   {
@@ -1015,7 +1010,7 @@ tnq_status noisy_driver(Ctx* ctx, Plan* p, int64_t traj_begin, int64_t n_traj, u
       TNQ_CUDA(cudaMemcpyAsync(bits_stage, bits + base * n, size_t(nv) * n, cudaMemcpyHostToDevice, ctx->stream));
       bsrc = bits_stage;
     }
-    TNQ_CUDA(fill_projections(ctx, pl, w, bsrc, nv, err_flag));
+    TNQ_CUDA(fill_projections(ctx, pl, w, bsrc, nv, p->flags + kFlagInput));
     tnq_status st = consume(-1, base, nv, 0, 0, bpos, tpos);  // batch start
     if (st != TNQ_OK) return st;
     const int64_t units = distinct ? int64_t(mult->size()) : n_traj;
@@ -1053,15 +1048,14 @@ tnq_status noisy_driver(Ctx* ctx, Plan* p, int64_t traj_begin, int64_t n_traj, u
     st = batch_end(base, nv);
     if (st != TNQ_OK) return st;
   }
-  int herr[2] = {0, 0};
-  TNQ_CUDA(cudaMemcpyAsync(herr, err_flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
+  const FlagValues herr = flags_take(p->flags);
   if (ctx->timing) {
     tnq_status ts = timing_collect(ctx);
     if (ts != TNQ_OK) return ts;
   }
-  if (herr[1]) return fail(TNQ_ERR_TIMEOUT, "a tensor-core GEMM wait expired; results are invalid");
-  if (herr[0]) return fail(TNQ_ERR_INVALID_ARG, "bitstring entries must be 0 or 1");
+  if (herr.wait) return fail(TNQ_ERR_TIMEOUT, "a tensor-core GEMM wait expired; results are invalid");
+  if (herr.input) return fail(TNQ_ERR_INVALID_ARG, "bitstring entries must be 0 or 1");
   return TNQ_OK;
 }
 
@@ -1120,7 +1114,8 @@ tnq_status exec_noisy(Ctx* ctx, Plan* p, int64_t n_traj, uint64_t seed, int64_t 
     p->dedup_n = n_traj;
   }
   p->last_distinct = (int64_t)p->dedup_mult.size();
-  return noisy_driver(ctx, p, 0, n_traj, seed, n_bs, bits, consume, batch_end, &p->dedup_picks, &p->dedup_mult);
+  st = noisy_driver(ctx, p, 0, n_traj, seed, n_bs, bits, consume, batch_end, &p->dedup_picks, &p->dedup_mult);
+  return st == TNQ_OK ? st : abandon(ctx, p, st);
 }
 
 tnq_status exec_traj_amplitudes(Ctx* ctx, Plan* p, uint64_t seed, int64_t traj_begin, int64_t n_traj, int64_t n_bs,
@@ -1156,16 +1151,16 @@ tnq_status exec_traj_amplitudes(Ctx* ctx, Plan* p, uint64_t seed, int64_t traj_b
     return TNQ_OK;
   };
   auto batch_end = [&](int64_t, int64_t) -> tnq_status { return TNQ_OK; };
-  return noisy_driver(ctx, p, traj_begin, n_traj, seed, n_bs, bits, consume, batch_end);
+  st = noisy_driver(ctx, p, traj_begin, n_traj, seed, n_bs, bits, consume, batch_end);
+  return st == TNQ_OK ? st : abandon(ctx, p, st);
 }
 
-tnq_status exec_expectation(Ctx* ctx, Plan* p, const double* coeffs, double* value, double* term_values) {
+static tnq_status run_expectation(Ctx* ctx, Plan* p, const double* coeffs, double* value, double* term_values) {
   if (!p->bound_ws) return fail(TNQ_ERR_WORKSPACE, "plan has no bound workspace");
   if (!p->expectation) return fail(TNQ_ERR_INVALID_ARG, "plan is not an expectation-value plan");
   if (!coeffs || !value) return fail(TNQ_ERR_INVALID_ARG, "NULL coefficients or value");
   TNQ_CUDA(cudaSetDevice(ctx->device));
   char* ws = static_cast<char*>(p->bound_ws);
-  int* err_flag = reinterpret_cast<int*>(ws + p->ws_misc);
   int8_t* bits_stage = reinterpret_cast<int8_t*>(ws + p->ws_bits);
   double2* stage = reinterpret_cast<double2*>(ws + p->ws_out_stage);
   const auto& rl = p->tensors[p->root].labels;
@@ -1175,10 +1170,9 @@ tnq_status exec_expectation(Ctx* ctx, Plan* p, const double* coeffs, double* val
   const int64_t tper = int64_t(1) << t;
   const size_t acc_bytes = 16 * (size_t(1) << p->tensors[p->root].rank);
   const int n_slices = 1 << p->slice_labels.size();
-  TNQ_CUDA(cudaMemsetAsync(err_flag, 0, 2 * sizeof(int), ctx->stream));
   // <0...0| closes every wire (the network is U, the Pauli operators, U^dagger)
   TNQ_CUDA(cudaMemsetAsync(bits_stage, 0, size_t(p->net.row_len), ctx->stream));
-  TNQ_CUDA(fill_projections(ctx, proj_leaves(p, ws), 0, bits_stage, 1, err_flag));
+  TNQ_CUDA(fill_projections(ctx, proj_leaves(p, ws), 0, bits_stage, 1, p->flags + kFlagInput));
   {
     tnq_status st = ensure_folded(ctx, p);
     if (st != TNQ_OK) return st;
@@ -1213,14 +1207,13 @@ tnq_status exec_expectation(Ctx* ctx, Plan* p, const double* coeffs, double* val
       for (auto& v : vals) v = host[0].x;
     }
   }
-  int herr[2] = {0, 0};
-  TNQ_CUDA(cudaMemcpyAsync(herr, err_flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
+  const FlagValues herr = flags_take(p->flags);
   if (ctx->timing) {
     tnq_status ts = timing_collect(ctx);
     if (ts != TNQ_OK) return ts;
   }
-  if (herr[1]) return fail(TNQ_ERR_TIMEOUT, "a tensor-core GEMM wait expired; results are invalid");
+  if (herr.wait) return fail(TNQ_ERR_TIMEOUT, "a tensor-core GEMM wait expired; results are invalid");
   double sum = 0.0;
   for (int64_t j = 0; j < p->n_terms; ++j) {
     sum += coeffs[j] * vals[size_t(j)];
@@ -1228,6 +1221,11 @@ tnq_status exec_expectation(Ctx* ctx, Plan* p, const double* coeffs, double* val
   }
   *value = sum;
   return TNQ_OK;
+}
+
+tnq_status exec_expectation(Ctx* ctx, Plan* p, const double* coeffs, double* value, double* term_values) {
+  const tnq_status st = run_expectation(ctx, p, coeffs, value, term_values);
+  return st == TNQ_OK || !p->bound_ws ? st : abandon(ctx, p, st);
 }
 
 // Partial-product bytes any split of an output of 2^rc elements can need.
@@ -1243,7 +1241,8 @@ size_t contract_workspace_bytes(int precision, int ra, int rb, int rc) {
 }
 
 tnq_status exec_contract_pair(Ctx* ctx, const void* A, int ra, const int* al, const void* B, int rb,
-                              const int* bl, void* C, int rc, const int* cl, void* ws, size_t ws_bytes) {
+                              const int* bl, void* C, int rc, const int* cl, void* ws, size_t ws_bytes,
+                              bool host_flag) {
   if (ra < 0 || rb < 0 || rc < 0 || ra > 31 || rb > 31 || rc > 31)
     return fail(TNQ_ERR_INVALID_ARG, "ranks must be in [0, 31]");
   std::vector<int> la(al, al + ra), lb(bl, bl + rb), lc(cl, cl + rc);
@@ -1288,10 +1287,25 @@ tnq_status exec_contract_pair(Ctx* ctx, const void* A, int ra, const int* al, co
   char* sb = w + ((32 * na + 4095) & ~size_t(4095));
   char* sc = sb + ((16 * na + 4095) & ~size_t(4095));
   int* err = reinterpret_cast<int*>(sc + ((8 * (size_t(1) << rc) + 4095) & ~size_t(4095)));
-  char* part = reinterpret_cast<char*>(err) + 4096;
-  // only the tensor-core kernels' bounded waits can raise the flag
+  char* part = reinterpret_cast<char*>(err) + 4096;  // (err as laid out in the scratch)
+  // only the tensor-core kernels' bounded waits can raise the flag; it sits in
+  // mapped host memory, or in the scratch for callers without any
   const bool flagged = ctx->precision != TNQ_PREC_FP32;
-  if (flagged) TNQ_CUDA(cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
+  struct Slot {
+    int* p = nullptr;
+    cudaStream_t st;
+    bool idle = false;
+    ~Slot() {
+      if (!p) return;
+      if (!idle) cudaStreamSynchronize(st);  // an abandoned call's kernels may still raise it
+      flags_put(p);
+    }
+  } slot;
+  slot.st = ctx->stream;
+  if (flagged && host_flag) slot.p = flags_get();
+  const bool dev_flag = flagged && !slot.p;
+  if (slot.p) err = slot.p + kFlagWait;
+  if (dev_flag) TNQ_CUDA(cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
   const bool direct = out == lc;
   DirectOut dout;
   dout.C = C;
@@ -1307,8 +1321,10 @@ tnq_status exec_contract_pair(Ctx* ctx, const void* A, int ra, const int* al, co
     TNQ_CUDA(perm(ctx, d, sc, C, nullptr, 0, 16.0 * std::ldexp(1.0, rc)));
   }
   int herr = 0;
-  if (flagged) TNQ_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  if (dev_flag) TNQ_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
+  slot.idle = true;
+  if (slot.p) herr = flags_take(slot.p).wait;
   if (ctx->timing) {
     tnq_status ts = timing_collect(ctx);
     if (ts != TNQ_OK) return ts;

@@ -37,6 +37,7 @@ struct Ctx {
 };
 
 void plan_release_graph(Plan* p);
+void plan_release_flags(Plan* p);
 tnq_status exec_autotune(Ctx* ctx, Plan* p, int reps, int* n_tc, int* n_cuda);
 
 // Timing helpers: bracket a launch when ctx->timing is set.
@@ -54,7 +55,7 @@ tnq_status exec_traj_amplitudes(Ctx* ctx, Plan* p, uint64_t seed, int64_t traj_b
                                 const int8_t* bits, double* out);
 tnq_status exec_expectation(Ctx* ctx, Plan* p, const double* coeffs, double* value, double* term_values);
 tnq_status exec_contract_pair(Ctx* ctx, const void* A, int ra, const int* al, const void* B, int rb,
-                              const int* bl, void* C, int rc, const int* cl, void* ws, size_t ws_bytes);
+                              const int* bl, void* C, int rc, const int* cl, void* ws, size_t ws_bytes, bool host_flag = true);
 size_t contract_workspace_bytes(int precision, int ra, int rb, int rc);
 
 tnq_status cuda_fail(cudaError_t e, const char* what);

@@ -88,7 +88,7 @@ extern "C" tnq_status tnq_contract_pair_noalloc(tnq_ctx* c, const void* A, int r
   run.sm_count = user.sm_count;
   run.tc_min_work = user.tc_min_work;
   tnq_status st = exec_contract_pair(&run, A, ra, a_labels, B, rb, b_labels, C, rc, c_labels, scratch,
-                                     kNoAllocScratchBytes);
+                                     kNoAllocScratchBytes, false);
   c->c.launches += run.launches;
   return st;
 }

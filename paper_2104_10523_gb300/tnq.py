@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+from array import array
 
 import numpy as np
 
@@ -106,11 +107,11 @@ def load() -> C.CDLL:
         "tnq_amplitudes": ([vp, vp, i64, vp, vp], i32),
         "tnq_noisy_probabilities": ([vp, vp, i64, u64, i64, vp, vp, vp], i32),
         "tnq_contract_workspace_bytes": ([i32, i32, i32, i32], sz),
-        "tnq_contract_pair": ([vp, vp, i32, ip, vp, i32, ip, vp, i32, ip, vp, sz], i32),
+        "tnq_contract_pair": ([vp, vp, i32, vp, vp, i32, vp, vp, i32, vp, vp, sz], i32),
         "tnq_ctx_launch_count": ([vp, C.POINTER(C.c_uint64)], i32),
         "tnq_ctx_set_timing": ([vp, i32], i32),
         "tnq_ctx_get_timings": ([vp, dp, i32, ip], i32),
-        "tnq_contract_pair_noalloc": ([vp, vp, i32, ip, vp, i32, ip, vp, i32, ip], i32),
+        "tnq_contract_pair_noalloc": ([vp, vp, i32, vp, vp, i32, vp, vp, i32, vp], i32),
         "tnq_trajectory_amplitudes": ([vp, vp, u64, i64, i64, i64, vp, vp], i32),
         "tnq_ctx_set_graphs": ([vp, i32], i32),
         "tnq_step_feature_count": ([], i32),
@@ -155,13 +156,22 @@ def _int_array(v):
     return (C.c_int * len(v))(*[int(x) for x in v])
 
 
+def _labels(v):
+    """Labels as the bytes of a C int array (a ctypes array costs several times as
+    much to build, on the order of the call itself for a small contraction)."""
+    try:
+        return array("i", v).tobytes()
+    except (TypeError, OverflowError):
+        return bytes(_int_array(v))
+
+
 def _ptr(x):
     """Data pointer of a torch tensor or a NumPy array (host or device)."""
     if x is None:
         return None
     if hasattr(x, "data_ptr"):
-        return C.c_void_p(x.data_ptr())
-    return C.c_void_p(x.ctypes.data)
+        return x.data_ptr()
+    return x.ctypes.data
 
 
 # ---------------------------------------------------------------- thin wrappers
@@ -323,16 +333,16 @@ def tnq_contract_workspace_bytes(precision, ra, rb, rc) -> int:
 
 
 def tnq_contract_pair(ctx, A, a_labels, B, b_labels, Cout, c_labels, workspace, nbytes):
-    check(load().tnq_contract_pair(ctx, _ptr(A), len(a_labels), _int_array(a_labels), _ptr(B), len(b_labels),
-                                   _int_array(b_labels), _ptr(Cout), len(c_labels), _int_array(c_labels),
+    check(load().tnq_contract_pair(ctx, _ptr(A), len(a_labels), _labels(a_labels), _ptr(B), len(b_labels),
+                                   _labels(b_labels), _ptr(Cout), len(c_labels), _labels(c_labels),
                                    _ptr(workspace), int(nbytes)))
 
 
 def tnq_contract_pair_noalloc(ctx, A, a_labels, B, b_labels, Cout, c_labels):
     """tnq_contract_pair without a workspace argument (scratch is static in the library)."""
-    check(load().tnq_contract_pair_noalloc(ctx, _ptr(A), len(a_labels), _int_array(a_labels), _ptr(B),
-                                           len(b_labels), _int_array(b_labels), _ptr(Cout), len(c_labels),
-                                           _int_array(c_labels)))
+    check(load().tnq_contract_pair_noalloc(ctx, _ptr(A), len(a_labels), _labels(a_labels), _ptr(B),
+                                           len(b_labels), _labels(b_labels), _ptr(Cout), len(c_labels),
+                                           _labels(c_labels)))
 
 
 def tnq_plan_autotune(ctx, plan, reps=3):
