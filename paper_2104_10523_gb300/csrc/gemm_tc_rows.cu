@@ -50,11 +50,8 @@
 //               tile): each thread owns one tile row and walks the item's K
 //               range in chunks of up to 16 complex values (loads
 //               of 16-byte pairs when the lowest stored bit is a K bit); the
-//               loads of the next chunks are issued before the current one is
-//               split and stored, and the register ring rotates by moves,
-//               which wait for the newest load, so in effect one chunk is in
-//               flight across each split (an unrolled ring without the moves
-//               measured slower);
+//               loads of the next chunk are in flight while one is split and
+//               stored;
 //   warp 8      allocates TMEM and (one thread) issues the MMAs of each tile
 //               into one of the TMEM accumulator buffers;
 //   warps 9-12  epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, 32
@@ -158,6 +155,22 @@ __device__ __forceinline__ void bf16_split2(float x0, float x1, uint32_t* hi, ui
   *lo = l0 | (l1 << 16);
 }
 
+// a - b and a + b of two floats each (one instruction a pair on sm_100 and up).
+__device__ __forceinline__ float2 sub2(float ax, float ay, float bx, float by) {
+  float2 r;
+  asm("{\n.reg .b64 a, b;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nsub.rn.f32x2 a, a, b;\nmov.b64 {%0, %1}, a;\n}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(ax), "f"(ay), "f"(bx), "f"(by));
+  return r;
+}
+__device__ __forceinline__ float2 add2(float ax, float ay, float bx, float by) {
+  float2 r;
+  asm("{\n.reg .b64 a, b;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nadd.rn.f32x2 a, a, b;\nmov.b64 {%0, %1}, a;\n}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(ax), "f"(ay), "f"(bx), "f"(by));
+  return r;
+}
+
 // Byte offset of 16-byte unit u of row r in a K-major tile of 128-byte-swizzled
 // atoms: atom u / 8 (atom columns atom_bytes apart), 8-row groups of 1024 bytes
 // within an atom, unit index XOR row-in-group.
@@ -166,44 +179,46 @@ __device__ __forceinline__ uint32_t swz(int r, int u, uint32_t atom_bytes) {
 }
 
 // Split chunk c (complex values c*CH .. c*CH+CH-1 of the row, zero beyond K)
-// and store its 16-byte units that the MMAs read (units < 2 * nks).
+// and store its 16-byte units.  Unit u of row r sits at swz(r, u); a chunk's UN
+// units are one aligned group of an atom's eight, so that the XOR with the
+// row-in-group splits into a part per chunk and a part per unit of the chunk.
 template <int CH>
-__device__ __forceinline__ void store_chunk(uint8_t* hi, uint8_t* lo, int r, const float2 (&v)[CH], int c,
-                                            int units, int kind_bf16, int split) {
+__device__ __forceinline__ void store_chunk(uint8_t* hi, uint32_t lo_off, int r, const float2 (&v)[CH], int c,
+                                            int kind_bf16, int split) {
+  constexpr int kUnitsBf16 = CH / 4, kUnitsTf32 = CH / 2;
+  const int un = kind_bf16 ? kUnitsBf16 : kUnitsTf32, u0 = c * un;
+  hi += uint32_t(u0 >> 3) * TR_ATOM_BYTES + uint32_t(r) * 128u + (uint32_t((u0 & 7) ^ (r & 7 & ~(un - 1))) << 4);
+  const uint32_t x = uint32_t(r & (un - 1)) << 4;
   if (kind_bf16) {
     // one unit: 4 complex values (8 BF16 reals)
 #pragma unroll
-    for (int j = 0; j < CH / 4; ++j) {
-      const int u = c * (CH / 4) + j;
-      if (u < units) {
-        uint4 h, l;
-        bf16_split2(v[4 * j].x, v[4 * j].y, &h.x, &l.x);
-        bf16_split2(v[4 * j + 1].x, v[4 * j + 1].y, &h.y, &l.y);
-        bf16_split2(v[4 * j + 2].x, v[4 * j + 2].y, &h.z, &l.z);
-        bf16_split2(v[4 * j + 3].x, v[4 * j + 3].y, &h.w, &l.w);
-        *reinterpret_cast<uint4*>(hi + swz(r, u, TR_ATOM_BYTES)) = h;
-        *reinterpret_cast<uint4*>(lo + swz(r, u, TR_ATOM_BYTES)) = l;
-      }
+    for (int j = 0; j < kUnitsBf16; ++j) {
+      uint4 h, l;
+      bf16_split2(v[4 * j].x, v[4 * j].y, &h.x, &l.x);
+      bf16_split2(v[4 * j + 1].x, v[4 * j + 1].y, &h.y, &l.y);
+      bf16_split2(v[4 * j + 2].x, v[4 * j + 2].y, &h.z, &l.z);
+      bf16_split2(v[4 * j + 3].x, v[4 * j + 3].y, &h.w, &l.w);
+      uint8_t* at = hi + ((uint32_t(j) << 4) ^ x);
+      *reinterpret_cast<uint4*>(at) = h;
+      *reinterpret_cast<uint4*>(at + lo_off) = l;
     }
   } else {
     // one unit: 2 complex values (4 TF32 reals)
 #pragma unroll
-    for (int j = 0; j < CH / 2; ++j) {
-      const int u = c * (CH / 2) + j;
-      if (u < units) {
-        float4 h, l;
-        h.x = tf32_rna(v[2 * j].x);
-        h.y = tf32_rna(v[2 * j].y);
-        h.z = tf32_rna(v[2 * j + 1].x);
-        h.w = tf32_rna(v[2 * j + 1].y);
-        *reinterpret_cast<float4*>(hi + swz(r, u, TR_ATOM_BYTES)) = h;
-        if (split) {
-          l.x = tf32_rna(v[2 * j].x - h.x);
-          l.y = tf32_rna(v[2 * j].y - h.y);
-          l.z = tf32_rna(v[2 * j + 1].x - h.z);
-          l.w = tf32_rna(v[2 * j + 1].y - h.w);
-          *reinterpret_cast<float4*>(lo + swz(r, u, TR_ATOM_BYTES)) = l;
-        }
+    for (int j = 0; j < kUnitsTf32; ++j) {
+      float4 h;
+      h.x = tf32_rna(v[2 * j].x);
+      h.y = tf32_rna(v[2 * j].y);
+      h.z = tf32_rna(v[2 * j + 1].x);
+      h.w = tf32_rna(v[2 * j + 1].y);
+      uint8_t* at = hi + ((uint32_t(j) << 4) ^ x);
+      *reinterpret_cast<float4*>(at) = h;
+      if (split) {
+        // The remainder of a nearest TF32 value has at most 12 significant bits:
+        // the MMA, which ignores the low 13 bits of a TF32 operand, drops one of
+        // them at most, as far as a rounding of the remainder would move it.
+        const float2 l0 = sub2(v[2 * j].x, v[2 * j].y, h.x, h.y), l1 = sub2(v[2 * j + 1].x, v[2 * j + 1].y, h.z, h.w);
+        *reinterpret_cast<float4*>(at + lo_off) = make_float4(l0.x, l0.y, l1.x, l1.y);
       }
     }
   }
@@ -284,22 +299,27 @@ __device__ __forceinline__ size_t deposit(long long v, const int* pos, int n) {
   return o;
 }
 
-// Chunk c of K-part kp of the row whose K = 0 element sits at stored offset `base`.
+// A chunk of the row whose first element of the chunk sits at p; kj: offsets of
+// the chunk's values within any chunk (beyond K they repeat valid ones, and the
+// values are zeroed).
 template <int CH>
-__device__ __forceinline__ void load_chunk(const TrParams& P, const uint32_t* koff, size_t base, int kp, int c,
+__device__ __forceinline__ void load_chunk(const TrParams& P, const float2* p, const uint32_t (&kj)[CH],
                                            float2 (&v)[CH]) {
-  const int k0 = kp * P.kc + c * CH;
   if (P.pairs) {
 #pragma unroll
     for (int j = 0; j < CH; j += 2) {
-      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (k0 + j < P.K) t = __ldg(reinterpret_cast<const float4*>(P.G + base + koff[k0 + j]));
+      const float4 t = __ldg(reinterpret_cast<const float4*>(p + kj[j]));
       v[j] = make_float2(t.x, t.y);
       v[j + 1] = make_float2(t.z, t.w);
     }
   } else {
 #pragma unroll
-    for (int j = 0; j < CH; ++j) v[j] = k0 + j < P.K ? __ldg(P.G + base + koff[k0 + j]) : make_float2(0.f, 0.f);
+    for (int j = 0; j < CH; ++j) v[j] = __ldg(p + kj[j]);
+  }
+  if (P.K < CH) {
+#pragma unroll
+    for (int j = 0; j < CH; ++j)
+      if (j >= P.K) v[j] = make_float2(0.f, 0.f);
   }
 }
 
@@ -309,7 +329,7 @@ __device__ __forceinline__ void load_chunk(const TrParams& P, const uint32_t* ko
 // instructions it issued), so each mode is its own kernel.
 // MINB: CTAs per SM (2 for launches whose stages, S' and TMEM buffers fit in
 // half an SM: twice the warps to hide the roles' latencies, 72 registers).
-template <int CH, int DEPTH, int MODE, int MINB>
+template <int CH, int MODE, int MINB>
 __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const __grid_constant__ TrParams P) {
   extern __shared__ uint8_t smem_raw[];
   // batch entry of a per-entry grid (0 otherwise), read where it is needed: the
@@ -391,7 +411,7 @@ __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const _
     // quotients and remainders from item to item instead of dividing.
     const int grp = warp >> 2, r = (warp & 3) * 32 + lane;
     const int nhi = P.gd.nrow - 7;
-    const int nch = P.nchunks, units = 2 * P.nks_part;
+    const int nch = P.nchunks;
     const uint32_t nst = uint32_t(P.stages);
     size_t soff = 0;
     for (int j = 0; j < P.gd.n_slice; ++j)
@@ -424,36 +444,36 @@ __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const _
         q.tile += gridDim.x;
       }
     };
-    // items (item, chunk c) in order: the loads of the next DEPTH chunks are in
-    // flight while one is split and stored.
+    // items (item, chunk c) in order: the loads of the next chunk are in flight
+    // while one is split and stored.  The two buffers rotate by moves; an
+    // unrolled ring (609 us) or a ring of asynchronous copies through shared
+    // memory (424 us) ran 16 x 2^23 x 16 slower (409): the kernel is bound by
+    // instruction issue, and those add instructions or instruction-cache misses.
+    uint32_t kj[CH];
+#pragma unroll
+    for (int j = 0; j < CH; ++j) kj[j] = koff[j];
     ItemCursor ql = first_item();  // load cursor: item, chunk, its tile's row base
     int cl = 0;
-    size_t bl = ql.tile < total ? row_base(ql.tile) : 0;
-    auto advance_load = [&]() {
+    const float2* bl = P.G + (ql.tile < total ? row_base(ql.tile) : 0);
+    auto load_next = [&](float2 (&v)[CH]) {
+      if (ql.tile < total) load_chunk<CH>(P, bl + koff[int(ql.kp) * P.kc + cl * CH], kj, v);
       if (++cl == nch) {
         cl = 0;
         const uint32_t t0 = ql.tile;
         next_item(ql);
-        if (ql.tile != t0) bl = ql.tile < total ? row_base(ql.tile) : 0;
+        if (ql.tile != t0 && ql.tile < total) bl = P.G + row_base(ql.tile);
       }
     };
-    float2 buf[DEPTH + 1][CH];
-#pragma unroll
-    for (int d = 0; d < DEPTH; ++d) {
-      if (ql.tile < total) load_chunk<CH>(P, koff, bl, int(ql.kp), cl, buf[d]);
-      advance_load();
-    }
     ItemCursor qc = first_item();  // convert cursor
     uint32_t s = uint32_t(grp), ph = 0;  // its stage and phase: j % stages, (j / stages) & 1
     int c = 0;
-    while (qc.tile < total) {
+    auto convert = [&](const float2 (&v)[CH]) {
+      if (qc.tile >= total) return false;
       // the empty wait orders this item after the MMAs of item j - stages,
       // whichever group converted that one, so any stage count works
-      if (ql.tile < total) load_chunk<CH>(P, koff, bl, int(ql.kp), cl, buf[DEPTH]);
-      advance_load();
       if (c == 0 && !mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1)) {
         atomicOr(P.err, 1);
-        break;
+        return false;
       }
       uint8_t* st = smem + size_t(s) * stage_bytes;
       if (c == 0 && P.stream_bp && r == 0) {
@@ -464,15 +484,11 @@ __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const _
         mbar_expect_tx(bar, 2u * P.bp_part);
         bulk_g2s(smem_u32(st + 2 * g_piece), src, 2u * P.bp_part, bar);
       }
-      store_chunk<CH>(st, st + g_piece, r, buf[0], c, units, kBF16, kSplit);
+      store_chunk<CH>(st, g_piece, r, v, c, kBF16, kSplit);
       if (c == nch - 1) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(smem_u32(&full_bar[s]));
       }
-#pragma unroll
-      for (int d = 0; d < DEPTH; ++d)
-#pragma unroll
-        for (int j = 0; j < CH; ++j) buf[d][j] = buf[d + 1][j];
       if (++c == nch) {
         c = 0;
         next_item(qc);
@@ -482,6 +498,15 @@ __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const _
           ph ^= 1u;
         }
       }
+      return true;
+    };
+    float2 va[CH], vb[CH];
+    load_next(va);
+    load_next(vb);
+    while (convert(va)) {
+      load_next(va);
+      if (!convert(vb)) break;
+      load_next(vb);
     }
   } else if (warp == TR_MMA_WARP) {
     if (lane == 0) {
@@ -595,7 +620,12 @@ __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const _
         }
         float o[EC];
 #pragma unroll
-        for (int j = 0; j < EC; ++j) o[j] = P.dual ? __uint_as_float(v[j]) + __uint_as_float(w[j]) : __uint_as_float(v[j]);
+        for (int j = 0; j < EC; j += 2) {
+          const float a = __uint_as_float(v[j]), b = __uint_as_float(v[j + 1]);
+          const float2 t2 = P.dual ? add2(a, b, __uint_as_float(w[j]), __uint_as_float(w[j + 1])) : make_float2(a, b);
+          o[j] = t2.x;
+          o[j + 1] = t2.y;
+        }
         if (c0 + EC < P.npad) {
           tmem_ld(c0 + EC);
         } else {
@@ -603,20 +633,24 @@ __global__ void __launch_bounds__(TR_THREADS, MINB) cgemm_tc_rows_kernel(const _
           __syncwarp();
           if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
         }
+        const int s0 = c0 / 2;
+        if (P.acc) {
 #pragma unroll
-        for (int j = 0; j < EC / 2; ++j) {
-          const int s = c0 / 2 + j;
-          if (s < P.ns) {
-            const float re = o[2 * j], im = o[2 * j + 1];
-            const size_t o_at = obase + size_t(s) * P.ng;
-            if (P.acc) {
-              double2 a = P.acc[o_at];
-              a.x += double(re);
-              a.y += double(im);
-              P.acc[o_at] = a;
-            } else {
-              P.C[o_at] = make_float2(re, im);
+          for (int j = 0; j < EC / 2; ++j)
+            if (s0 + j < P.ns) {
+              double2* at = P.acc + obase + size_t(s0 + j) * P.ng;
+              double2 a = *at;
+              a.x += double(o[2 * j]);
+              a.y += double(o[2 * j + 1]);
+              *at = a;
             }
+        } else {
+          float2* at = P.C + obase + size_t(s0) * P.ng;
+          const int left = P.ns - s0;
+#pragma unroll
+          for (int j = 0; j < EC / 2; ++j) {
+            if (j < left) *at = make_float2(o[2 * j], o[2 * j + 1]);
+            at += P.ng;
           }
         }
       }
@@ -705,12 +739,12 @@ size_t tc_rows_scratch_bytes(int ns, int K, int batch, int precision) {
 // kernels by [CH == 16][MODE]
 using TrKernel = void (*)(TrParams);
 const TrKernel kTrKernels[2][3] = {
-    {cgemm_tc_rows_kernel<8, 4, 0, 1>, cgemm_tc_rows_kernel<8, 4, 1, 1>, cgemm_tc_rows_kernel<8, 4, 2, 1>},
-    {cgemm_tc_rows_kernel<16, 2, 0, 1>, cgemm_tc_rows_kernel<16, 2, 1, 1>, cgemm_tc_rows_kernel<16, 2, 2, 1>},
+    {cgemm_tc_rows_kernel<8, 0, 1>, cgemm_tc_rows_kernel<8, 1, 1>, cgemm_tc_rows_kernel<8, 2, 1>},
+    {cgemm_tc_rows_kernel<16, 0, 1>, cgemm_tc_rows_kernel<16, 1, 1>, cgemm_tc_rows_kernel<16, 2, 1>},
 };
 // two CTAs per SM, by [MODE]
-const TrKernel kTrKernels2[3] = {cgemm_tc_rows_kernel<8, 2, 0, 2>, cgemm_tc_rows_kernel<8, 2, 1, 2>,
-                                 cgemm_tc_rows_kernel<8, 2, 2, 2>};
+const TrKernel kTrKernels2[3] = {cgemm_tc_rows_kernel<8, 0, 2>, cgemm_tc_rows_kernel<8, 1, 2>,
+                                 cgemm_tc_rows_kernel<8, 2, 2>};
 
 
 cudaError_t tc_rows_prepare() {
