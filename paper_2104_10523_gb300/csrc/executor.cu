@@ -253,10 +253,15 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
                           !use_dot(nM, nN, nK) &&
                           tc_rows_supported(1 << n_small, 1 << n_big, 1 << nK, 1 << nH, n_big + nH, ctx->precision) &&
                           tc_rows_scratch_bytes(1 << n_small, 1 << nK, 1 << nH, ctx->precision) <= tr_avail;
-  // A batch whose expanded small operands do not fit one CTA leaves the tensor
-  // cores unless a row's arithmetic would bound the CUDA cores: each batch
-  // entry would fill its own S' and few tiles.  The plain TF32 mode keeps its
-  // operand rounding.
+  // Low-intensity short-K steps leave the tensor cores for the gather kernel,
+  // which moves their bytes faster (the tall-skinny kernel is bound by the
+  // instructions of its hi/lo split): up to 7 flops per byte where the expanded
+  // small operands share a CTA (TF32x3 kernel, then FP32 gather, in us: 4 x 2^22 x
+  // 32 317 / 197, 8 x 2^22 x 16 166 / 131, 8 x 2^23 x 32 597 / 463, 32 x 2^23 x 8
+  // 465 / 426; above the line they draw level, 64 x 2^21 x 8 213 / 203, 16 x 2^23 x
+  // 16 398 / 392, then turn, 32 x 2^22 x 16 275 / 368, 16 x 2^21 x 32 167 / 211),
+  // to the gather kernel's own line where each batch entry would need its S' and
+  // few tiles (see gather_bound).  The plain TF32 mode keeps its operand rounding.
   //
   // In a plan the modes whose operands are rounded coarsely (2^-11, or 2^-17 for
   // the BF16 split) keep the tensor cores there and the order of every sum
@@ -265,7 +270,8 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   // choice of kernel would show in the amplitudes (1e-4 in TF32).
   const bool ordered = !direct && (ctx->precision == TNQ_PREC_TF32 || ctx->precision == TNQ_PREC_BF16X3);
   const bool batched = tc_rows_ok && choice == -1 && !ordered && gather_bound(nM, nN, nK) &&
-                       !tc_rows_shared_ok(1 << n_small, 1 << nK, 1 << nH, ctx->precision);
+                       (!tc_rows_shared_ok(1 << n_small, 1 << nK, 1 << nH, ctx->precision) ||
+                        flops_per_byte(n_small, nK) <= 7.0);
   const bool tc_rows = tc_rows_ok && !batched;
   const bool round_tf32 = batched && ctx->precision == TNQ_PREC_TF32;
   // The A side is never the larger one (both hold the H and K labels), so M is

@@ -18,6 +18,13 @@ namespace {
 constexpr int GATHER_SMAX = 128;  // small-operand rows of the gather kernel
 constexpr int GATHER_REPS = 4;    // row blocks of a CTA
 
+// CTAs an SM the register allocation leaves room for: without the bound the
+// compiler unrolls into 80 registers at K = 8 and a quarter of the warps goes
+// (8 x 2^23 x 8 176 -> 192 us a call).
+constexpr int gather_min_ctas(int K, int rows) {
+  return K <= 2 ? (rows == 2 ? 8 : 6) : K == 4 ? 6 : K == 8 ? 4 : K == 16 ? (rows == 2 ? 5 : 4) : rows == 2 ? 3 : 2;
+}
+
 // Nearest TF32 value, ties away from zero (finite inputs).
 __device__ __forceinline__ float2 tf32_rna2(float2 v) {
   return make_float2(__uint_as_float((__float_as_uint(v.x) + 0x1000u) & 0xffffe000u),
@@ -30,24 +37,27 @@ __device__ __forceinline__ float2 tf32_rna2(float2 v) {
 // dep(k, kpos) further on.  One thread owns ROWS rows, held in registers; a CTA
 // owns cta_rows consecutive rows of the batch-major row index, so with short
 // rows (ng < cta_rows) it serves several batch entries, whose S rows it stages
-// together, gathered from their stored layout (one 16-byte pad per entry spreads the entries over the banks);
-// with ROWS = 2 a CTA stays within one entry.  A CTA of a single entry walks
+// together, gathered from their stored layout (one 16-byte pad per entry spreads
+// the entries over the banks); with ROWS = 2 a CTA stays within one entry.  A CTA
+// of a single entry walks
 // reps blocks of rows, so that staging S (a dependent gather before the first
 // row can be used) is paid once for all of them.
 // ROUND rounds both operands to TF32 first (the products are then exact in
 // FP32: the arithmetic of the plain TF32 mode on the CUDA cores).
 //
 // Bound: HBM while 4 FFMA per (s, k) of a row stay below the 8 (K + ns) bytes
-// it moves.  One launch for every batch entry: 4096 entries of 4 x 2^12 x 8
+// it moves, then the shared-memory reads of S (16 bytes to 32 lanes take four
+// cycles of the one port), which ROWS = 2 halves: 16 x 2^23 x 16 466 -> 392 us,
+// 8 x 2^23 x 32 545 -> 463 (from K = 16 on in CTAs of 128 threads, whose load and
+// compute phases overlap better, five of them an SM at K = 16).  8 x 2^25 x 8
+// moves 6.8 TB/s.  One launch for every batch entry: 4096 entries of 4 x 2^12 x 8
 // took 33.5 ms as one tensor-core launch each (8 us a launch).
-template <int K, int ROWS, bool ROUND>
-__global__ void __launch_bounds__(256) cgemm_rows_gather_kernel(const float2* __restrict__ S,
-                                                                const __grid_constant__ SmallDesc sd,
-                                                                const float2* __restrict__ G,
-                                                                const __grid_constant__ GatherDesc gd,
-                                                                float2* __restrict__ C, double2* __restrict__ acc,
-                                                                int ns, int log_per, int log_ng, int cta_rows,
-                                                                int reps, int entries, int slice_id) {
+template <int K, int ROWS, bool ROUND, int T>
+__global__ void __launch_bounds__(T, gather_min_ctas(K, ROWS))
+    cgemm_rows_gather_kernel(const float2* __restrict__ S, const __grid_constant__ SmallDesc sd,
+                             const float2* __restrict__ G, const __grid_constant__ GatherDesc gd,
+                             float2* __restrict__ C, double2* __restrict__ acc, int ns, int log_per, int log_ng,
+                             int cta_rows, int reps, int entries, int slice_id) {
   extern __shared__ __align__(16) float2 Ss[];  // [entries][ns * K + 2]
   __shared__ unsigned long long blk_base[GATHER_REPS];
   const int t = threadIdx.x;
@@ -63,13 +73,13 @@ __global__ void __launch_bounds__(256) cgemm_rows_gather_kernel(const float2* __
       if ((R0 >> j) & 1) o |= 1ull << gd.rowpos[j];
     blk_base[t] = o;
   }
-  for (int i = t; i < entries * per; i += 256) {
+  for (int i = t; i < entries * per; i += T) {
     const float2 v = __ldg(S + small_dep(sd, (uint32_t(h0) << log_per) + i));
     Ss[i + 2 * (i >> log_per)] = ROUND ? tf32_rna2(v) : v;
   }
   size_t lo = 0;
 #pragma unroll
-  for (int j = 0; j < 8; ++j)
+  for (int j = 0; (1 << j) < T; ++j)
     if (j < gd.nrow && ((t >> j) & 1)) lo |= size_t(1) << gd.rowpos[j];
   __syncthreads();
   const bool pairs = K > 1 && gd.kpos[0] == 0;
@@ -79,9 +89,9 @@ __global__ void __launch_bounds__(256) cgemm_rows_gather_kernel(const float2* __
     float2 gv[ROWS][K];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
-      live[r] = r * 256 + t < cta_rows;
+      live[r] = r * T + t < cta_rows;
       size_t base = size_t(blk_base[it]) | lo;
-      if (r) base |= size_t(1) << gd.rowpos[8];  // ROWS <= 2: the row bit above the thread bits
+      if (r) base |= size_t(1) << gd.rowpos[T == 256 ? 8 : 7];  // ROWS <= 2: the row bit above the thread bits
 #pragma unroll
       for (int kk = 0; kk < K; ++kk) gv[r][kk] = make_float2(0.f, 0.f);
       if (live[r]) {
@@ -120,7 +130,7 @@ __global__ void __launch_bounds__(256) cgemm_rows_gather_kernel(const float2* __
     const float2* Sr = Ss;
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
-      const long long R = R0 + (live[r] ? r * 256 + t : 0);
+      const long long R = R0 + (live[r] ? r * T + t : 0);
       const size_t h = size_t(R >> log_ng);
       obase[r] = ((h * size_t(ns)) << log_ng) + size_t(R & ((1ll << log_ng) - 1));
       if (ROWS == 1) Sr = Ss + (int(h) - h0) * pitch;
@@ -188,8 +198,9 @@ cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const SmallDesc& sd, co
   if (total != 1ll << gd.nrow) return cudaErrorInvalidConfiguration;
   // two rows a thread (each S value read serves both) while registers allow
   // and the halved grid still covers the chip
-  const int rows = K <= 8 && ng >= 512 && total >= 512ll * 4 * std::max(1, sm_count) ? 2 : 1;
-  long long cta_rows = std::min<long long>(total, 256 * rows);
+  const int rows = ng >= 512 && total >= 512ll * 4 * std::max(1, sm_count) ? 2 : 1;
+  const int threads = K >= 16 && rows == 2 ? 128 : 256;
+  long long cta_rows = std::min<long long>(total, threads * rows);
   const long long entry_bytes = 8ll * (ns * K + 2);
   // S rows of every entry of the CTA within 32 KB: fewer rows where many entries meet
   while (cta_rows > ng && (cta_rows / ng) * entry_bytes > 32 * 1024) cta_rows /= 2;
@@ -206,8 +217,8 @@ cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const SmallDesc& sd, co
   float2* Cp = reinterpret_cast<float2*>(C);
   double2* Ap = reinterpret_cast<double2*>(acc);
 #define TNQ_GATHER1(K_, R_, T_) \
-  cgemm_rows_gather_kernel<K_, R_, T_><<<grid, 256, smem, st>>>(Sp, sd, Gp, gd, Cp, Ap, ns, log_per, log_ng, int(cta_rows), reps, entries, \
-                                                      slice_id)
+  cgemm_rows_gather_kernel<K_, R_, T_, (K_ >= 16 && R_ == 2 ? 128 : 256)><<<grid, threads, smem, st>>>(       \
+      Sp, sd, Gp, gd, Cp, Ap, ns, log_per, log_ng, int(cta_rows), reps, entries, slice_id)
 #define TNQ_GATHER(K_, R_)                   \
   do {                                       \
     if (round_tf32) TNQ_GATHER1(K_, R_, true); \
@@ -223,8 +234,8 @@ cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const SmallDesc& sd, co
     case 2: TNQ_GATHER12(2); break;
     case 4: TNQ_GATHER12(4); break;
     case 8: TNQ_GATHER12(8); break;
-    case 16: TNQ_GATHER(16, 1); break;
-    default: TNQ_GATHER(32, 1);
+    case 16: TNQ_GATHER12(16); break;
+    default: TNQ_GATHER12(32);
   }
 #undef TNQ_GATHER12
 #undef TNQ_GATHER

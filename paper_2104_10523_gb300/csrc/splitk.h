@@ -25,16 +25,22 @@ inline bool skinny(int nM, int nN, int nK) {
   return s <= 4;
 }
 
+// Flops per byte of a skinny step: 8 M K flops and 8 (M + K) bytes per row of the
+// large operand.
+inline double flops_per_byte(int nS, int nK) {
+  const double m = std::ldexp(1.0, nS), k = std::ldexp(1.0, nK);
+  return m * k / (m + k);
+}
+
 // Whether the short-K gather kernel runs the step near the memory bound: K of at
-// most 32 (a row sits in registers) and a small side of at most 128 rows whose
-// 8 M K flops per row of the large operand stay below about 10 flops per byte
-// moved, the FFMA rate over the memory rate (60 TF/s achieved, 6 TB/s).
+// most 32 (a row sits in registers) and a small side of at most 128 rows at no
+// more than about 10 flops per byte, the FFMA rate over the memory rate (60 TF/s
+// achieved, 6 TB/s).
 inline bool gather_bound(int nM, int nN, int nK) {
   const int s = nM < nN ? nM : nN;
   if (nK > 5 || s > 7) return false;
   if (s <= 5) return true;  // register rows beat staged or tiled kernels even above that line
-  const double m = std::ldexp(1.0, s), k = std::ldexp(1.0, nK);
-  return m * k <= 10.0 * (m + k);
+  return flops_per_byte(s, nK) <= 10.0;
 }
 
 // Tiny outputs (M, N <= 8) with a long contracted dimension never fill a
