@@ -226,9 +226,9 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   // idle.  An autotuned choice (0 CUDA cores, 1 tensor cores) overrides the rule.
   const double work = std::ldexp(1.0, nH + nM + nN + nK);
   const bool tc_ok = ctx->precision != TNQ_PREC_FP32 && tc_gemm_supported(1 << nM, 1 << nN, 1 << nK, ctx->precision);
-  const bool use_tc = choice == 1 ? tc_ok
-                      : choice == 0 ? false
-                                    : tc_ok && !skinny(nM, nN, nK) && work >= ctx->tc_min_work;
+  bool use_tc = choice == 1 ? tc_ok
+                : choice == 0 ? false
+                              : tc_ok && !skinny(nM, nN, nK) && work >= ctx->tc_min_work;
   const size_t out_elems = size_t(1) << (nH + nM + nN);
   const int prec = use_tc ? ctx->precision : TNQ_PREC_FP32;
   StepOperands op;
@@ -273,6 +273,12 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
                        (!tc_rows_shared_ok(1 << n_small, 1 << nK, 1 << nH, ctx->precision) ||
                         flops_per_byte(n_small, nK) <= 7.0);
   const bool tc_rows = tc_rows_ok && !batched;
+  // The general tensor-core GEMM converts both operands in passes of their own:
+  // low-intensity steps it would take (rows too short for the tall-skinny kernel)
+  // go to the gather kernel too.
+  if (use_tc && choice == -1 && !ordered && !tc_rows && !batched && gather_bound(nM, nN, nK) &&
+      flops_per_byte(n_small, nK) <= 7.0 && ctx->precision != TNQ_PREC_TF32)
+    use_tc = false;
   const bool round_tf32 = batched && ctx->precision == TNQ_PREC_TF32;
   // The A side is never the larger one (both hold the H and K labels), so M is
   // the small side of a skinny step.

@@ -111,9 +111,10 @@ __global__ void __launch_bounds__(SM_THREADS) cgemm_small_kernel(const __grid_co
 // step by its place among the level's warp-sized units.
 // The cluster grows with the largest level: one CTA for at most 2^10 outputs (a
 // block barrier is cheaper than a cluster's), eight of 16 warps for at most 2^13,
-// sixteen of 32 warps above (eight where a cluster of sixteen cannot be placed;
-// a level of 2^14 outputs is then one round of the warps).  A 4x5 noisy pass
-// (levels of 2^14) took 132 us with eight of 16 warps, 48 with sixteen of 32.
+// sixteen of 32 warps above (eight where a cluster of sixteen cannot be placed).
+// A 4x5 noisy pass, whose levels hold many steps of 2^14 outputs, took 132 us with
+// eight of 16 warps and 48 with sixteen of 32; a 3x4 batch loses 5 us to the
+// wider launch.
 constexpr int PROG_CTAS = 16, PROG_CTAS_PORTABLE = 8, PROG_THREADS = 1024;
 
 struct ProgLevels {
@@ -156,38 +157,66 @@ __global__ void __launch_bounds__(PROG_THREADS)
         at += __popc(m);
       }
       const ProgOp& op = ops[at];
-      const uint32_t idx = (u - op.warp_begin) * 32 + lane;
-      const uint32_t o = idx >> op.log_l, L = 1u << op.log_l, K = 1u << op.nk;
-      const bool live = o < 1u << op.n_out;
+      // Output index o = idx >> log_l: its bits above the lanes' are the same for
+      // the whole warp, so lane j contributes bit j's offsets and the warp ORs them;
+      // the lanes' own bits are at most five.  (A loop over the record's bits in
+      // every lane was a chain of shared-memory reads, most of a level's time.)
+      const int n_out = op.n_out, log_l = op.log_l, nk = op.nk, lane_bits = 5 - log_l;
+      const uint32_t idx = (u - op.warp_begin) * 32 + lane, L = 1u << log_l;
+      const uint32_t o = idx >> log_l;
+      const bool live = o < 1u << n_out;
       uint32_t oa = 0, ob = 0, oc = 0;
-      for (int j = 0; j < op.n_out; ++j) {
-        const uint4 w = op.bit[j];
-        if ((o >> j) & 1) {
+      if (lane >= lane_bits && lane < n_out && ((o >> lane) & 1)) {
+        const uint4 w = op.bit[lane];
+        oa = w.x;
+        ob = w.y;
+        oc = w.z;
+      }
+      oa = __reduce_or_sync(0xffffffffu, oa);
+      ob = __reduce_or_sync(0xffffffffu, ob);
+      oc = __reduce_or_sync(0xffffffffu, oc);
+#pragma unroll
+      for (int j = 0; j < 5; ++j)
+        if (j < lane_bits && j < n_out && ((o >> j) & 1)) {
+          const uint4 w = op.bit[j];
           oa |= w.x;
           ob |= w.y;
           oc |= w.z;
         }
-      }
+      // K index: its low log_l bits are the lane's, the others count the
+      // iterations; lane q holds the offsets of iteration q (of 32 at a time)
+#pragma unroll
+      for (int j = 0; j < 5; ++j)
+        if (j < log_l && ((idx >> j) & 1)) {
+          const uint2 w = op.kbit[j];
+          oa |= w.x;
+          ob |= w.y;
+        }
+      const float2* A = reinterpret_cast<const float2*>(op.a) + (live ? oa : 0);
+      const float2* B = reinterpret_cast<const float2*>(op.b) + (live ? ob : 0);
+      const int kb_iter = nk - log_l, iters = 1 << kb_iter;
       float re = 0.f, im = 0.f;
-      if (live) {
-        const float2* A = reinterpret_cast<const float2*>(op.a) + oa;
-        const float2* B = reinterpret_cast<const float2*>(op.b) + ob;
-#pragma unroll 4
-        for (uint32_t k = idx & (L - 1); k < K; k += L) {
-          uint32_t ka = 0, kb = 0;
-          for (int j = 0; j < op.nk; ++j) {
-            const uint2 w = op.kbit[j];
-            if ((k >> j) & 1) {
-              ka |= w.x;
-              kb |= w.y;
-            }
+      for (int i0 = 0; i0 < iters; i0 += 32) {
+        uint32_t qa = 0, qb = 0;
+#pragma unroll
+        for (int j = 0; j < PROG_MAX_K; ++j)
+          if (j < kb_iter && (((i0 + lane) >> j) & 1)) {
+            const uint2 w = op.kbit[log_l + j];
+            qa |= w.x;
+            qb |= w.y;
           }
+        const int n = min(32, iters - i0);
+#pragma unroll 4
+        for (int i = 0; i < n; ++i) {
+          const uint32_t ka = __shfl_sync(0xffffffffu, qa, i), kb = __shfl_sync(0xffffffffu, qb, i);
           // plain loads: earlier levels of this launch may have written them
-          const float2 a = A[ka], b = B[kb];
-          re = fmaf(a.x, b.x, re);
-          re = fmaf(-a.y, b.y, re);
-          im = fmaf(a.x, b.y, im);
-          im = fmaf(a.y, b.x, im);
+          if (live) {
+            const float2 a = A[ka], b = B[kb];
+            re = fmaf(a.x, b.x, re);
+            re = fmaf(-a.y, b.y, re);
+            im = fmaf(a.x, b.y, im);
+            im = fmaf(a.y, b.x, im);
+          }
         }
       }
       for (uint32_t d = 1; d < L; d <<= 1) {
