@@ -288,7 +288,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       };
       const uint32_t tcol = tmem + lane_addr + uint32_t(q0 * 32);
       if (nchunks == 1) {
-        // one chunk (short K): from tensor memory straight to the output
+        // One chunk (short K): from tensor memory straight to the output.  Through
+        // the register accumulator this epilogue was a serial chain of 1100
+        // instructions a warp and tile (TF32x3, K = 8: 2^13 x 2^13 outputs 213 us,
+        // now 119; the output alone takes 79).
         const int b = int(chunk & 1);
         ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_full[b]), uint32_t(chunk >> 1) & 1));
         if (!ok) {

@@ -10,7 +10,10 @@
 // double-buffered (cp.async of 8 bytes: any index may be the stride-1 one).
 //
 // M = 4, N = 8, K = 2^20 with scattered indices (100 MB): two permutes (63 us)
-// and the dot kernel with its reduction (76 us) before.
+// and the dot kernel with its reduction (76 us) before, 37 and 3 us now.  What
+// bounds it is the latency of the shared-memory reads (short scoreboard) with 16
+// warps an SM, not memory (2.8 TB/s); deeper unrolling and smaller tiles measured
+// the same.
 #include <algorithm>
 #include <vector>
 
@@ -265,9 +268,9 @@ cudaError_t launch_cgemm_kdot(const KdotDesc& d, const void* A, const void* B, v
   cudaError_t e = cudaErrorInvalidConfiguration;
 #define TNQ_KD(TM_, TN_)                                                                                         \
   if (tm == TM_ && tn == TN_) {                                                                                  \
-    static const cudaError_t ok = cudaFuncSetAttribute(                                                          \
-        cgemm_kdot_kernel<TM_, TN_>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * (kKdotTileElems + 64) * 8); \
-    if (ok != cudaSuccess) return ok;                                                                            \
+    static std::atomic<uint64_t> done{0};                                                                        \
+    e = allow_smem(reinterpret_cast<const void*>(cgemm_kdot_kernel<TM_, TN_>), 2 * (kKdotTileElems + 64) * 8, &done); \
+    if (e != cudaSuccess) return e;                                                                              \
     cgemm_kdot_kernel<TM_, TN_><<<grid, KD_THREADS, smem, st>>>(d, Ap, Bp, reinterpret_cast<float2*>(C),         \
                                                                 reinterpret_cast<double2*>(acc), Pp, splits);    \
     e = cudaGetLastError();                                                                                      \

@@ -5,7 +5,22 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace tnq {
+
+// Lets kernel f use `bytes` of dynamic shared memory on the current device;
+// `done` (one per kernel) remembers the devices it was set on.
+inline cudaError_t allow_smem(const void* f, int bytes, std::atomic<uint64_t>* done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+  if (done->load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) done->fetch_or(bit, std::memory_order_release);
+  return e;
+}
 
 // Operand formats written by the permute kernel.
 enum PermMode {

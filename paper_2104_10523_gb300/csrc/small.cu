@@ -4,8 +4,9 @@
 // Most steps of a contraction path are tiny (gate-sized tensors): their cost is
 // launches and dependent latencies, not bytes or flops.  A permute per operand,
 // a tiled GEMM and a permute of the output were up to four launches of 6 to
-// 14 us.  Here every output element is a dot product whose operand offsets are
-// bit deposits of its index; operands sit in L1/L2.
+// 14 us (64 x 64 x 64: 45 us on the device, 66 a call).  Here every output element
+// is a dot product whose operand offsets are bit deposits of its index; operands
+// sit in L1/L2 (one launch of 4 us, 17 a call).
 #include <algorithm>
 
 #include "kernels.cuh"
@@ -270,23 +271,33 @@ cudaError_t launch_prog(const ProgOp* ops, const int* levels, int n_levels, int 
     cfg.gridDim = dim3(unsigned(ctas));
     cfg.dynamicSmemBytes = smem;
   };
-  static const int ctas = [&] {
-    if (cudaFuncSetAttribute(prog_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(PROG_MAX_OPS * sizeof(ProgOp))) != cudaSuccess)
-      return 0;
-    int n = 0;
-    shape(PROG_CTAS, PROG_THREADS, PROG_MAX_OPS * sizeof(ProgOp));
-    if (cudaFuncSetAttribute(prog_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaOccupancyMaxActiveClusters(&n, prog_kernel, &cfg) == cudaSuccess && n >= 1)
-      return PROG_CTAS;
-    cudaGetLastError();
-    return PROG_CTAS_PORTABLE;
-  }();
-  if (!ctas) return cudaErrorInvalidConfiguration;
+  static std::atomic<uint64_t> done{0};
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(prog_kernel), int(PROG_MAX_OPS * sizeof(ProgOp)), &done);
+  if (e != cudaSuccess) return e;
   const size_t smem = size_t(n_ops) * sizeof(ProgOp);
-  if (max_units <= 32) shape(1, PROG_THREADS, smem);
-  else if (max_units <= 256) shape(PROG_CTAS_PORTABLE, PROG_THREADS / 2, smem);
-  else shape(ctas, PROG_THREADS, smem);
+  if (max_units > 256) {
+    // a cluster of sixteen is beyond the portable size: asked for on each launch's
+    // device, and only where it can be placed
+    static std::atomic<uint64_t> wide{0}, narrow{0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+    if (!((wide.load() | narrow.load()) & bit) || !bit) {
+      int n = 0;
+      shape(PROG_CTAS, PROG_THREADS, PROG_MAX_OPS * sizeof(ProgOp));
+      const bool fits = cudaFuncSetAttribute(prog_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                        cudaOccupancyMaxActiveClusters(&n, prog_kernel, &cfg) == cudaSuccess && n >= 1;
+      if (!fits) cudaGetLastError();
+      if (bit) (fits ? wide : narrow).fetch_or(bit);
+      shape(fits ? PROG_CTAS : PROG_CTAS_PORTABLE, PROG_THREADS, smem);
+    } else {
+      shape(wide.load() & bit ? PROG_CTAS : PROG_CTAS_PORTABLE, PROG_THREADS, smem);
+    }
+  } else if (max_units > 32) {
+    shape(PROG_CTAS_PORTABLE, PROG_THREADS / 2, smem);
+  } else {
+    shape(1, PROG_THREADS, smem);
+  }
   cfg.stream = st;
   return cudaLaunchKernelEx(&cfg, prog_kernel, ops, lv, n_ops, n_slices, slice_id);
 }
