@@ -850,7 +850,7 @@ cudaError_t launch_tc_rows_one(const void* Ssmall, const SmallDesc& sd, const vo
   }
   const int ch = (two || P.kc <= 8) ? 8 : 16;
   P.nchunks = (P.kc + ch - 1) / ch;
-  P.pairs = gd.nk >= 1 && gd.kpos[0] == 0;
+  P.pairs = gd.nk >= 1 && gd.kpos[0] == 0 && (reinterpret_cast<uintptr_t>(Gsrc) & 15) == 0;
   P.row_tab = gd.nrow - 7 <= 4 * TR_ROWTAB_DIGITS ? 1 : 0;
   for (int j = 7; j < gd.nrow; ++j)
     if (gd.rowpos[j] >= 32) P.row_tab = 0;

@@ -96,6 +96,7 @@ struct GatherDesc {
   int kpos[8];
   int n_slice;
   int slice_src[32];
+  int pairs;  // set by launch_cgemm_rows_gather: K bit 0 is stored bit 0 of a 16-byte aligned operand
 };
 // Small operand read in place: bit j of its [K][rows][batch] index (K bits
 // lowest) sits at stored position pos[j].

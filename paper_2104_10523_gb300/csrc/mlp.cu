@@ -465,7 +465,7 @@ void CostModel::layout() {
   o_dz1 = take(4 * B * h);
   o_dz2 = take(4 * B * h);
   o_loss = take(8);
-  o_part = take(fused() ? 4 * (P + 1) * kGradSplits : 0);
+  o_part = take(fits_fused() ? 4 * (P + 1) * kGradSplits : 0);
   ws_bytes = off;
 }
 

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(T, gather_min_ctas(K, ROWS))
   for (int j = 0; (1 << j) < T; ++j)
     if (j < gd.nrow && ((t >> j) & 1)) lo |= size_t(1) << gd.rowpos[j];
   __syncthreads();
-  const bool pairs = K > 1 && gd.kpos[0] == 0;
+  const bool pairs = K > 1 && gd.pairs;
   for (int it = 0; it < reps; ++it) {
     const long long R0 = C0 + (long long)it * cta_rows;
     bool live[ROWS];
@@ -212,13 +212,15 @@ cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const SmallDesc& sd, co
   while (reps < GATHER_REPS && 2 * reps * cta_rows <= ng && total / (2 * reps * cta_rows) >= 16ll * std::max(1, sm_count))
     reps *= 2;
   const unsigned grid = unsigned(total / (cta_rows * reps));
+  GatherDesc g = gd;
+  g.pairs = gd.nk >= 1 && gd.kpos[0] == 0 && (reinterpret_cast<uintptr_t>(Gsrc) & 15) == 0;
   const float2* Sp = reinterpret_cast<const float2*>(Ssmall);
   const float2* Gp = reinterpret_cast<const float2*>(Gsrc);
   float2* Cp = reinterpret_cast<float2*>(C);
   double2* Ap = reinterpret_cast<double2*>(acc);
 #define TNQ_GATHER1(K_, R_, T_) \
   cgemm_rows_gather_kernel<K_, R_, T_, (K_ >= 16 && R_ == 2 ? 128 : 256)><<<grid, threads, smem, st>>>(       \
-      Sp, sd, Gp, gd, Cp, Ap, ns, log_per, log_ng, int(cta_rows), reps, entries, slice_id)
+      Sp, sd, Gp, g, Cp, Ap, ns, log_per, log_ng, int(cta_rows), reps, entries, slice_id)
 #define TNQ_GATHER(K_, R_)                   \
   do {                                       \
     if (round_tf32) TNQ_GATHER1(K_, R_, true); \

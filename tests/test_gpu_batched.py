@@ -71,3 +71,31 @@ def test_large_small_operand_is_permuted():
     """A small operand beyond 2^22 elements leaves the in-place read."""
     got, ref = contract("fp32", 1, 2, 2, 20, seed=3)
     assert rel(got, ref) <= TOL["fp32"], rel(got, ref)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "tf32x3"])
+@pytest.mark.parametrize("m,n,k", [(6, 14, 3), (3, 16, 3), (2, 3, 14), (4, 5, 4)])
+def test_operands_eight_byte_aligned(prec, m, n, k):
+    """Operands and output that start on an odd complex value: the kernels that
+    read them in place fall back to 8-byte accesses."""
+    import torch
+    from paper_2104_10523_gb300 import build, tnq as T
+    build.build()
+    rng = np.random.default_rng(m + n + k)
+    al, bl = list(range(k)) + list(range(100, 100 + m)), list(range(k)) + list(range(200, 200 + n))
+    ol = list(range(200, 200 + n)) + list(range(100, 100 + m))
+    A, B = ((rng.standard_normal(2 ** len(x)) + 1j * rng.standard_normal(2 ** len(x))).astype(np.complex64)
+            for x in (al, bl))
+
+    def odd(x):
+        t = torch.zeros(x.size + 1, dtype=torch.complex64, device="cuda")
+        t[1:] = torch.from_numpy(x).cuda()
+        return t[1:]
+
+    C = odd(np.zeros(2 ** len(ol), np.complex64))
+    ctx = T.Context(0, prec)
+    nb = T.tnq_contract_workspace_bytes(T.PRECISIONS[prec], len(al), len(bl), len(ol))
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    T.tnq_contract_pair(ctx.h, odd(A), al, odd(B), bl, C, ol, ws, nb)
+    got, ref = C.cpu().numpy(), contraction.contract_labeled(A, al, B, bl, ol)
+    assert rel(got, ref) <= TOL[prec], rel(got, ref)
