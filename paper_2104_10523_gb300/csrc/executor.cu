@@ -17,6 +17,7 @@
 #include "executor.h"
 #include "flags.h"
 #include "kernels.cuh"
+#include "rules.h"
 #include "gemm_tc.cuh"
 #include "traj.cuh"
 #include "splitk.h"
@@ -178,9 +179,10 @@ bool host_bits_ok(const Plan* p, int64_t n_bs, const int8_t* bits) {
   return true;
 }
 
-// Where a step's output goes when it may be written in another index order
-// than [N][M][H]: to C with index order `labels` (all of them), `done` telling
-// whether the step did so (else it wrote its own order to the step's C).
+// Output of a pairwise call: C with index order `labels` (all of them), which a
+// step may write itself in that order, `done` telling whether it did so (else it
+// wrote [N][M][H] to the step's C).  C is NULL where it overlaps an operand that
+// the step's kernels still read.
 struct DirectOut {
   void* C = nullptr;
   const std::vector<int>* labels = nullptr;
@@ -293,7 +295,7 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   const bool kdot = !small && !gather && !use_tc && use_kdot(nM, nN, nK) && part;
   signed char pos_c[32];  // positions in C of the output bits [N][M][H]
   for (int j = 0; j < nN + nM + nH && j < 32; ++j) pos_c[j] = (signed char)j;
-  if ((small || kdot) && direct) {
+  if ((small || kdot) && direct && direct->C) {
     for (int j = 0; j < nN + nM + nH; ++j) {
       const int l = j < nN ? b_req[nK + j] : a_req[nK + j - nN];
       pos_c[j] = (signed char)(std::find(direct->labels->begin(), direct->labels->end(), l) - direct->labels->begin());
@@ -1318,16 +1320,22 @@ tnq_status exec_contract_pair(Ctx* ctx, const void* A, int ra, const int* al, co
   const bool dev_flag = flagged && !slot.p;
   if (slot.p) err = slot.p + kFlagWait;
   if (dev_flag) TNQ_CUDA(cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
-  const bool direct = out == lc;
+  // An output that shares memory with an operand is written once the contraction
+  // has read them: through the scratch, whatever its order.
+  const size_t bytes_a = size_t(8) << ra, bytes_b = size_t(8) << rb, bytes_c = size_t(8) << rc;
+  const bool overlap = ranges_overlap(C, bytes_c, A, bytes_a) || ranges_overlap(C, bytes_c, B, bytes_b);
+  const bool ordered_out = out == lc, direct = ordered_out && !overlap;
   DirectOut dout;
-  dout.C = C;
+  dout.C = overlap ? nullptr : C;
   dout.labels = &lc;
   std::vector<int> none;
   tnq_status st = run_gemm_step(ctx, pa, xa, xa != a_req, pb, xb, xb != b_req, a_req, b_req, none, 0,
                                 (int)Hh.size(), (int)M.size(), (int)N.size(), (int)K.size(), sa, sb,
                                 direct ? C : (void*)sc, nullptr, err, part, size_t(sb - sa), -1, &dout);
   if (st != TNQ_OK) return st;
-  if (!direct && !dout.done) {
+  if (ordered_out && overlap) {
+    TNQ_CUDA(cudaMemcpyAsync(C, sc, bytes_c, cudaMemcpyDeviceToDevice, ctx->stream));
+  } else if (!direct && !dout.done) {
     PermDesc d;
     build_perm_desc(out.data(), (int)out.size(), lc.data(), rc, nullptr, 0, PM_C64, 0, &d);
     TNQ_CUDA(perm(ctx, d, sc, C, nullptr, 0, 16.0 * std::ldexp(1.0, rc)));

@@ -1,0 +1,15 @@
+// Host-side rules about the buffers a caller hands over (no CUDA in here).
+#pragma once
+
+#include <stddef.h>
+#include <stdint.h>
+
+namespace tnq {
+
+// Whether the n bytes at p and the m bytes at q share a byte.
+inline bool ranges_overlap(const void* p, size_t n, const void* q, size_t m) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(q);
+  return a < b ? b - a < n : a - b < m;
+}
+
+}  // namespace tnq

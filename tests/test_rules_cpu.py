@@ -1,0 +1,21 @@
+"""Rules of csrc/rules.h, compiled with the host compiler: no GPU, no CUDA."""
+import os
+import subprocess
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2104_10523_gb300", "csrc")
+
+
+def run(tmp_path, body, extra=()):
+    src = tmp_path / "t.cpp"
+    src.write_text('#include <cstdio>\n#include "rules.h"\nusing namespace tnq;\nint main() {\n%s\nreturn 0;\n}\n' % body)
+    exe = tmp_path / "t"
+    subprocess.run(["g++", "-std=c++17", "-Wall", "-Werror", "-I", CSRC, *extra, str(src), "-o", str(exe)], check=True)
+    return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
+
+
+def test_ranges_overlap(tmp_path):
+    cases = [(0, 8, 8, 8, 0), (8, 8, 0, 8, 0), (0, 9, 8, 8, 1), (8, 8, 0, 9, 1), (0, 64, 16, 8, 1), (16, 8, 0, 64, 1),
+             (0, 8, 0, 8, 1), (0, 8, 64, 8, 0)]
+    body = "\n".join(f'printf("%d\\n", ranges_overlap((void*){0x1000 + p}, {n}, (void*){0x1000 + q}, {m}));'
+                     for p, n, q, m, _ in cases)
+    assert run(tmp_path, body) == [str(c[4]) for c in cases]
