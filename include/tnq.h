@@ -15,7 +15,8 @@
  *     handles (tnq_circuit, tnq_plan, tnq_ctx) are owned by the library and
  *     released with the matching *_destroy call;
  *   - a buffer argument may be a host or a device pointer where the call
- *     says so; the library checks which with cudaPointerGetAttributes;
+ *     says so; the library checks which with cudaPointerGetAttributes
+ *     (device memory of another GPU than the context's is copied, not addressed);
  *   - device memory: the library allocates none on its own; every byte it
  *     uses on the GPU lives in the workspace the caller binds to a plan;
  *   - host memory: error flags sit in one 256 KB block of pinned memory, made

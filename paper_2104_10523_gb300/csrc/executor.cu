@@ -68,13 +68,19 @@ tnq_status timing_collect(Ctx* ctx) {
 
 namespace {
 
-bool is_device_ptr(const void* p) {
+// Where a caller's buffer lives: on some device (else the host reads and writes
+// it), and whether kernels of this context may address it.
+struct Where {
+  bool device = false, direct = false;
+};
+Where where(const Ctx* ctx, const void* p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return {};
   }
-  return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+  const bool dev = a.type == cudaMemoryTypeDevice, managed = a.type == cudaMemoryTypeManaged;
+  return {dev || managed, kernels_reach(dev, managed, a.device, ctx->device)};
 }
 
 int tc_mode_a(int prec) {
@@ -725,7 +731,7 @@ tnq_status exec_bind(Ctx* ctx, Plan* p, void* ws, size_t bytes) {
   if (!ws) return fail(TNQ_ERR_WORKSPACE, "workspace is NULL");
   if (bytes < p->ws_total)
     return fail(TNQ_ERR_WORKSPACE, "workspace too small: need " + std::to_string(p->ws_total) + " bytes");
-  if (!is_device_ptr(ws)) return fail(TNQ_ERR_WORKSPACE, "workspace must be device memory");
+  if (!where(ctx, ws).device) return fail(TNQ_ERR_WORKSPACE, "workspace must be device memory");
   TNQ_CUDA(cudaSetDevice(ctx->device));
   plan_release_graph(p);
   char* base = static_cast<char*>(ws);
@@ -801,8 +807,8 @@ tnq_status exec_amplitudes_range(Ctx* ctx, Plan* p, int64_t n_bs, const int8_t* 
   const int64_t per = int64_t(1) << w;
   const int64_t n_out = int64_t(1) << p->net.open_qubits.size();  // amplitudes per bitstring
   const int64_t vals = p->density ? 1 : 2;                          // doubles per result
-  const bool bits_dev = is_device_ptr(bits), out_dev = is_device_ptr(out);
-  if (!bits_dev && !host_bits_ok(p, n_bs, bits))
+  const Where bits_at = where(ctx, bits), out_at = where(ctx, out);
+  if (!bits_at.device && !host_bits_ok(p, n_bs, bits))
     return fail(TNQ_ERR_INVALID_ARG, p->net.open_qubits.empty()
                                          ? "bitstring entries must be 0 or 1"
                                          : "bitstring entries must be -1 at the plan's open qubits and 0 or 1 elsewhere");
@@ -816,17 +822,17 @@ tnq_status exec_amplitudes_range(Ctx* ctx, Plan* p, int64_t n_bs, const int8_t* 
     return fail(TNQ_ERR_INVALID_ARG, "slice range outside [0, 2^n_sliced)");
   // the captured graph covers every slice; partial ranges launch directly
   const bool graphs = ctx->use_graphs && !ctx->timing && slice_begin == 0 && slice_count == n_slices;
-  // results are written where the caller wants them when that is device memory
-  // the kernel's 16-byte (complex) or 8-byte stores can address
-  const bool out_direct = out_dev && reinterpret_cast<uintptr_t>(out) % (p->density ? 8 : 16) == 0;
+  // results are written where the caller wants them when that is memory the
+  // kernel's 16-byte (complex) or 8-byte stores can address
+  const bool out_direct = out_at.direct && reinterpret_cast<uintptr_t>(out) % (p->density ? 8 : 16) == 0;
   auto enqueue = [&]() -> tnq_status {
     tnq_status st = ensure_folded(ctx, p);
     if (st != TNQ_OK) return st;
     for (int64_t base = 0; base < n_bs; base += per) {
       int64_t nv = std::min<int64_t>(per, n_bs - base);
-      const int8_t* bsrc = bits_dev ? bits + base * rl : bits_stage;
-      if (!bits_dev)
-        TNQ_CUDA(cudaMemcpyAsync(bits_stage, bits + base * rl, size_t(nv) * rl, cudaMemcpyHostToDevice, ctx->stream));
+      const int8_t* bsrc = bits_at.direct ? bits + base * rl : bits_stage;
+      if (!bits_at.direct)
+        TNQ_CUDA(cudaMemcpyAsync(bits_stage, bits + base * rl, size_t(nv) * rl, cudaMemcpyDefault, ctx->stream));
       TNQ_CUDA(fill_projections(ctx, pl, w, bsrc, nv, p->flags + kFlagInput));
       if (graphs) {
         st = ensure_graph(ctx, p);
@@ -842,8 +848,7 @@ tnq_status exec_amplitudes_range(Ctx* ctx, Plan* p, int64_t n_bs, const int8_t* 
                                (int)opos.size(), p->density, ctx->stream));
       ctx->launches++;
       if (!out_direct)
-        TNQ_CUDA(cudaMemcpyAsync(user, out_stage, size_t(nv * n_out * vals) * 8,
-                                 out_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, ctx->stream));
+        TNQ_CUDA(cudaMemcpyAsync(user, out_stage, size_t(nv * n_out * vals) * 8, cudaMemcpyDefault, ctx->stream));
     }
     TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
     return TNQ_OK;
@@ -1000,8 +1005,8 @@ tnq_status noisy_driver(Ctx* ctx, Plan* p, int64_t traj_begin, int64_t n_traj, u
   char* ws = static_cast<char*>(p->bound_ws);
   const int n = p->net.row_len, w = p->batch_log2, t = p->traj_log2;
   const int64_t per = int64_t(1) << w, tper = int64_t(1) << t;
-  const bool bits_dev = is_device_ptr(bits);
-  if (!bits_dev && !host_bits_ok(p, n_bs, bits))
+  const Where bits_at = where(ctx, bits);
+  if (!bits_at.device && !host_bits_ok(p, n_bs, bits))
     return fail(TNQ_ERR_INVALID_ARG, "bitstring entries must be 0 or 1");
   int8_t* bits_stage = reinterpret_cast<int8_t*>(ws + p->ws_bits);
   const ProjLeaves pl = proj_leaves(p, ws);
@@ -1018,10 +1023,10 @@ tnq_status noisy_driver(Ctx* ctx, Plan* p, int64_t traj_begin, int64_t n_traj, u
   for (int64_t base = 0; base < n_bs; base += per) {
     const int64_t nv = std::min<int64_t>(per, n_bs - base);
     const int8_t* bsrc;
-    if (bits_dev) {
+    if (bits_at.direct) {
       bsrc = bits + base * n;
     } else {
-      TNQ_CUDA(cudaMemcpyAsync(bits_stage, bits + base * n, size_t(nv) * n, cudaMemcpyHostToDevice, ctx->stream));
+      TNQ_CUDA(cudaMemcpyAsync(bits_stage, bits + base * n, size_t(nv) * n, cudaMemcpyDefault, ctx->stream));
       bsrc = bits_stage;
     }
     TNQ_CUDA(fill_projections(ctx, pl, w, bsrc, nv, p->flags + kFlagInput));
@@ -1094,7 +1099,7 @@ tnq_status exec_noisy(Ctx* ctx, Plan* p, int64_t n_traj, uint64_t seed, int64_t 
   double* p2sum = reinterpret_cast<double*>(ws + p->ws_p2sum);
   double* stage = reinterpret_cast<double*>(ws + p->ws_out_stage);
   const int64_t per = int64_t(1) << p->batch_log2;
-  const bool p_dev = is_device_ptr(p_out), se_dev = se_out && is_device_ptr(se_out);
+  const bool p_direct = where(ctx, p_out).direct, se_direct = se_out && where(ctx, se_out).direct;
   auto consume = [&](int phase, int64_t, int64_t nv, int64_t, int64_t nt, const std::vector<int>& bpos,
                      const std::vector<int>& tpos) -> tnq_status {
     if (phase < 0) {
@@ -1109,14 +1114,14 @@ tnq_status exec_noisy(Ctx* ctx, Plan* p, int64_t n_traj, uint64_t seed, int64_t 
     return TNQ_OK;
   };
   auto batch_end = [&](int64_t base, int64_t nv) -> tnq_status {
-    double* pd = p_dev ? p_out + base : stage;
-    double* sd = se_out ? (se_dev ? se_out + base : stage + per) : nullptr;
+    double* pd = p_direct ? p_out + base : stage;
+    double* sd = se_out ? (se_direct ? se_out + base : stage + per) : nullptr;
     TNQ_CUDA(launch_noisy_finalize(psum, p2sum, nv, n_traj, pd, sd, ctx->stream));
     ctx->launches++;
-    if (!p_dev) TNQ_CUDA(cudaMemcpyAsync(p_out + base, stage, 8 * nv, cudaMemcpyDeviceToHost, ctx->stream));
-    if (se_out && !se_dev)
-      TNQ_CUDA(cudaMemcpyAsync(se_out + base, stage + per, 8 * nv, cudaMemcpyDeviceToHost, ctx->stream));
-    if (!p_dev || (se_out && !se_dev)) TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (!p_direct) TNQ_CUDA(cudaMemcpyAsync(p_out + base, stage, 8 * nv, cudaMemcpyDefault, ctx->stream));
+    if (se_out && !se_direct)
+      TNQ_CUDA(cudaMemcpyAsync(se_out + base, stage + per, 8 * nv, cudaMemcpyDefault, ctx->stream));
+    if (!p_direct || (se_out && !se_direct)) TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
     return TNQ_OK;
   };
   // identical trajectories (most draws pick the identity-like operator A_0)
@@ -1139,16 +1144,17 @@ tnq_status exec_traj_amplitudes(Ctx* ctx, Plan* p, uint64_t seed, int64_t traj_b
   if (traj_begin < 0) return fail(TNQ_ERR_INVALID_ARG, "traj_begin must be >= 0");
   TNQ_CUDA(cudaSetDevice(ctx->device));
   char* ws = static_cast<char*>(p->bound_ws);
-  const bool out_dev = is_device_ptr(out);
+  const bool out_direct = where(ctx, out).direct;
   const int64_t per = int64_t(1) << p->batch_log2;
   double2* stage = reinterpret_cast<double2*>(ws + p->ws_out_stage);
-  // Device output: one kernel writes the chunk.  Host output: the staging area
-  // holds 2^batch_log2 complex values, so each trajectory row goes through it.
+  // Output the kernels can address: one of them writes the chunk.  Otherwise
+  // (host memory, another GPU) each trajectory row goes through the staging area,
+  // which holds 2^batch_log2 complex values.
   auto consume = [&](int phase, int64_t base, int64_t nv, int64_t tb, int64_t nt, const std::vector<int>& bpos,
                      const std::vector<int>& tpos) -> tnq_status {
     if (phase < 0) return TNQ_OK;
     double2* o = reinterpret_cast<double2*>(out);
-    if (out_dev) {
+    if (out_direct) {
       TNQ_CUDA(launch_traj_amplitudes_out(ws + p->ws_acc, nv, 0, nt, bpos.data(), (int)bpos.size(), tpos.data(),
                                           (int)tpos.size(), o + tb * n_bs + base, n_bs, ctx->stream));
       ctx->launches++;
@@ -1158,8 +1164,7 @@ tnq_status exec_traj_amplitudes(Ctx* ctx, Plan* p, uint64_t seed, int64_t traj_b
       TNQ_CUDA(launch_traj_amplitudes_out(ws + p->ws_acc, nv, j, 1, bpos.data(), (int)bpos.size(), tpos.data(),
                                           (int)tpos.size(), stage, per, ctx->stream));
       ctx->launches++;
-      TNQ_CUDA(cudaMemcpyAsync(o + (tb + j) * n_bs + base, stage, 16 * size_t(nv), cudaMemcpyDeviceToHost,
-                               ctx->stream));
+      TNQ_CUDA(cudaMemcpyAsync(o + (tb + j) * n_bs + base, stage, 16 * size_t(nv), cudaMemcpyDefault, ctx->stream));
       TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
     }
     return TNQ_OK;

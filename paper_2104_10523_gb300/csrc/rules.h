@@ -12,4 +12,11 @@ inline bool ranges_overlap(const void* p, size_t n, const void* q, size_t m) {
   return a < b ? b - a < n : a - b < m;
 }
 
+// Whether kernels on device ctx_device may address caller memory of the given
+// kind (device memory of `device`, managed, or neither: host).  Memory of another
+// GPU is only copied: peer access may be off.
+inline bool kernels_reach(bool device_memory, bool managed, int device, int ctx_device) {
+  return managed || (device_memory && device == ctx_device);
+}
+
 }  // namespace tnq

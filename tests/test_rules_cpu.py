@@ -19,3 +19,18 @@ def test_ranges_overlap(tmp_path):
     body = "\n".join(f'printf("%d\\n", ranges_overlap((void*){0x1000 + p}, {n}, (void*){0x1000 + q}, {m}));'
                      for p, n, q, m, _ in cases)
     assert run(tmp_path, body) == [str(c[4]) for c in cases]
+
+
+def test_kernels_reach_own_device_and_managed_memory_only(tmp_path):
+    """Device memory of another GPU is not addressed from kernels, host memory neither."""
+    cases = [(1, 0, 0, 0, 1), (1, 0, 1, 1, 1), (1, 0, 1, 0, 0), (1, 0, 0, 1, 0), (0, 1, 0, 1, 1), (0, 0, 0, 0, 0)]
+    body = "\n".join(f'printf("%d\\n", kernels_reach({d}, {m}, {at}, {ctx}));' for d, m, at, ctx, _ in cases)
+    assert run(tmp_path, body) == [str(c[4]) for c in cases]
+
+
+def test_buffers_are_asked_for_the_context_device():
+    """Every caller buffer that kernels may address is classified by its device
+    against the context's, not by being device memory alone."""
+    src = open(os.path.join(CSRC, "executor.cu")).read()
+    assert "kernels_reach(dev, managed, a.device, ctx->device)" in src
+    assert src.count("cudaPointerGetAttributes") == 1 and "is_device_ptr" not in src
