@@ -20,7 +20,9 @@
  *   - device memory: the library allocates none on its own; every byte it
  *     uses on the GPU lives in the workspace the caller binds to a plan;
  *   - host memory: error flags sit in one 256 KB block of pinned memory, made
- *     by the first call that needs one and kept until the process exits;
+ *     by the first call that needs one and kept until the process exits; beyond
+ *     4096 bound plans, or where no memory can be pinned, they sit in the
+ *     workspace, at the cost of a clear and a small copy per call;
  *   - calls never throw; on failure they return a status other than TNQ_OK
  *     and leave a message for tnq_last_error();
  *   - GPU calls are ordered on the context's stream and return after the

@@ -506,6 +506,25 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   return TNQ_OK;
 }
 
+// Error flags of a plan's kernels: its slot of mapped host memory, or two ints of
+// its workspace where no slot was to be had when it was bound.
+int* plan_flags(const Plan* p, char* ws) { return p->flags ? p->flags : reinterpret_cast<int*>(ws + p->ws_misc); }
+
+// Reads and clears them once the stream is idle.
+tnq_status take_flags(Ctx* ctx, Plan* p, FlagValues* f) {
+  if (p->flags) {
+    *f = flags_take(p->flags);
+    return TNQ_OK;
+  }
+  int* dev = plan_flags(p, static_cast<char*>(p->bound_ws));
+  int v[2] = {0, 0};
+  TNQ_CUDA(cudaMemcpyAsync(v, dev, sizeof(v), cudaMemcpyDeviceToHost, ctx->stream));
+  TNQ_CUDA(cudaMemsetAsync(dev, 0, sizeof(v), ctx->stream));
+  TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
+  *f = FlagValues{v[kFlagInput], v[kFlagWait]};
+  return TNQ_OK;
+}
+
 tnq_status run_step(Ctx* ctx, Plan* p, size_t si, int slice_id, char* ws, int choice) {
   static const std::vector<int> kNoSlices;
   auto& s = p->steps[si];
@@ -517,7 +536,7 @@ tnq_status run_step(Ctx* ctx, Plan* p, size_t si, int slice_id, char* ws, int ch
   const std::vector<int>& sl = s.sliced_batch ? kNoSlices : p->slice_labels;
   return run_gemm_step(ctx, ws + ta.offset, ta.labels, s.perm_a, ws + tb.offset, tb.labels, s.perm_b, s.a_req,
                        s.b_req, sl, s.sliced_batch ? 0 : slice_id, s.nH, s.nM, s.nN, s.nK, ws + p->ws_scratch_a,
-                       ws + p->ws_scratch_b, C, acc, p->flags + kFlagWait,
+                       ws + p->ws_scratch_b, C, acc, plan_flags(p, ws) + kFlagWait,
                        ws + p->ws_partial, p->ws_scratch_b - p->ws_scratch_a, choice);
 }
 
@@ -678,8 +697,10 @@ tnq_status enqueue_slices(Ctx* ctx, Plan* p, int64_t slice_begin, int64_t slice_
 // Kernels of an abandoned call may still run and raise the plan's flags: wait
 // for them, so that the next call starts with flags of its own.
 tnq_status abandon(Ctx* ctx, Plan* p, tnq_status st) {
+  const std::string why = tnq_last_error();
+  FlagValues f;
   cudaStreamSynchronize(ctx->stream);
-  if (p->flags) flags_take(p->flags);
+  if (take_flags(ctx, p, &f) != TNQ_OK) fail(st, why);  // the first error stands
   return st;
 }
 
@@ -778,8 +799,11 @@ tnq_status exec_bind(Ctx* ctx, Plan* p, void* ws, size_t bytes) {
       TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
     }
   }
-  if (!p->flags && !(p->flags = flags_get()))
-    return fail(TNQ_ERR_CUDA, "no mapped host memory for the plan's error flags");
+  if (!p->flags) p->flags = flags_get();
+  if (!p->flags) {
+    TNQ_CUDA(cudaMemsetAsync(plan_flags(p, base), 0, 2 * sizeof(int), ctx->stream));
+    TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
+  }
   {
     tnq_status st = upload_programs(ctx, p, base);
     if (st != TNQ_OK) return st;
@@ -833,7 +857,7 @@ tnq_status exec_amplitudes_range(Ctx* ctx, Plan* p, int64_t n_bs, const int8_t* 
       const int8_t* bsrc = bits_at.direct ? bits + base * rl : bits_stage;
       if (!bits_at.direct)
         TNQ_CUDA(cudaMemcpyAsync(bits_stage, bits + base * rl, size_t(nv) * rl, cudaMemcpyDefault, ctx->stream));
-      TNQ_CUDA(fill_projections(ctx, pl, w, bsrc, nv, p->flags + kFlagInput));
+      TNQ_CUDA(fill_projections(ctx, pl, w, bsrc, nv, plan_flags(p, ws) + kFlagInput));
       if (graphs) {
         st = ensure_graph(ctx, p);
         if (st != TNQ_OK) return st;
@@ -855,7 +879,8 @@ tnq_status exec_amplitudes_range(Ctx* ctx, Plan* p, int64_t n_bs, const int8_t* 
   };
   tnq_status st = enqueue();
   if (st != TNQ_OK) return abandon(ctx, p, st);
-  const FlagValues herr = flags_take(p->flags);
+  FlagValues herr;
+  if (tnq_status fs = take_flags(ctx, p, &herr); fs != TNQ_OK) return fs;
   if (ctx->timing) {
     tnq_status ts = timing_collect(ctx);
     if (ts != TNQ_OK) return ts;
@@ -936,7 +961,9 @@ tnq_status exec_autotune(Ctx* ctx, Plan* p, int reps, int* n_tc, int* n_cuda) {
   cudaEventDestroy(e1);
   if (result != TNQ_OK) return abandon(ctx, p, result);
   TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
-  if (flags_take(p->flags).wait) return fail(TNQ_ERR_TIMEOUT, "a tensor-core GEMM wait expired during autotuning");
+  FlagValues herr;
+  if (tnq_status fs = take_flags(ctx, p, &herr); fs != TNQ_OK) return fs;
+  if (herr.wait) return fail(TNQ_ERR_TIMEOUT, "a tensor-core GEMM wait expired during autotuning");
   p->kernel_choice = choice;
   p->tuned_precision = ctx->precision;
   p->folded_precision = -1;  // the timing runs overwrote the folded outputs
@@ -1029,7 +1056,7 @@ tnq_status noisy_driver(Ctx* ctx, Plan* p, int64_t traj_begin, int64_t n_traj, u
       TNQ_CUDA(cudaMemcpyAsync(bits_stage, bits + base * n, size_t(nv) * n, cudaMemcpyDefault, ctx->stream));
       bsrc = bits_stage;
     }
-    TNQ_CUDA(fill_projections(ctx, pl, w, bsrc, nv, p->flags + kFlagInput));
+    TNQ_CUDA(fill_projections(ctx, pl, w, bsrc, nv, plan_flags(p, ws) + kFlagInput));
     tnq_status st = consume(-1, base, nv, 0, 0, bpos, tpos);  // batch start
     if (st != TNQ_OK) return st;
     const int64_t units = distinct ? int64_t(mult->size()) : n_traj;
@@ -1068,7 +1095,8 @@ tnq_status noisy_driver(Ctx* ctx, Plan* p, int64_t traj_begin, int64_t n_traj, u
     if (st != TNQ_OK) return st;
   }
   TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
-  const FlagValues herr = flags_take(p->flags);
+  FlagValues herr;
+  if (tnq_status fs = take_flags(ctx, p, &herr); fs != TNQ_OK) return fs;
   if (ctx->timing) {
     tnq_status ts = timing_collect(ctx);
     if (ts != TNQ_OK) return ts;
@@ -1191,7 +1219,7 @@ static tnq_status run_expectation(Ctx* ctx, Plan* p, const double* coeffs, doubl
   const int n_slices = 1 << p->slice_labels.size();
   // <0...0| closes every wire (the network is U, the Pauli operators, U^dagger)
   TNQ_CUDA(cudaMemsetAsync(bits_stage, 0, size_t(p->net.row_len), ctx->stream));
-  TNQ_CUDA(fill_projections(ctx, proj_leaves(p, ws), 0, bits_stage, 1, p->flags + kFlagInput));
+  TNQ_CUDA(fill_projections(ctx, proj_leaves(p, ws), 0, bits_stage, 1, plan_flags(p, ws) + kFlagInput));
   {
     tnq_status st = ensure_folded(ctx, p);
     if (st != TNQ_OK) return st;
@@ -1227,7 +1255,8 @@ static tnq_status run_expectation(Ctx* ctx, Plan* p, const double* coeffs, doubl
     }
   }
   TNQ_CUDA(cudaStreamSynchronize(ctx->stream));
-  const FlagValues herr = flags_take(p->flags);
+  FlagValues herr;
+  if (tnq_status fs = take_flags(ctx, p, &herr); fs != TNQ_OK) return fs;
   if (ctx->timing) {
     tnq_status ts = timing_collect(ctx);
     if (ts != TNQ_OK) return ts;

@@ -231,8 +231,9 @@ struct Plan {
   int graph_policy = -1;          // kernel policy the graph was captured with
   double graph_capture_ms = 0;
   int64_t graph_nodes = 0;
-  // device binding; error flags of the plan's kernels (mapped host memory, held
-  // from the first binding on: captured graphs name them)
+  // device binding; error flags of the plan's kernels (a slot of mapped host memory,
+  // held from the first binding on: captured graphs name it; NULL: two ints at
+  // ws_misc, where every slot was taken or no host memory could be pinned)
   int* flags = nullptr;
   void* bound_ws = nullptr;
   size_t bound_bytes = 0;
