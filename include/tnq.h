@@ -293,11 +293,12 @@ tnq_status tnq_trajectory_amplitudes(tnq_ctx* ctx, tnq_plan* p, uint64_t seed, i
  * tensors A (rank ra, labels a_labels) and B (rank rb, labels b_labels) into
  * C (rank rc, labels c_labels): C = sum over the labels A and B share but C
  * lacks of A*B.  Labels shared by A, B and C are batch indices.  A, B, C:
- * device complex64; C may share memory with A or B (a gate applied in place):
+ * device complex64, 8-byte aligned; C may share memory with A or B (a gate applied in place):
  * the result then reaches C through the workspace, after both have been read.
  * workspace: device scratch of at least
  * tnq_contract_workspace_bytes(...) bytes.  Uses the context's precision.
- * Errors: INVALID_ARG (label sets inconsistent, rank > 31), WORKSPACE, CUDA. */
+ * Errors: INVALID_ARG (label sets inconsistent, rank > 31, an operand or the
+ * output not 8-byte aligned), WORKSPACE, CUDA. */
 size_t tnq_contract_workspace_bytes(int precision, int ra, int rb, int rc);
 tnq_status tnq_contract_pair(tnq_ctx* ctx, const void* A, int ra, const int* a_labels,
                              const void* B, int rb, const int* b_labels, void* C, int rc,

@@ -459,7 +459,7 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   TNQ_CUDA(perm(ctx, d, a_src, scratch_a, a1, slice_id, 8.0 * na + a_half_bytes(prec, na) * (prec == TNQ_PREC_TF32 ? 1 : 2)));
   op.a0 = scratch_a;
   op.a1 = prec == TNQ_PREC_TF32 ? nullptr : a1;
-  if (prec == TNQ_PREC_TF32 && !perm_b) {
+  if (prec == TNQ_PREC_TF32 && !perm_b && aligned(16, b_src)) {  // (a tensor map's base is 16-byte aligned)
     op.b0 = b_src;
   } else {
     build_perm_desc(b_labels.data(), (int)b_labels.size(), b_req.data(), (int)b_req.size(), slice_labels.data(),
@@ -848,7 +848,7 @@ tnq_status exec_amplitudes_range(Ctx* ctx, Plan* p, int64_t n_bs, const int8_t* 
   const bool graphs = ctx->use_graphs && !ctx->timing && slice_begin == 0 && slice_count == n_slices;
   // results are written where the caller wants them when that is memory the
   // kernel's 16-byte (complex) or 8-byte stores can address
-  const bool out_direct = out_at.direct && reinterpret_cast<uintptr_t>(out) % (p->density ? 8 : 16) == 0;
+  const bool out_direct = out_at.direct && aligned(p->density ? 8 : 16, out);
   auto enqueue = [&]() -> tnq_status {
     tnq_status st = ensure_folded(ctx, p);
     if (st != TNQ_OK) return st;
@@ -1127,7 +1127,8 @@ tnq_status exec_noisy(Ctx* ctx, Plan* p, int64_t n_traj, uint64_t seed, int64_t 
   double* p2sum = reinterpret_cast<double*>(ws + p->ws_p2sum);
   double* stage = reinterpret_cast<double*>(ws + p->ws_out_stage);
   const int64_t per = int64_t(1) << p->batch_log2;
-  const bool p_direct = where(ctx, p_out).direct, se_direct = se_out && where(ctx, se_out).direct;
+  const bool p_direct = where(ctx, p_out).direct && aligned(8, p_out);
+  const bool se_direct = se_out && where(ctx, se_out).direct && aligned(8, se_out);
   auto consume = [&](int phase, int64_t, int64_t nv, int64_t, int64_t nt, const std::vector<int>& bpos,
                      const std::vector<int>& tpos) -> tnq_status {
     if (phase < 0) {
@@ -1172,11 +1173,11 @@ tnq_status exec_traj_amplitudes(Ctx* ctx, Plan* p, uint64_t seed, int64_t traj_b
   if (traj_begin < 0) return fail(TNQ_ERR_INVALID_ARG, "traj_begin must be >= 0");
   TNQ_CUDA(cudaSetDevice(ctx->device));
   char* ws = static_cast<char*>(p->bound_ws);
-  const bool out_direct = where(ctx, out).direct;
+  const bool out_direct = where(ctx, out).direct && aligned(16, out);
   const int64_t per = int64_t(1) << p->batch_log2;
   double2* stage = reinterpret_cast<double2*>(ws + p->ws_out_stage);
-  // Output the kernels can address: one of them writes the chunk.  Otherwise
-  // (host memory, another GPU) each trajectory row goes through the staging area,
+  // Output the kernels can address: one of them writes the chunk.  Otherwise (host
+  // memory, another GPU, a start that is not 16-byte aligned) each trajectory row goes through the staging area,
   // which holds 2^batch_log2 complex values.
   auto consume = [&](int phase, int64_t base, int64_t nv, int64_t tb, int64_t nt, const std::vector<int>& bpos,
                      const std::vector<int>& tpos) -> tnq_status {
@@ -1306,6 +1307,7 @@ tnq_status exec_contract_pair(Ctx* ctx, const void* A, int ra, const int* al, co
     if (!has(lb, l) && !has(lc, l)) return fail(TNQ_ERR_INVALID_ARG, "label of A neither shared nor kept");
   for (int l : lb)
     if (!has(la, l) && !has(lc, l)) return fail(TNQ_ERR_INVALID_ARG, "label of B neither shared nor kept");
+  if (!aligned(8, A, B, C)) return fail(TNQ_ERR_INVALID_ARG, "A, B and C must be 8-byte aligned");
   if (!ws || ws_bytes < contract_workspace_bytes(ctx->precision, ra, rb, rc))
     return fail(TNQ_ERR_WORKSPACE, "workspace too small for tnq_contract_pair");
   TNQ_CUDA(cudaSetDevice(ctx->device));

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "kernels.cuh"
+#include "rules.h"
 
 namespace tnq {
 
@@ -365,9 +366,11 @@ __global__ void __launch_bounds__(PV_THREADS) permute_vec_kernel(const PermDesc 
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-bool perm_vec_ok(const PermDesc& d) {
-  // pairs: source bit 0 and destination bit 0 are both the tile's first bit,
-  // and A' expansions keep a pair inside one row (at least two K elements)
+bool perm_vec_ok(const PermDesc& d, const void* src, const void* dst0, const void* dst1) {
+  // pairs: source bit 0 and destination bit 0 are both the tile's first bit, both
+  // sides 16-byte aligned (a caller's tensor need not be), and A' expansions keep
+  // a pair inside one row (at least two K elements)
+  if (!aligned(16, src, dst0, dst1)) return false;
   if (d.u < 2 || d.tile_src[0] != 0 || d.tile_dst_sorted[0] != 0) return false;
   if (d.mode >= PM_AEXP_F32 && d.mode <= PM_AEXP_BF16X3 && d.kbits < 1) return false;
   return true;
@@ -376,7 +379,7 @@ bool perm_vec_ok(const PermDesc& d) {
 cudaError_t launch_permute(const PermDesc& d, const void* src, void* dst0, void* dst1, int slice_id,
                            int sm_count, cudaStream_t st) {
   size_t n_outer = size_t(1) << d.n_outer;
-  if (perm_vec_ok(d)) {
+  if (perm_vec_ok(d, src, dst0, dst1)) {
     // persistent CTAs: as many as are resident at once
     static int per_sm = 0;
     if (per_sm == 0) {

@@ -19,4 +19,12 @@ inline bool kernels_reach(bool device_memory, bool managed, int device, int ctx_
   return managed || (device_memory && device == ctx_device);
 }
 
+// Whether every address is a multiple of n.  Complex64 tensors of a caller are
+// 8-byte aligned and no more (a slice may start at an odd element): 16-byte
+// accesses and tensor maps ask first.
+template <typename... P>
+bool aligned(size_t n, const P*... p) {
+  return (... && (reinterpret_cast<uintptr_t>(p) % n == 0));
+}
+
 }  // namespace tnq

@@ -34,3 +34,23 @@ def test_buffers_are_asked_for_the_context_device():
     src = open(os.path.join(CSRC, "executor.cu")).read()
     assert "kernels_reach(dev, managed, a.device, ctx->device)" in src
     assert src.count("cudaPointerGetAttributes") == 1 and "is_device_ptr" not in src
+
+
+def test_aligned(tmp_path):
+    cases = [(16, (0x1000, 0x2000, 0), 1), (16, (0x1008, 0x2000, 0), 0), (16, (0x1000, 0x2008, 0), 0),
+             (16, (0x1000, 0x2000, 0x3008), 0), (8, (0x1008, 0x2000, 0x3010), 1), (8, (0x1004, 0x2000, 0), 0)]
+    body = "\n".join('printf("%%d\\n", aligned(%d, (void*)%d, (void*)%d, (void*)%d));' % (n, *p) for n, p, _ in cases)
+    assert run(tmp_path, body) == [str(c[2]) for c in cases]
+
+
+def test_sixteen_byte_accesses_to_caller_tensors_ask_first():
+    """The vectorised permute and the tensor map over an operand read in place are
+    the two places a caller's A, B or C meets accesses wider than 8 bytes beside
+    the pair loads of the gather and tall-skinny kernels."""
+    def src(name):
+        return open(os.path.join(CSRC, name)).read()
+
+    assert "if (!aligned(16, src, dst0, dst1)) return false;" in src("kernels.cu")
+    assert "!perm_b && aligned(16, b_src)" in src("executor.cu")
+    for name in ("skinny.cu", "gemm_tc_rows.cu"):
+        assert "(reinterpret_cast<uintptr_t>(Gsrc) & 15) == 0" in src(name)
