@@ -18,7 +18,8 @@
  *     says so; the library checks which with cudaPointerGetAttributes
  *     (device memory of another GPU than the context's is copied, not addressed);
  *   - device memory: the library allocates none on its own; every byte it
- *     uses on the GPU lives in the workspace the caller binds to a plan;
+ *     uses on the GPU lives in the workspace the caller binds to a plan (which
+ *     may start at any address: the sizes asked for hold its alignment);
  *   - host memory: error flags sit in one 256 KB block of pinned memory, made
  *     by the first call that needs one and kept until the process exits; beyond
  *     4096 bound plans, or where no memory can be pinned, they sit in the

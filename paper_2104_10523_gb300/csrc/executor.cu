@@ -755,7 +755,7 @@ tnq_status exec_bind(Ctx* ctx, Plan* p, void* ws, size_t bytes) {
   if (!where(ctx, ws).device) return fail(TNQ_ERR_WORKSPACE, "workspace must be device memory");
   TNQ_CUDA(cudaSetDevice(ctx->device));
   plan_release_graph(p);
-  char* base = static_cast<char*>(ws);
+  char* base = workspace_base(ws);
   std::vector<float> buf;
   for (size_t i = 0; i < p->net.leaves.size(); ++i) {
     const Leaf& L = p->net.leaves[i];
@@ -808,8 +808,8 @@ tnq_status exec_bind(Ctx* ctx, Plan* p, void* ws, size_t bytes) {
     tnq_status st = upload_programs(ctx, p, base);
     if (st != TNQ_OK) return st;
   }
-  p->bound_ws = ws;
-  p->bound_bytes = bytes;
+  p->bound_ws = base;
+  p->bound_bytes = bytes - size_t(base - static_cast<char*>(ws));
   p->folded_precision = -1;
   return TNQ_OK;
 }
@@ -1286,6 +1286,9 @@ static size_t partial_bound(int rc) {
 size_t contract_workspace_bytes(int precision, int ra, int rb, int rc) {
   (void)precision;
   size_t na = size_t(1) << std::max(ra, rb), nb = na;
+  // three regions rounded up to 4096 bytes, the flag's, and the bytes in front of
+  // an aligned base
+  static_assert(kWorkspaceAlign <= 4096, "the fifth unit covers the base's alignment");
   return 32 * na + 16 * nb + 8 * (size_t(1) << rc) + partial_bound(rc) + 5 * 4096;
 }
 
@@ -1331,7 +1334,7 @@ tnq_status exec_contract_pair(Ctx* ctx, const void* A, int ra, const int* al, co
   b_req.insert(b_req.end(), Hh.begin(), Hh.end());
   out.insert(out.end(), M.begin(), M.end());
   out.insert(out.end(), Hh.begin(), Hh.end());
-  char* w = static_cast<char*>(ws);
+  char* w = workspace_base(ws);
   size_t na = size_t(1) << std::max(ra, rb);
   char* sa = w;
   char* sb = w + ((32 * na + 4095) & ~size_t(4095));

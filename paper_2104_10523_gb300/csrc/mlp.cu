@@ -19,6 +19,7 @@
 
 #include "executor.h"
 #include "mlp.h"
+#include "rules.h"
 
 namespace tnq {
 
@@ -465,8 +466,8 @@ void CostModel::layout() {
   o_dz1 = take(4 * B * h);
   o_dz2 = take(4 * B * h);
   o_loss = take(8);
-  o_part = take(fits_fused() ? 4 * (P + 1) * kGradSplits : 0);
-  ws_bytes = off;
+  o_part = take(fused() ? 4 * (P + 1) * kGradSplits : 0);
+  ws_bytes = off + kWorkspaceAlign;
 }
 
 // Parameter offsets (floats) inside the flat vector: W1, b1, W2, b2, W3, b3.
@@ -646,7 +647,7 @@ tnq_status mlp_bind(Ctx* ctx, CostModel* m, void* ws, size_t bytes) {
   if (!ws || bytes < m->ws_bytes)
     return fail(TNQ_ERR_WORKSPACE, "cost-model workspace needs " + std::to_string(m->ws_bytes) + " bytes");
   MLP_CUDA(cudaSetDevice(ctx->device));
-  m->ws = ws;
+  m->ws = workspace_base(ws);
   return mlp_upload(ctx, m, m->host_params.data());
 }
 

@@ -21,9 +21,7 @@ struct CostModel {
   size_t o_params = 0, o_grads = 0, o_m = 0, o_v = 0, o_w1b = 0, o_w2b = 0, o_w3b = 0, o_x = 0, o_t = 0, o_z1 = 0,
          o_a1 = 0, o_z2 = 0, o_a2 = 0, o_y = 0, o_dy = 0, o_sq = 0, o_dz1 = 0, o_dz2 = 0, o_loss = 0, o_part = 0;
   // whether the fused row kernel holds the hidden weights (mlp.cu)
-  bool fits_fused() const { return h <= 256 && h % 8 == 0; }
-  // ... and may copy them 16 bytes at a time
-  bool fused() const { return fits_fused() && (reinterpret_cast<uintptr_t>(ws) & 15) == 0; }
+  bool fused() const { return h <= 256 && h % 8 == 0; }
   size_t n_params() const;
   void layout();
 };

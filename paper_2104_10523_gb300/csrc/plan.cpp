@@ -21,6 +21,7 @@
 
 #include "internal.h"
 #include "splitk.h"
+#include "rules.h"
 #include "gemm_tc.cuh"
 #include "kernels.cuh"
 #include "mlp.h"
@@ -397,7 +398,7 @@ void layout_steps(Plan* p) {
   p->ws_qtab = align_up(p->ws_p2sum + 8 * per, 256);
   p->ws_picks = align_up(p->ws_qtab + 4 * (p->net.proj_src.size() + n_open), 256);
   off = align_up(p->ws_picks + p->picks.size(), 256);
-  p->ws_total = off;
+  p->ws_total = off + kWorkspaceAlign;
 }
 
 // Device program of the trajectory leaves: per leaf its factors in circuit

@@ -27,4 +27,12 @@ bool aligned(size_t n, const P*... p) {
   return (... && (reinterpret_cast<uintptr_t>(p) % n == 0));
 }
 
+// A caller's workspace is used from its first multiple of kWorkspaceAlign on (bulk
+// copies and 16-byte loads address it); the sizes the library asks for hold the
+// bytes in front of it.
+constexpr size_t kWorkspaceAlign = 256;
+inline char* workspace_base(void* ws) {
+  return reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(ws) + kWorkspaceAlign - 1) / kWorkspaceAlign * kWorkspaceAlign);
+}
+
 }  // namespace tnq

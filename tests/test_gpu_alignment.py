@@ -2,7 +2,8 @@
 operand permutes and the output permute that keep the lowest bit in place, and a
 plain-TF32 operand handed to the general GEMM in its stored order, against the
 FP64 oracle; device outputs of trajectory amplitudes and noisy probabilities at
-an odd double, bitwise equal to aligned ones; 4-byte alignment is refused.
+an odd double, bitwise equal to aligned ones; 4-byte alignment is refused;
+workspaces may start at any address.
 """
 import numpy as np
 import pytest
@@ -86,3 +87,58 @@ def test_four_byte_alignment_is_refused():
         with pytest.raises(T.TnqError) as e:
             T.tnq_contract_pair(ctx.h, x[s[0]:], [0, 1], x[s[1]:], [1, 2], x[s[2]:], [0, 2], ws, nb)
         assert e.value.status == T.TNQ_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("prec", ["fp32", "tf32x3"])
+@pytest.mark.parametrize("at", [1, 8, 255])
+def test_workspace_at_any_address(prec, at):
+    """Bitwise what an aligned workspace gives, and nothing written outside it."""
+    import torch
+    from paper_2104_10523_gb300 import build, tnq as T
+    from workloads import grid_circuit
+    build.build()
+    ctx = T.Context(0, prec)
+    guard = 512
+
+    def workspace(nb, shift):
+        w = torch.full((nb + shift + guard,), 0xa5, dtype=torch.uint8, device="cuda")
+        return w, w[shift:shift + nb]
+
+    def untouched(w, nb, shift):
+        return bool((w[:shift] == 0xa5).all()) and bool((w[shift + nb:] == 0xa5).all())
+
+    bits = random_bitstrings(12, 9, 3)
+    plan = T.Plan(T.Circuit(grid_circuit(3, 4, 8, 1234)), batch_log2=2, n_candidates=4, seed=1)
+    nb = int(plan.info["workspace_bytes"])
+    got = []
+    for shift in (0, at):
+        w, ws = workspace(nb, shift)
+        T.tnq_plan_bind(ctx.h, plan.h, ws, nb)
+        got.append(ctx.amplitudes(plan, bits))
+        assert untouched(w, nb, shift)
+    assert np.array_equal(got[0], got[1])
+    rng = np.random.default_rng(7)
+    for m, n, k in ((8, 8, 8), (6, 14, 6), (5, 9, 8)):
+        al, bl = ([int(v) for v in rng.permutation(x)] for x in (
+            list(range(m)) + list(range(200, 200 + k)), list(range(100, 100 + n)) + list(range(200, 200 + k))))
+        ol = [int(v) for v in rng.permutation(list(range(m)) + list(range(100, 100 + n)))]
+        A, B = (torch.randn(2 ** len(x), dtype=torch.complex64, device="cuda") for x in (al, bl))
+        nb = T.tnq_contract_workspace_bytes(T.PRECISIONS[prec], len(al), len(bl), len(ol))
+        out = []
+        for shift in (0, at):
+            w, ws = workspace(nb, shift)
+            C = torch.full((2 ** len(ol),), float("nan"), dtype=torch.complex64, device="cuda")
+            T.tnq_contract_pair(ctx.h, A, al, B, bl, C, ol, ws, nb)
+            assert untouched(w, nb, shift)
+            out.append(C)
+        assert torch.equal(out[0], out[1])
+    grads = []
+    X, t = rng.uniform(size=(40, 16)).astype(np.float32), rng.standard_normal(40).astype(np.float32)
+    for shift in (0, at):
+        m = T.CostModel(ctx, hidden=64, max_batch=64, seed=3)
+        nb = m.ws.numel()
+        w, ws = workspace(nb, shift)
+        T.check(T.load().tnq_cost_model_bind(ctx.h, m.h, T.C.c_void_p(ws.data_ptr()), nb))
+        grads.append(m.gradients(X, t)[0])
+        assert untouched(w, nb, shift)
+    assert np.array_equal(grads[0], grads[1])

@@ -54,3 +54,12 @@ def test_sixteen_byte_accesses_to_caller_tensors_ask_first():
     assert "!perm_b && aligned(16, b_src)" in src("executor.cu")
     for name in ("skinny.cu", "gemm_tc_rows.cu"):
         assert "(reinterpret_cast<uintptr_t>(Gsrc) & 15) == 0" in src(name)
+
+
+def test_workspace_base(tmp_path):
+    """The first multiple of 256, within the bytes the sizes asked for add."""
+    at = [0x1000, 0x1001, 0x1008, 0x10ff, 0x1100]
+    body = "\n".join(f'printf("%zu\\n", (size_t)workspace_base((void*){p}));' for p in at)
+    assert run(tmp_path, body) == [str((p + 255) // 256 * 256) for p in at]
+    body = 'printf("%zu\\n", kWorkspaceAlign);'
+    assert run(tmp_path, body) == ["256"]
