@@ -338,11 +338,12 @@ tnq_status tnq_contract_pair_noalloc(tnq_ctx* ctx, const void* A, int ra, const 
 tnq_status tnq_plan_autotune(tnq_ctx* ctx, tnq_plan* p, int reps, int* n_tensor_core, int* n_cuda_core);
 
 /* Replay batches from a CUDA graph (1, the default) or launch every kernel
- * directly (0).  With graphs on, the first batch of a plan at a given precision
- * captures every slice and step of one batch into a graph (on a private stream);
- * it and later batches, ragged ones included, replay the graph on the context's
- * stream.  The results are identical either way.  Timed runs
- * (tnq_ctx_set_timing) and partial slice ranges always launch directly. */
+ * directly (0).  With graphs on, the first full batch of a plan at a given
+ * precision, or the second ragged one, captures every slice and step of one batch
+ * into a graph (on a private stream); it and later batches, ragged ones included,
+ * replay the graph on the context's stream.  The results are identical either
+ * way.  A plan's first ragged batch without a graph, timed runs
+ * (tnq_ctx_set_timing) and partial slice ranges launch directly. */
 tnq_status tnq_ctx_set_graphs(tnq_ctx* ctx, int enable);
 
 /* Which kernels run the steps of a plan.  TNQ_KERNELS_DEFAULT: the plan's

@@ -229,6 +229,7 @@ struct Plan {
   void* graph_exec = nullptr;     // cudaGraphExec_t
   int graph_precision = -1;
   int graph_policy = -1;          // kernel policy the graph was captured with
+  int ragged_precision = -1, ragged_policy = -1;  // mode of the last ragged batch launched without a graph
   double graph_capture_ms = 0;
   int64_t graph_nodes = 0;
   // device binding; error flags of the plan's kernels (a slot of mapped host memory,
