@@ -33,6 +33,7 @@
 #include <mutex>
 
 #include "gemm_tc.cuh"
+#include "kernels.cuh"
 #include "tc_ptx.cuh"
 #include "../../include/tnq.h"
 
@@ -397,18 +398,15 @@ bool make_map(CUtensorMap* m, const void* base, bool bf16, uint64_t inner, uint6
 }  // namespace
 
 cudaError_t tc_gemm_prepare() {
-  // one-time set-up outside any stream capture: the driver entry point and the
-  // largest dynamic shared memory any configuration of the kernel uses
-  static cudaError_t result = cudaErrorUnknown;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    result = encode_fn() ? cudaSuccess : cudaErrorNotSupported;
-    if (result == cudaSuccess)
-      result = cudaFuncSetAttribute(cgemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    TC_SMEM_BUDGET + 8 * TC_STAGE_OUT + 1024);
-    if (result == cudaSuccess) result = tc_rows_prepare();
+  // set-up of a device, outside any stream capture: the driver entry point and the
+  // largest dynamic shared memory any configuration of the kernels uses
+  static std::atomic<uint64_t> done{0};
+  return once_per_device(&done, [] {
+    if (!encode_fn()) return cudaErrorNotSupported;
+    const cudaError_t e = cudaFuncSetAttribute(cgemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               TC_SMEM_BUDGET + 8 * TC_STAGE_OUT + 1024);
+    return e == cudaSuccess ? tc_rows_prepare() : e;
   });
-  return result;
 }
 
 bool tc_gemm_supported(int M, int N, int K, int precision) {

@@ -65,7 +65,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "gemm_tc.cuh"
 #include "kernels.cuh"
@@ -748,19 +747,16 @@ const TrKernel kTrKernels2[3] = {cgemm_tc_rows_kernel<8, 0, 2>, cgemm_tc_rows_ke
 
 
 cudaError_t tc_rows_prepare() {
-  static cudaError_t result = cudaErrorUnknown;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    result = cudaSuccess;
+  static std::atomic<uint64_t> done{0};
+  return once_per_device(&done, [] {
+    cudaError_t e = cudaSuccess;
     for (const auto& row : kTrKernels)
       for (TrKernel k : row)
-        if (result == cudaSuccess)
-          result = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TR_SMEM_MAX));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TR_SMEM_MAX));
     for (TrKernel k : kTrKernels2)
-      if (result == cudaSuccess)
-        result = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TR_SMEM_HALF));
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TR_SMEM_HALF));
+    return e;
   });
-  return result;
 }
 
 bool tc_rows_supported(int ns, int ng, int K, int batch, int nrow, int precision) {

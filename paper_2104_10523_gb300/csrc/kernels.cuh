@@ -9,17 +9,26 @@
 
 namespace tnq {
 
-// Lets kernel f use `bytes` of dynamic shared memory on the current device;
-// `done` (one per kernel) remembers the devices it was set on.
-inline cudaError_t allow_smem(const void* f, int bytes, std::atomic<uint64_t>* done) {
+// Calls set() once on every device that is current when this runs; `done` (one per
+// use) remembers the devices where it succeeded.
+template <typename Set>
+cudaError_t once_per_device(std::atomic<uint64_t>* done, Set set) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const uint64_t bit = dev < 64 ? 1ull << dev : 0;
   if (done->load(std::memory_order_acquire) & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  e = set();
   if (e == cudaSuccess) done->fetch_or(bit, std::memory_order_release);
   return e;
+}
+
+// Lets kernel f use `bytes` of dynamic shared memory, always the same number (a
+// limit set for one launch could be lowered by another thread before it), on the
+// current device.
+inline cudaError_t allow_smem(const void* f, int bytes, std::atomic<uint64_t>* done) {
+  return once_per_device(done,
+                         [&] { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
 }
 
 // Operand formats written by the permute kernel.

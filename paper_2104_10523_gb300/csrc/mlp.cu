@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "executor.h"
+#include "kernels.cuh"
 #include "mlp.h"
 #include "rules.h"
 
@@ -542,7 +543,8 @@ static tnq_status rows_pass(Ctx* ctx, CostModel* m, int B, bool back) {
   const size_t smem = mr_smem(m->d_in, m->h);
   const unsigned grid = unsigned((B + MR_ROWS - 1) / MR_ROWS);
   auto k = back ? mlp_rows_kernel<true> : mlp_rows_kernel<false>;
-  MLP_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+  static std::atomic<uint64_t> done[2];
+  MLP_CUDA(allow_smem(reinterpret_cast<const void*>(k), int(mr_smem(m->d_in, 256)), &done[back]));
   k<<<grid, MR_THREADS, smem, ctx->stream>>>(a);
   MLP_CUDA(cudaGetLastError());
   ctx->launches++;

@@ -63,3 +63,19 @@ def test_workspace_base(tmp_path):
     assert run(tmp_path, body) == [str((p + 255) // 256 * 256) for p in at]
     body = 'printf("%zu\\n", kWorkspaceAlign);'
     assert run(tmp_path, body) == ["256"]
+
+
+def test_shared_memory_limits_are_fixed_and_per_device():
+    """Dynamic shared-memory limits go through once_per_device (a process-wide flag
+    would leave a second device at the default limit) with a size that does not
+    depend on the call (two threads could lower each other's limit)."""
+    import glob
+    import re
+    for f in glob.glob(os.path.join(CSRC, "*.cu*")):
+        src = open(f).read()
+        for m in re.finditer(r"cudaFuncAttributeMaxDynamicSharedMemorySize", src):
+            at = src.rfind("once_per_device(", 0, m.start())
+            end = src.find("\n}", at)
+            assert at >= 0 and m.start() < end, (f, src.count("\n", 0, m.start()) + 1)
+    prep = open(os.path.join(CSRC, "gemm_tc.cu")).read()
+    assert prep.count("call_once") == 1  # the driver entry point: one per process
