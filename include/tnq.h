@@ -328,8 +328,9 @@ tnq_status tnq_contract_pair_noalloc(tnq_ctx* ctx, const void* A, int ra, const 
 
 /* Autotune a bound plan for the context's precision: every step that could run
  * on the tensor cores is timed (CUDA events, best of `reps` after a warm-up run,
- * on the plan's workspace) both there and on the CUDA cores (row-streaming,
- * dot or tiled FP32 kernel); a tall-skinny step (one operand of at most 128
+ * on the plan's workspace) both there and on the CUDA cores (one-launch, gather,
+ * long-K or tiled FP32 kernel; small steps that run several to a launch are not
+ * timed and count as placed on the CUDA cores); a tall-skinny step (one operand of at most 128
  * rows, K <= 256) is also timed with the large operand gathered, split and
  * multiplied in one tensor-core kernel.  The fastest choice is kept in the plan for
  * that precision; later calls at that precision follow it (and re-capture

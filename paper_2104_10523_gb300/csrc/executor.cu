@@ -924,13 +924,12 @@ tnq_status exec_autotune(Ctx* ctx, Plan* p, int reps, int* n_tc, int* n_cuda) {
   ctx->timing = false;
   int ntc = 0, ncc = 0;
   tnq_status result = TNQ_OK;
-  // small steps that run in a step program have one choice
+  // small steps that run in a step program are not timed: they stay on the CUDA cores
   std::vector<char> grouped(n, 0);
   if (programs_allowed(ctx))
     for (const StepGroup& g : p->groups)
       for (int si : g.steps) grouped[si] = 1;
   for (size_t si = 0; si < n && result == TNQ_OK; ++si) {
-    if (grouped[si]) continue;
     const Step& s = p->steps[si];
     const bool tc_ok = ctx->precision != TNQ_PREC_FP32 &&
                        tc_gemm_supported(1 << s.nM, 1 << s.nN, 1 << s.nK, ctx->precision) &&
@@ -946,6 +945,10 @@ tnq_status exec_autotune(Ctx* ctx, Plan* p, int reps, int* n_tc, int* n_cuda) {
     if (tc_ok) cands[nc++] = 1;
     if (rows_ok) cands[nc++] = 2;
     if (nc == 1) continue;  // one candidate only
+    if (grouped[si]) {
+      ++ncc;
+      continue;
+    }
     float best = 0;
     int pick = -1;
     for (int ci = 0; ci < nc && result == TNQ_OK; ++ci) {
