@@ -391,7 +391,8 @@ tnq_status tnq_cost_model_train(tnq_ctx* ctx, tnq_cost_model* m, const float* X,
                                 int epochs, int batch, float lr, float* final_loss);
 /* Predictions y [n] for host rows X [n][d_in]. */
 tnq_status tnq_cost_model_predict(tnq_ctx* ctx, tnq_cost_model* m, const float* X, int64_t n, float* y);
-/* Features of every step of a plan for the kernels `precision` runs them on:
+/* Features of every step of a plan: sizes, permuted operands and the shape class
+ * of the step at `precision` (a fixed rule, independent of which kernel runs it),
  * out [n_steps][tnq_step_feature_count()]. */
 tnq_status tnq_plan_step_features(const tnq_plan* p, int precision, float* out);
 /* As tnq_plan_create (BEST candidate set), but the candidate with the least
@@ -412,10 +413,12 @@ tnq_status tnq_ctx_launch_count(const tnq_ctx* ctx, uint64_t* count);
  * launches is bracketed by CUDA events on its stream, and one record per
  * launch is kept (enabling clears earlier records).  These per-step timings
  * (shape, algorithmic flops and bytes, duration) are also the training data
- * of the learned path cost model. */
+ * of the learned path cost model.  Steps that otherwise run several to a launch
+ * are launched one by one while timing is on (with the same results). */
 tnq_status tnq_ctx_set_timing(tnq_ctx* ctx, int enable);
 /* Copy up to max_records records, 10 doubles each:
- * {kind (0 permute, 1 CUDA-core GEMM, 2 tensor-core GEMM, 3 other), plan step,
+ * {kind (0 permute, 1 CUDA-core GEMM, 2 tensor-core GEMM, 3 other, 4 skinny
+ *  CUDA-core GEMM, 5 tall-skinny tensor-core GEMM), plan step,
  *  log2 H, log2 M, log2 N, log2 K, algorithmic flops, algorithmic bytes,
  *  milliseconds, 0}.  *n_out receives the number available. */
 tnq_status tnq_ctx_get_timings(const tnq_ctx* ctx, double* rec, int max_records, int* n_out);

@@ -766,8 +766,8 @@ bool tc_rows_supported(int ns, int ng, int K, int batch, int nrow, int precision
   // stream S' through the stages)
   if (ns < 1 || ns > 128 || K < 1 || K > TR_KMAX || ng < 128 || (ng & 127) || batch < 1 || nrow < 7) return false;
   if (K > TR_RESIDENT_KMAX) return K >= 128 && tr_stages_streamed(tr_atoms(K, bf16), tr_npad(ns)).stages >= 2;
-  // S' of one batch entry must fit beside at least two stages (larger batches
-  // run one launch per entry)
+  // S' of one batch entry must fit beside at least two stages (where those of all
+  // entries do not, each CTA serves one entry)
   const size_t bp = tr_bprime_bytes(ns, K, 1, bf16);
   return bp <= size_t(TR_BPRIME_BUDGET) && tr_stages(tr_atoms(K, bf16), bp).stages >= 2;
 }

@@ -148,7 +148,6 @@ struct Step {
 struct StepGroup {
   std::vector<int> steps;        // by level
   std::vector<int> level_begin;  // n_levels + 1 entries into steps
-  int cls = 2;
   size_t rec_begin = 0;          // first record of the group in the program region
   int max_units = 0;             // warp-sized units of its largest level (set when the records are made)
 };

@@ -131,7 +131,9 @@ void layout_steps(Plan* p) {
     // K and H orders follow the larger operand, except in dot-shaped steps
     // (at most 8 x 8 outputs per batch entry, at least 2^10 K values): there they
     // follow the operand whose stored layout starts with the longer run of K
-    // labels, which the dot kernel then reads in place
+    // labels.  No kernel needs that (the long-K kernel picks its own tiles); it is
+    // the order in which one-launch steps add their K values, and it decides which
+    // operand counts as permuted in the features the cost model was trained on.
     int nk_all = 0, nm = 0, nn = 0;
     for (int l : lb)
       if (contains(la, l) && !contains(out_set, l)) ++nk_all;
@@ -224,7 +226,7 @@ void layout_steps(Plan* p) {
     return !s.fold && s.nH + s.nM + s.nN <= kProgMaxOut && s.nK <= kProgMaxK &&
            s.nH + s.nM + s.nN + s.nK <= kProgMaxWork;
   };
-  auto add_group = [&](const std::vector<int>& members, int c) {
+  auto add_group = [&](const std::vector<int>& members) {
     // levels by dependence within the group; groups are cut at the launch's limit
     for (size_t at = 0; at < members.size();) {
       const size_t end = std::min(members.size(), at + kProgMaxOps);
@@ -245,7 +247,6 @@ void layout_steps(Plan* p) {
         p->exec.push_back(members[at]);
       } else {
         StepGroup g;
-        g.cls = c;
         for (auto& v : by) {
           g.level_begin.push_back((int)g.steps.size());
           g.steps.insert(g.steps.end(), v.begin(), v.end());
@@ -272,18 +273,18 @@ void layout_steps(Plan* p) {
         rest.push_back(i);
       }
     }
-    add_group(early, c);
+    add_group(early);
     std::vector<int> run;
     for (int i : rest) {
       if (prog_step(p->steps[i])) {
         run.push_back(i);
         continue;
       }
-      add_group(run, c);
+      add_group(run);
       run.clear();
       p->exec.push_back(i);
     }
-    add_group(run, c);
+    add_group(run);
   }
 
   // ---- workspace: [leaves][arena of intermediates][scratch A][scratch B][acc][misc]
@@ -477,9 +478,12 @@ static void build_traj_program(const Circuit& c, Plan* p) {
 
 // Per-step features for the cost model (16 floats per step): log2 sizes of the
 // batch, row, column and contracted dimensions and of the work, operand and
-// output elements (scaled by 1/32), whether each operand is permuted, which
-// kernel the executor dispatches the step to at this precision, log2 of the
-// algorithmic bytes, and whether it is the root step.
+// output elements (scaled by 1/32), whether each operand is permuted, the shape
+// class of the step at this precision (tensor-core GEMM, skinny, dot-shaped,
+// other), log2 of the algorithmic bytes, and whether it is the root step.  The
+// class is a fixed rule on shapes, the one stored models were trained with; which
+// kernel runs the step is run_gemm_step's choice (or the autotuner's), and steps
+// that run several to a launch are still described, and timed, one by one.
 void step_features(const Plan& p, int precision, std::vector<float>* out) {
   out->clear();
   for (size_t i = 0; i < p.steps.size(); ++i) {
