@@ -159,7 +159,7 @@ def _int_array(v):
 def _labels(v):
     """Labels as the bytes of a C int array (a ctypes array costs several times as
     much to build, on the order of the call itself for a small contraction)."""
-    if isinstance(v, (bytes, bytearray)):  # one label a byte; array() would take them as its raw contents
+    if v.__class__ is not list and isinstance(v, (bytes, bytearray)):  # one label a byte; array() would take them as its raw contents
         return bytes(_int_array(v))
     try:
         return array("i", v).tobytes()
