@@ -294,11 +294,15 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   // Small steps of the CUDA-core path, and of the tall-skinny kernel's where a
   // launch of it (about 10 us) is all latency, run in one launch.
   // `ordered` long-K steps run there too, one lane an output.
-  const bool long_ordered = ordered && !use_tc && !gather && use_kdot(nM, nN, nK) && !use_dot(nM, nN, nK) && part &&
-                            nM + nN + nH <= SMALL_MAX_OUT;
-  const bool small = long_ordered || (!use_tc && small_step(nH, nM, nN, nK) &&
+  const bool long_k = !use_tc && !gather && use_kdot(nM, nN, nK) && part;
+  const bool fits_small = small_step(nH, nM, nN, nK);
+  // Many rows: the rows kernel, after a permute where the order asks for one.
+  const bool rows = long_k && !fits_small && !use_dot(nM, nN, nK) && !ordered &&
+                    rows_faster(perm_b, nM, nN, nH, nK);
+  const bool long_ordered = ordered && long_k && !rows && !use_dot(nM, nN, nK) && nM + nN + nH <= SMALL_MAX_OUT;
+  const bool small = long_ordered || (!use_tc && fits_small &&
                                       (!tc_rows || (choice == -1 && !ordered && work <= kSmallTcRows)));
-  const bool kdot = !small && !gather && !use_tc && use_kdot(nM, nN, nK) && part;
+  const bool kdot = !small && !rows && long_k;
   signed char pos_c[32];  // positions in C of the output bits [N][M][H]
   for (int j = 0; j < nN + nM + nH && j < 32; ++j) pos_c[j] = (signed char)j;
   if ((small || kdot) && direct && direct->C) {
@@ -419,7 +423,7 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
     ctx->launches++;
     return TNQ_OK;
   }
-  if (prec == TNQ_PREC_FP32) {
+  if (prec == TNQ_PREC_FP32) {  // rows kernel, tiled GEMM: both operands with K lowest
     if (perm_a) {
       build_perm_desc(a_labels.data(), (int)a_labels.size(), a_req.data(), (int)a_req.size(), slice_labels.data(),
                       ns, PM_C64, nK, &d);
@@ -436,13 +440,16 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
     } else {
       op.b0 = b_src;
     }
-    KernelRecord r{1, ctx->cur_step, nH, nM, nN, nK, 8.0 * work,
+    KernelRecord r{rows ? 4 : 1, ctx->cur_step, nH, nM, nN, nK, 8.0 * work,
                    8.0 * (std::ldexp(1.0, nH + nM + nK) + std::ldexp(1.0, nH + nN + nK) +
                           (acc ? 2.0 : 1.0) * std::ldexp(1.0, nH + nM + nN)),
                    0.f};
-    const int splits = part ? simt_splits(nH, nM, nN, nK) : 1;
+    const int splits = rows ? ordered_splits(nH, nM, nN, nK) : part ? simt_splits(nH, nM, nN, nK) : 1;
     int slot = timing_begin(ctx);
-    TNQ_CUDA(launch_cgemm_simt(op.a0, op.b0, C, acc, part, splits, 1 << nM, 1 << nN, 1 << nK, 1 << nH, ctx->stream));
+    if (rows)
+      TNQ_CUDA(launch_cgemm_rows(op.a0, op.b0, C, acc, part, splits, 1 << nM, 1 << nN, 1 << nK, 1 << nH, ctx->stream));
+    else
+      TNQ_CUDA(launch_cgemm_simt(op.a0, op.b0, C, acc, part, splits, 1 << nM, 1 << nN, 1 << nK, 1 << nH, ctx->stream));
     if (splits > 1) {
       TNQ_CUDA(launch_reduce_splits(part, splits, out_elems, C, acc, ctx->sm_count, ctx->stream, ordered));
       ctx->launches++;

@@ -127,6 +127,11 @@ cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const SmallDesc& sd, co
                                      int ns, int ng, int K, int batch, int slice_id, bool round_tf32, int sm_count,
                                      cudaStream_t st);
 
+// rows kernel (see skinny.cu): S [batch][ns][K], G [batch][ng][K], output [batch][ns][ng],
+// ns <= 32; splits > 1 leaves FP32 sums of equal K ranges in part.
+cudaError_t launch_cgemm_rows(const void* S, const void* G, void* C, void* acc, void* part, int splits, int ns, int ng,
+                              int K, int batch, cudaStream_t st);
+
 // One small contraction reading both operands in place (see small.cu): bit j of
 // an output index (2^n_out of them) sits at stored position pa[j] of A, pb[j]
 // of B (-1: not an index of that operand) and pc[j] of C; bit j of the

@@ -1,4 +1,4 @@
-// Bandwidth-oriented complex GEMM for skinny contraction steps of short K.
+// Bandwidth-oriented complex GEMMs for skinny contraction steps.
 //
 // Many steps of a contraction path have a tiny side: few output rows (a small
 // operand meeting a large one).  Their cost is reading the large operand once
@@ -6,7 +6,9 @@
 //
 //   C[h][s][g] = sum_k S[h][s][k] G[h][g][k] for a small side of at most 128
 //   rows and K of at most 32: each thread loads its rows of the large operand,
-//   in their stored bit layout, into registers.
+//   in their stored bit layout, into registers (gather kernel).  Many rows of a
+//   longer K, up to 32 of them on the small side: a thread per row of the large
+//   operand, both operands staged from [row][K] order (rows kernel).
 #include <algorithm>
 
 #include "kernels.cuh"
@@ -182,7 +184,100 @@ __global__ void __launch_bounds__(T, gather_min_ctas(K, ROWS))
   }
 }
 
+// ------------------------------------------------------------------ rows kernel
+// C[h][s][g] = sum_k S[h][s][k] G[h][g][k] for K of 64 and more, at most 32 rows of
+// S: a CTA owns 128 rows of G, one a thread, and walks K (or its share of it) 32
+// values at a time, which it stages in shared memory by coalesced loads.  Every
+// output is one sum in ascending K.
+//
+// Bound: HBM while few rows of S meet G, the FFMA pipe at 32.  8 x 2^20 x 64 takes 467
+// us a call with G in this order and 655 after a permute of G (long-K kernel: 1394
+// and 1434); 32 x 2^20 x 64 522 (1336).  It needs G with K
+// lowest, a permute where G is stored otherwise; beside the long-K kernel, which
+// reads any order but spends a CTA's table set-up on 16 or 32 rows, it wins where
+// rows are many and K is short, see rows_faster().
+constexpr int RW_THREADS = 128;  // rows of G per CTA
+constexpr int RW_KC = 32;        // K values staged per iteration
+constexpr int RW_SMAX = 32;
+
+__global__ void __launch_bounds__(RW_THREADS) cgemm_rows_kernel(const float2* __restrict__ S,
+                                                                const float2* __restrict__ G, float2* __restrict__ C,
+                                                                double2* __restrict__ acc, float2* __restrict__ part,
+                                                                int ns, int ng, int K, int batch, int kchunk,
+                                                                int tiles_g) {
+  __shared__ float2 Gs[RW_THREADS][RW_KC + 1];
+  __shared__ float2 Ss[RW_SMAX][RW_KC + 1];
+  const int t = threadIdx.x;
+  const int g0 = int(blockIdx.x % tiles_g) * RW_THREADS, h = int(blockIdx.x / tiles_g);
+  const int kbeg = int(blockIdx.y) * kchunk, kend = min(K, kbeg + kchunk);
+  const float2* Sh = S + size_t(h) * ns * K;
+  const float2* Gh = G + size_t(h) * ng * K;
+  float ar[RW_SMAX], ai[RW_SMAX];
+#pragma unroll
+  for (int s = 0; s < RW_SMAX; ++s) ar[s] = ai[s] = 0.f;
+  for (int k0 = kbeg; k0 < kend; k0 += RW_KC) {
+    const int kc = min(RW_KC, kend - k0);
+    for (int idx = t; idx < RW_THREADS * RW_KC; idx += RW_THREADS) {
+      const int r = idx / RW_KC, kk = idx % RW_KC;
+      Gs[r][kk] = g0 + r < ng && kk < kc ? Gh[size_t(g0 + r) * K + k0 + kk] : make_float2(0.f, 0.f);
+    }
+    for (int idx = t; idx < RW_SMAX * RW_KC; idx += RW_THREADS) {
+      const int r = idx / RW_KC, kk = idx % RW_KC;
+      Ss[r][kk] = r < ns && kk < kc ? Sh[size_t(r) * K + k0 + kk] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    for (int kk = 0; kk < kc; ++kk) {
+      const float2 g = Gs[t][kk];
+#pragma unroll
+      for (int s = 0; s < RW_SMAX; ++s) {
+        if (s < ns) {
+          const float2 a = Ss[s][kk];
+          ar[s] = fmaf(a.x, g.x, ar[s]);
+          ar[s] = fmaf(-a.y, g.y, ar[s]);
+          ai[s] = fmaf(a.x, g.y, ai[s]);
+          ai[s] = fmaf(a.y, g.x, ai[s]);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (g0 + t >= ng) return;
+  const size_t base = size_t(h) * ns * ng + size_t(g0 + t);
+#pragma unroll
+  for (int s = 0; s < RW_SMAX; ++s) {
+    if (s < ns) {
+      const size_t o = base + size_t(s) * ng;
+      if (part) {
+        part[size_t(blockIdx.y) * batch * ns * ng + o] = make_float2(ar[s], ai[s]);
+      } else if (acc) {
+        double2 v = acc[o];
+        v.x += ar[s];
+        v.y += ai[s];
+        acc[o] = v;
+      } else {
+        C[o] = make_float2(ar[s], ai[s]);
+      }
+    }
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_cgemm_rows(const void* S, const void* G, void* C, void* acc, void* part, int splits, int ns, int ng,
+                              int K, int batch, cudaStream_t st) {
+  if (ns < 1 || ns > RW_SMAX || splits < 1 || splits > 65535 || (splits > 1 && !part))
+    return cudaErrorInvalidConfiguration;
+  const long long tiles_g = (ng + RW_THREADS - 1) / RW_THREADS;
+  if (tiles_g * batch > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  const int kchunk = ((K + splits - 1) / splits + RW_KC - 1) / RW_KC * RW_KC;
+  if ((long long)kchunk * (splits - 1) >= K) return cudaErrorInvalidConfiguration;  // an empty split
+  const dim3 grid{unsigned(tiles_g * batch), unsigned(splits), 1u};
+  cgemm_rows_kernel<<<grid, RW_THREADS, 0, st>>>(
+      reinterpret_cast<const float2*>(S), reinterpret_cast<const float2*>(G), reinterpret_cast<float2*>(C),
+      reinterpret_cast<double2*>(acc), splits > 1 ? reinterpret_cast<float2*>(part) : nullptr, ns, ng, K, batch, kchunk,
+      int(tiles_g));
+  return cudaGetLastError();
+}
 
 cudaError_t launch_cgemm_rows_gather(const void* Ssmall, const SmallDesc& sd, const void* Gsrc, const GatherDesc& gd,
                                      void* C, void* acc,

@@ -81,6 +81,32 @@ inline int kdot_splits(int nH, int nM, int nN, int nK) {
   return int(std::max(1.0, std::min({std::floor(kSplitTargetCtas / units), tiles, cap})));
 }
 
+// Whether the rows kernel takes a long-K step from the long-K kernel, whose CTAs pay
+// for their tables on 16 or 32 rows of the large operand: where rows (batch entries
+// included) are many, K is short and a batch entry fills the rows kernel's tile of
+// 128 rows (half of it at K = 64).  The table holds log2 of the rows from which, by
+// log2 of the small side's rows and of K (from 6 on; 99: never); `permuted`: G is not
+// stored with K lowest, so the rows kernel needs a permute first.  Time of the long-K
+// kernel over the rows kernel's, call against call: K = 64, 8 x 2^20 3.0 in place
+// and 2.2 permuted, 2^16 1.6 and 1.1, 2^14 0.9 and 0.6; K = 128, 8 x 2^20 1.7 and 1.2;
+// K = 256, 8 x 2^19 1.1 and 0.8; K = 512, 32 x 2^18 1.1 and 0.8; below 0.8 beyond.
+inline bool rows_faster(bool permuted, int nM, int nN, int nH, int nK) {
+  static constexpr signed char from[2][6][5] = {{{16, 21, 99, 99, 99},
+                                                 {15, 16, 99, 99, 99},
+                                                 {15, 16, 19, 99, 99},
+                                                 {15, 16, 19, 99, 99},
+                                                 {15, 16, 99, 99, 99},
+                                                 {15, 16, 17, 18, 19}},
+                                                {{18, 99, 99, 99, 99},
+                                                 {17, 18, 99, 99, 99},
+                                                 {16, 17, 99, 99, 99},
+                                                 {16, 17, 99, 99, 99},
+                                                 {17, 18, 99, 99, 99},
+                                                 {16, 17, 99, 99, 99}}};
+  if (nM > 5 || nK < 6 || nK > 10 || nN < (nK == 6 ? 6 : 7)) return false;
+  return nN + nH - (nN == 6) >= from[permuted][nM][nK - 6];
+}
+
 // K splits of a long-K step whose sums keep a fixed order (one lane per output,
 // ascending K): at least 256 K values a split.
 inline int ordered_splits(int nH, int nM, int nN, int nK) {

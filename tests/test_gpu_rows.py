@@ -1,0 +1,46 @@
+"""GPU parity of the rows kernel (long-K steps with many rows): at the line from the
+long-K kernel and on both sides of it, one row of the small side and 32, rows in
+one batch entry and in many, half-filled tiles, K of one stage pair and more,
+operands in the order it asks for and permuted.  64 sampled rows of the large
+operand are compared with FP64 sums; FP32 sums of K <= 2^10 terms stay below 1e-5
+in relative L2.
+"""
+import numpy as np
+import pytest
+
+from oracle import contraction
+from test_gpu_batched import TOL, rel
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("order", ["stored", "scattered"])
+@pytest.mark.parametrize("m,n,k,h", [  # (log2 M, N, K, H)
+    (3, 14, 6, 0), (3, 15, 6, 0), (2, 16, 6, 0), (0, 18, 6, 0), (1, 7, 6, 10), (4, 6, 6, 12), (5, 17, 6, 0), (3, 17, 7, 0),
+    (5, 8, 7, 9), (5, 17, 8, 0), (2, 19, 8, 0)])
+def test_rows(order, m, n, k, h):
+    import torch
+    from paper_2104_10523_gb300 import build, tnq as T
+    build.build()
+    rng = np.random.default_rng(m + n + k + h)
+    ml, nl, kl, hl = (list(range(100 * i, 100 * i + d)) for i, d in enumerate((m, n, k, h)))
+    al, bl = kl + ml + hl, kl + nl + hl
+    if order == "scattered":
+        al, bl = ([int(v) for v in rng.permutation(x)] for x in (al, bl))
+    ol = [x for x in bl if x in nl] + [x for x in al if x in ml] + [x for x in bl if x in hl]
+    g = torch.Generator(device="cuda")
+    g.manual_seed(7)
+    A, B = (torch.randn(2 ** len(x), dtype=torch.complex64, device="cuda", generator=g) for x in (al, bl))
+    C = torch.full((2 ** len(ol),), float("nan"), dtype=torch.complex64, device="cuda")
+    ctx = T.Context(0, "fp32")
+    nb = T.tnq_contract_workspace_bytes(T.PRECISIONS["fp32"], len(al), len(bl), len(ol))
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    T.tnq_contract_pair(ctx.h, A, al, B, bl, C, ol, ws, nb)
+    assert bool(torch.isfinite(torch.view_as_real(C)).all())
+    row_labels = ol[:n] + ol[n + m:]  # one large-operand row of one batch entry
+    rows = rng.choice(2 ** (n + h), size=64, replace=False)
+    rows[:2] = 0, 2 ** (n + h) - 1
+    ref = contraction.sampled_rows(A.cpu().numpy(), al, B.cpu().numpy(), bl, ol, rows, row_labels)
+    at = np.array([[(int(r) & (2 ** n - 1)) | j << n | (int(r) >> n) << (n + m) for j in range(2 ** m)] for r in rows])
+    got = C[torch.from_numpy(at.reshape(-1)).cuda()].cpu().numpy().reshape(at.shape)
+    assert rel(got, ref) <= TOL["fp32"], rel(got, ref)

@@ -79,3 +79,15 @@ def test_shared_memory_limits_are_fixed_and_per_device():
             assert at >= 0 and m.start() < end, (f, src.count("\n", 0, m.start()) + 1)
     prep = open(os.path.join(CSRC, "gemm_tc.cu")).read()
     assert prep.count("call_once") == 1  # the driver entry point: one per process
+
+
+def test_long_k_steps_with_many_rows_take_the_rows_kernel(tmp_path):
+    """The lines of splitk.h at the sizes they were measured at: (permuted, log2 M, N,
+    H, K) of steps the long-K kernel ran up to 3 times slower than the rows kernel, and of
+    steps that stay where they are."""
+    faster = [(0, 3, 20, 0, 6, 1), (1, 3, 20, 0, 6, 1), (0, 3, 14, 0, 6, 0), (1, 3, 15, 0, 6, 0), (0, 1, 10, 9, 6, 1),
+              (0, 5, 17, 0, 8, 1), (1, 5, 19, 0, 8, 0), (0, 3, 5, 14, 6, 0), (0, 0, 20, 0, 7, 0), (0, 3, 20, 0, 11, 0),
+              (0, 6, 20, 0, 6, 0), (0, 3, 20, 0, 5, 0)]
+    src = "\n".join(f'printf("%d\\n", rows_faster({p}, {m}, {n}, {h}, {k}));' for p, m, n, h, k, _ in faster)
+    got = run(tmp_path, src, extra=("-include", os.path.join(CSRC, "splitk.h")))
+    assert got == [str(x[-1]) for x in faster]
