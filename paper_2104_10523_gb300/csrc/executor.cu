@@ -297,8 +297,8 @@ tnq_status run_gemm_step(Ctx* ctx, const void* a_src, const std::vector<int>& a_
   const bool long_k = !use_tc && !gather && use_kdot(nM, nN, nK) && part;
   const bool fits_small = small_step(nH, nM, nN, nK);
   // Many rows: the rows kernel, after a permute where the order asks for one.
-  const bool rows = long_k && !fits_small && !use_dot(nM, nN, nK) && !ordered &&
-                    rows_faster(perm_b, nM, nN, nH, nK);
+  const bool rows = long_k && !fits_small && !use_dot(nM, nN, nK) &&
+                    (ordered ? rows_ordered(perm_b, nM, nN, nH, nK) : rows_faster(perm_b, nM, nN, nH, nK));
   const bool long_ordered = ordered && long_k && !rows && !use_dot(nM, nN, nK) && nM + nN + nH <= SMALL_MAX_OUT;
   const bool small = long_ordered || (!use_tc && fits_small &&
                                       (!tc_rows || (choice == -1 && !ordered && work <= kSmallTcRows)));

@@ -107,6 +107,22 @@ inline bool rows_faster(bool permuted, int nM, int nN, int nH, int nK) {
   return nN + nH - (nN == 6) >= from[permuted][nM][nK - 6];
 }
 
+// Whether the rows kernel takes a long-K step whose sums keep a fixed order from the
+// one-launch kernel (one lane an output, both operands uncoalesced): the same sums in
+// the same order, so the choice never shows in the results.  One-lane time over
+// rows time by log2 of the large operand's elements t, 2^nN rows: 16 rows of S 1.6
+// at t = 21, 5.6 at 24, up to 17 at 26 (permuted first: 0.6, 1.4 to 4, 1.5 to 4.7);
+// 8 rows 1.1, 3 and 8 (0.5, 0.9 to 2.2, 1 to 2.5); 4 rows 0.6, 1.6 and 4.5 (0.5, 0.6
+// to 1.4, 0.7 to 1.4); 2 rows 0.6, 0.9 and 0.9, but 1.4 to 2.3 from K = 2^18 on; with
+// fewer rows in S or in a batch entry of G the one-launch kernel stays ahead.
+inline bool rows_ordered(bool permuted, int nM, int nN, int nH, int nK) {
+  const int t = nN + nH + nK;
+  if (nM >= 4) return nN >= 5 && t >= (permuted ? 23 : 21);
+  if (nM == 3) return nN >= 6 && t >= (permuted ? 24 : 22);
+  if (nM == 2) return !permuted && nN >= 7 && t >= 22;
+  return nM == 1 && !permuted && nN >= 7 && nK >= 18;
+}
+
 // K splits of a long-K step whose sums keep a fixed order (one lane per output,
 // ascending K): at least 256 K values a split.
 inline int ordered_splits(int nH, int nM, int nN, int nK) {

@@ -4,12 +4,17 @@ one batch entry and in many, half-filled tiles, K of one stage pair and more,
 operands in the order it asks for and permuted.  64 sampled rows of the large
 operand are compared with FP64 sums; FP32 sums of K <= 2^10 terms stay below 1e-5
 in relative L2.
+
+In plain TF32 and BF16x3 plans it takes steps whose sums keep a fixed order: the
+amplitudes of such a plan stay within the modes' bounds (5e-3, and 5e-5 for a deep
+network) of the FP32 plan's.
 """
 import numpy as np
 import pytest
 
 from oracle import contraction
 from test_gpu_batched import TOL, rel
+from workloads import grid_circuit, random_bitstrings
 
 pytestmark = pytest.mark.gpu
 
@@ -44,3 +49,20 @@ def test_rows(order, m, n, k, h):
     at = np.array([[(int(r) & (2 ** n - 1)) | j << n | (int(r) >> n) << (n + m) for j in range(2 ** m)] for r in rows])
     got = C[torch.from_numpy(at.reshape(-1)).cuda()].cpu().numpy().reshape(at.shape)
     assert rel(got, ref) <= TOL["fp32"], rel(got, ref)
+
+
+def test_ordered_sums():
+    from paper_2104_10523_gb300 import build, tnq as T
+    build.build()
+    plan = T.Plan(T.Circuit(grid_circuit(4, 6, 14, 8)), batch_log2=4, n_candidates=8, seed=1, max_intermediate_log2=26)
+    st = plan.steps()
+    H, M, N, K = st[:, 3], st[:, 4], st[:, 5], st[:, 6]
+    assert np.any((M == 4) & (N >= 7) & (K >= 9) & (H + N + K >= 23))  # a step it takes
+    bits = random_bitstrings(24, 16, 3)
+    amp = {}
+    for prec in ("fp32", "tf32", "bf16x3"):
+        ctx = T.Context(0, prec)
+        ctx.bind(plan)
+        amp[prec] = ctx.amplitudes(plan, bits)
+    assert rel(amp["tf32"], amp["fp32"]) <= 5e-3
+    assert rel(amp["bf16x3"], amp["fp32"]) <= 5e-5

@@ -83,11 +83,14 @@ def test_shared_memory_limits_are_fixed_and_per_device():
 
 def test_long_k_steps_with_many_rows_take_the_rows_kernel(tmp_path):
     """The lines of splitk.h at the sizes they were measured at: (permuted, log2 M, N,
-    H, K) of steps the long-K kernel ran up to 3 times slower than the rows kernel, and of
-    steps that stay where they are."""
+    H, K) of steps the long-K and the one-launch kernel ran up to 3 and 17 times
+    slower than the rows kernel, and of steps that stay where they are."""
     faster = [(0, 3, 20, 0, 6, 1), (1, 3, 20, 0, 6, 1), (0, 3, 14, 0, 6, 0), (1, 3, 15, 0, 6, 0), (0, 1, 10, 9, 6, 1),
               (0, 5, 17, 0, 8, 1), (1, 5, 19, 0, 8, 0), (0, 3, 5, 14, 6, 0), (0, 0, 20, 0, 7, 0), (0, 3, 20, 0, 11, 0),
               (0, 6, 20, 0, 6, 0), (0, 3, 20, 0, 5, 0)]
+    ordered = [(0, 4, 14, 0, 10, 1), (1, 4, 12, 0, 12, 1), (0, 3, 6, 0, 17, 1), (1, 3, 10, 0, 12, 0), (0, 1, 8, 0, 18, 1),
+               (1, 1, 8, 0, 18, 0), (0, 0, 14, 0, 12, 0), (0, 2, 4, 6, 14, 0)]
     src = "\n".join(f'printf("%d\\n", rows_faster({p}, {m}, {n}, {h}, {k}));' for p, m, n, h, k, _ in faster)
+    src += "\n" + "\n".join(f'printf("%d\\n", rows_ordered({p}, {m}, {n}, {h}, {k}));' for p, m, n, h, k, _ in ordered)
     got = run(tmp_path, src, extra=("-include", os.path.join(CSRC, "splitk.h")))
-    assert got == [str(x[-1]) for x in faster]
+    assert got == [str(x[-1]) for x in faster + ordered]
