@@ -103,6 +103,70 @@ __global__ void __launch_bounds__(SM_THREADS) cgemm_small_kernel(const __grid_co
   }
 }
 
+// The same sums, in the same order, where one lane an output (log_l = 0) leaves the
+// chip idle: a warp an output, whose lanes load 32 K values at once, then all add them
+// up in ascending K, each taken from its lane by shuffles.  One lane alone waits for a
+// few uncoalesced loads at a time.
+__global__ void __launch_bounds__(SM_THREADS) cgemm_small_ordered_kernel(const __grid_constant__ SmallOp op,
+                                                                         float2* __restrict__ part) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t o = (blockIdx.x * SM_THREADS + threadIdx.x) >> 5;
+  if (o >> op.n_out) return;  // whole warps
+  const uint32_t kchunk = (1u << op.nk) / gridDim.y, kbeg = blockIdx.y * kchunk;
+  uint32_t oa = 0, ob = 0, oc = 0;
+  for (int j = 0; j < op.n_out; ++j)
+    if ((o >> j) & 1) {
+      oa |= op.pa[j] < 0 ? 0u : 1u << op.pa[j];
+      ob |= op.pb[j] < 0 ? 0u : 1u << op.pb[j];
+      oc |= 1u << op.pc[j];
+    }
+  for (int j = 0; j < 5; ++j)
+    if ((lane >> j) & 1) {  // nk >= 5: the low K bits are the lane's
+      oa |= 1u << op.ka[j];
+      ob |= 1u << op.kb[j];
+    }
+  auto load = [&](uint32_t k, float2* a, float2* b) {
+    uint32_t qa = oa, qb = ob;
+    for (int j = 5; j < op.nk; ++j)
+      if ((k >> j) & 1) {
+        qa |= 1u << op.ka[j];
+        qb |= 1u << op.kb[j];
+      }
+    *a = __ldg(op.A + qa);
+    *b = __ldg(op.B + qb);
+  };
+  float re = 0.f, im = 0.f;
+  float2 a, b, an, bn;
+  load(kbeg, &a, &b);
+  for (uint32_t k0 = 0; k0 < kchunk; k0 += 32, a = an, b = bn) {
+    if (k0 + 32 < kchunk) load(kbeg + k0 + 32, &an, &bn);
+    if (op.round_tf32) {
+      a = tf32_rna2(a);
+      b = tf32_rna2(b);
+    }
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      const float ax = __shfl_sync(0xffffffffu, a.x, i), ay = __shfl_sync(0xffffffffu, a.y, i);
+      const float bx = __shfl_sync(0xffffffffu, b.x, i), by = __shfl_sync(0xffffffffu, b.y, i);
+      re = fmaf(ax, bx, re);
+      re = fmaf(-ay, by, re);
+      im = fmaf(ax, by, im);
+      im = fmaf(ay, bx, im);
+    }
+  }
+  if (lane) return;
+  if (part) {
+    part[(size_t(blockIdx.y) << op.n_out) + oc] = make_float2(re, im);
+  } else if (op.acc) {
+    double2 v = op.acc[oc];
+    v.x += re;
+    v.y += im;
+    op.acc[oc] = v;
+  } else {
+    op.C[oc] = make_float2(re, im);
+  }
+}
+
 // ------------------------------------------------------------------ step program
 // A run of small steps in one launch: one cluster (the grid) of CTAs walks the steps level
 // by level, a cluster barrier between levels (the barrier's release and acquire
@@ -307,14 +371,30 @@ int small_lanes_log2(int n_out, int nk) {
   return std::max(0, std::min({5, nk, 16 - n_out}));
 }
 
+// Whether a warp an output is faster than a lane an output: up to 2^12 sums (outputs
+// x splits) of at least 64 values.  Calls in us, lane and warp: 2^8 sums of 2^10 134
+// and 45, 2^12 of 2^8 54 and 35, 2^12 of 2^6 29 and 22; 2^13 level (34 and 34 at
+// 2^7), 2^14 of 2^8 52 and 83.
+static bool small_ordered_warps(int n_out, int nk, int splits) {
+  int ls = 0;
+  while ((1 << ls) < splits) ++ls;
+  return nk - ls >= 6 && n_out + ls <= 12;
+}
+
 cudaError_t launch_cgemm_small(const SmallOp& op, void* part, int splits, cudaStream_t st) {
   if (op.n_out < 0 || op.n_out > SMALL_MAX_OUT || op.nk < 0 || op.nk > 31 || op.log_l < 0 || op.log_l > 5 ||
       splits < 1 || splits > 65535 || (splits & (splits - 1)) || splits > (1 << std::min(op.nk, 16)) ||
       (splits > 1 && !part))
     return cudaErrorInvalidConfiguration;
+  float2* const parts = splits > 1 ? reinterpret_cast<float2*>(part) : nullptr;
+  if (op.log_l == 0 && small_ordered_warps(op.n_out, op.nk, splits)) {
+    const dim3 grid{unsigned(((32ll << op.n_out) + SM_THREADS - 1) / SM_THREADS), unsigned(splits), 1u};
+    cgemm_small_ordered_kernel<<<grid, SM_THREADS, 0, st>>>(op, parts);
+    return cudaGetLastError();
+  }
   const long long threads = 1ll << (op.n_out + op.log_l);
   const dim3 grid{unsigned((threads + SM_THREADS - 1) / SM_THREADS), unsigned(splits), 1u};
-  cgemm_small_kernel<<<grid, SM_THREADS, 0, st>>>(op, splits > 1 ? reinterpret_cast<float2*>(part) : nullptr);
+  cgemm_small_kernel<<<grid, SM_THREADS, 0, st>>>(op, parts);
   return cudaGetLastError();
 }
 

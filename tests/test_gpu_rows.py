@@ -5,9 +5,9 @@ operands in the order it asks for and permuted.  64 sampled rows of the large
 operand are compared with FP64 sums; FP32 sums of K <= 2^10 terms stay below 1e-5
 in relative L2.
 
-In plain TF32 and BF16x3 plans it takes steps whose sums keep a fixed order: the
-amplitudes of such a plan stay within the modes' bounds (5e-3, and 5e-5 for a deep
-network) of the FP32 plan's.
+In plain TF32 and BF16x3 plans it takes steps whose sums keep a fixed order, as the
+one-launch kernel does, a lane or a warp an output: the amplitudes of such a plan
+stay within the modes' bounds (5e-3, and 5e-5 for a deep network) of the FP32 plan's.
 """
 import numpy as np
 import pytest
@@ -51,14 +51,19 @@ def test_rows(order, m, n, k, h):
     assert rel(got, ref) <= TOL["fp32"], rel(got, ref)
 
 
-def test_ordered_sums():
+@pytest.mark.parametrize("rows,cols,cycles,w,max_log2,seed,shape", [
+    (4, 6, 14, 4, 26, 1, lambda H, M, N, K: (M == 4) & (N >= 7) & (K >= 9) & (H + N + K >= 23)),  # rows kernel
+    (4, 4, 12, 2, 18, 60, lambda H, M, N, K: (N <= 3) & (K >= 10) & (H + M + N + K <= 18)),       # a warp an output
+    (4, 5, 9, 0, 19, 16, lambda H, M, N, K: (N <= 3) & (K >= 10) & (H + M + N + K <= 18))])
+def test_ordered_sums(rows, cols, cycles, w, max_log2, seed, shape):
     from paper_2104_10523_gb300 import build, tnq as T
     build.build()
-    plan = T.Plan(T.Circuit(grid_circuit(4, 6, 14, 8)), batch_log2=4, n_candidates=8, seed=1, max_intermediate_log2=26)
+    n = rows * cols
+    plan = T.Plan(T.Circuit(grid_circuit(rows, cols, cycles, seed if seed > 1 else 8)), batch_log2=w, n_candidates=8,
+                  seed=seed, max_intermediate_log2=max_log2)
     st = plan.steps()
-    H, M, N, K = st[:, 3], st[:, 4], st[:, 5], st[:, 6]
-    assert np.any((M == 4) & (N >= 7) & (K >= 9) & (H + N + K >= 23))  # a step it takes
-    bits = random_bitstrings(24, 16, 3)
+    assert np.any(shape(st[:, 3], st[:, 4], st[:, 5], st[:, 6]))  # a step it is about
+    bits = random_bitstrings(n, max(8, 2 ** w), 3)
     amp = {}
     for prec in ("fp32", "tf32", "bf16x3"):
         ctx = T.Context(0, prec)
